@@ -244,11 +244,8 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.K64, nc * (size_t)h->ldc);
     L.take(d.K32, nc * (size_t)h->ldc);
     L.take(d.Pinv, (size_t)(h->n_sub + 1) * kNB * kNB);
-    {   // slices and exponents of one pivot block for the tensor-core trailing update (local or coarse)
-        const int nloc = std::max(1, h->n_sub_real), ncor = (int)nc;
-        L.take(d.oz_slices, std::max(oz_slice_elems(nloc, h->max_ns), oz_slice_elems(1, ncor)));
-        L.take(d.oz_exps, 2 * std::max((size_t)nloc * h->max_ns, (size_t)ncor));
-    }
+    // slices and exponents of one pivot block of the tensor-core elimination (local or coarse)
+    L.take(d.oz, std::max(oz_bytes(std::max(1, h->n_sub_real), h->max_ns), oz_bytes(1, (int)nc)));
     L.take(d.dinv, nm);
     for (int k = 0; k < 3; ++k) L.take(d.e[k], nd);
     for (int k = 0; k < 3; ++k) L.take(d.mu[k], nd);
@@ -1065,6 +1062,24 @@ int dd_bind_workspace(dd_handle* h, void* dev, size_t bytes, void* stream) {
     return DD_OK;
 }
 
+namespace {
+
+// The exchange sweep of the r block of every stored local matrix, or of all of K~cc.
+int eliminate(dd_handle* h, bool coarse, cudaStream_t s) {
+    const int n = coarse ? (int)h->corner_dof.size() : h->max_nr;
+    const bool tensor = h->prm.factor_mode == DD_FACTOR_TENSOR;
+    for (int k0 = 0; k0 < n; k0 += tensor ? kOzNB : kNB) {
+        Prof P(h, ST_FACTOR, s, 3);
+        const int rc = launch_sweep(h, coarse, k0, s);
+        if (rc) return rc;
+    }
+    if (!tensor) return 0;
+    Prof P(h, ST_FACTOR, s, 1);
+    return launch_mirror(h, coarse, s);
+}
+
+}  // namespace
+
 int dd_factor(dd_handle* h, double dt, void* stream) {
     if (!h) return DD_ERR_ARG;
     if (!h->bound) return h->fail(DD_ERR_STATE, "dd_factor before dd_bind_workspace");
@@ -1083,20 +1098,14 @@ int dd_factor(dd_handle* h, double dt, void* stream) {
         Prof P(h, ST_FACTOR, s, 1);
         CK(h, launch_robin_add(h, alpha, s), "Robin term");
     }
-    for (int k0 = 0; k0 < h->max_nr; k0 += kNB) {
-        Prof P(h, ST_FACTOR, s, 3);
-        CK(h, launch_sweep(h, false, k0, s), "local elimination");
-    }
+    CK(h, eliminate(h, false, s), "local elimination");
     const int nc = (int)h->corner_dof.size();
     if (nc && h->ldc) {
         {
             Prof P(h, ST_FACTOR, s, 1);
             CK(h, launch_coarse_assemble(h, s), "coarse assemble");
         }
-        for (int k0 = 0; k0 < nc; k0 += kNB) {
-            Prof P(h, ST_FACTOR, s, 3);
-            CK(h, launch_sweep(h, true, k0, s), "coarse inverse");
-        }
+        CK(h, eliminate(h, true, s), "coarse inverse");
     }
     {
         Prof P(h, ST_FACTOR, s, 3);

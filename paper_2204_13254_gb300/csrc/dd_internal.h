@@ -323,9 +323,8 @@ struct DevPtrs {
     uint32_t* sym_tl[GEMV_NMODES] = {};   // tiles of each packed mode, every subdomain in row order
     double* K64 = nullptr;           // K~cc^-1, n_corner x ldc
     float* K32 = nullptr;
-    double* Pinv = nullptr;          // [n_sub+1][NB*NB] pivot-block inverses while factoring
-    uint16_t* oz_slices = nullptr;   // DD_FACTOR_TENSOR: BF16 slices of one pivot block's panels
-    int32_t* oz_exps = nullptr;      // and their row / column exponents
+    double* Pinv = nullptr;          // [n_sub+1][NB*NB] pivot-block inverses (DD_FACTOR_FP64)
+    unsigned char* oz = nullptr;     // DD_FACTOR_TENSOR: slices and exponents of one pivot block
     double* dinv = nullptr;          // [n_lambda] inverse Jacobi diagonal
     // particles (dd_set_beam): state, per-tet geometry and faces
     double* px = nullptr;            // [n_p*3] positions
@@ -562,7 +561,8 @@ struct dd_handle {
     }
 };
 
-constexpr int kNB = 32;              // pivot block of the dense elimination
+constexpr int kNB = 32;              // pivot block of the dense elimination (DD_FACTOR_FP64)
+constexpr int kOzNB = 64;            // pivot block of the tensor-core elimination (DD_FACTOR_TENSOR)
 // default tile shapes per mode (LOCAL, SCHUR_C, CORNER, RECOVER, COARSE, SCHUR_G, COUPLED):
 // rows per CTA, and lanes per row for FP32 and FP64 (8 lanes for FP64 keeps the
 // FP64 reduction adds off GB300's narrow FP64 pipe)
@@ -583,6 +583,7 @@ size_t dd_workspace_layout(dd_handle* h, bool assign);
 int launch_csr_combine(const dd_handle* h, double ca, void* stream);
 int launch_dense_assemble(const dd_handle* h, void* stream);
 int launch_sweep(const dd_handle* h, bool coarse, int k0, void* stream);
+int launch_mirror(const dd_handle* h, bool coarse, void* stream);
 int launch_coarse_assemble(const dd_handle* h, void* stream);
 int launch_factor_finish(const dd_handle* h, void* stream);
 int launch_rhs(const dd_handle* h, const double* e_n, const double* src, double src_sign, double dt, void* stream);
@@ -630,9 +631,10 @@ size_t sym_smem_bytes(const dd_handle* h);
 // rectangle has no symmetric twin, so one problem gains almost nothing; an ensemble shares the reads).
 bool sym_active(const dd_handle* h, int mode);
 // ozaki.cu
-size_t oz_slice_elems(int nm, int nmax);
-int launch_oz_update(const MatDesc* mats, double* M, int nm, int nmax, int k0, uint16_t* slices, int32_t* exps,
-                     int32_t* err, void* stream);
+size_t oz_bytes(int nm, int nmax);
+int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, unsigned char* ws, int32_t* status,
+                    int32_t* err, void* stream);
+int launch_oz_mirror(const MatDesc* mats, double* M, int nm, int nmax, void* stream);
 // tensor.cu
 void build_tc(dd_handle* h);
 int launch_tc_pack(const dd_handle* h, void* stream);

@@ -1142,6 +1142,8 @@ int launch_sweep(const dd_handle* h, bool coarse, int k0, void* stream) {
     double* M = coarse ? h->d.K64 : h->d.M64;
     const int nm = coarse ? 1 : h->n_sub_real;
     const int nmax = coarse ? (int)h->corner_dof.size() : h->max_ns;
+    if (h->prm.factor_mode == DD_FACTOR_TENSOR)
+        return launch_oz_sweep(mats, M, nm, nmax, k0, h->d.oz, h->d.status, &h->d.sc->wait_err, stream);
     double* Pinv = coarse ? h->d.Pinv + (size_t)h->n_sub * kNB * kNB : h->d.Pinv;
     // chunks of rows (column panel), and of columns (row panel) for the coarse matrix, whose
     // thousands of rows one CTA per pivot block would serialise; the many local matrices keep one CTA
@@ -1149,16 +1151,15 @@ int launch_sweep(const dd_handle* h, bool coarse, int k0, void* stream) {
     const unsigned gp = coarse ? (unsigned)((nmax + kThreads - 1) / kThreads) : 1u;
     const unsigned gc = (unsigned)((nmax + kColRows - 1) / kColRows);
     k_sweep_pivot<<<dim3((unsigned)nm, gp), kThreads, 0, S(stream)>>>(mats, M, k0, Pinv, h->d.status);
-    if (h->prm.factor_mode == DD_FACTOR_TENSOR) {
-        const int rc = launch_oz_update(mats, M, nm, nmax, k0, h->d.oz_slices, h->d.oz_exps, &h->d.sc->wait_err, stream);
-        if (rc) return rc;
-    } else {
-        const int tiles = (nmax + 63) / 64;
-        dim3 grid(tiles, tiles, nm);
-        k_sweep_update<<<grid, kThreads, 0, S(stream)>>>(mats, M, k0);
-    }
+    const int tiles = (nmax + 63) / 64;
+    k_sweep_update<<<dim3(tiles, tiles, nm), kThreads, 0, S(stream)>>>(mats, M, k0);
     k_sweep_colpanel<<<dim3((unsigned)nm, gc), kThreads, 0, S(stream)>>>(mats, M, k0, Pinv);
     return (int)cudaGetLastError();
+}
+
+int launch_mirror(const dd_handle* h, bool coarse, void* stream) {
+    return launch_oz_mirror(coarse ? h->d.coarse_desc : h->d.mats, coarse ? h->d.K64 : h->d.M64,
+                            coarse ? 1 : h->n_sub_real, coarse ? (int)h->corner_dof.size() : h->max_ns, stream);
 }
 
 int launch_coarse_assemble(const dd_handle* h, void* stream) {

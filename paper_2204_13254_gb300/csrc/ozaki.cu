@@ -1,28 +1,40 @@
-// FP64-accurate trailing update of the elimination on the tensor cores (sm_103a).
+// FP64-accurate elimination on the tensor cores (sm_103a): the exchange sweep of
+// every symmetric matrix of a batch in 64-wide pivot blocks, its products formed
+// from BF16 slices on tcgen05 instead of FP64 FMAs (the Ozaki splitting of a
+// product into exact low-precision products).
 //
-// The exchange sweep's trailing update C[i][j] += A[i][:] B[:][j] (A the pivot
-// block's column panel, B its row panel already multiplied by -P^-1, K = 32) is
-// formed from BF16 slices on tcgen05 instead of FP64 FMAs (the Ozaki splitting
-// of a product into exact low-precision products):
-//  * each row i of A is scaled by a power of two 2^-e_i so that |A_ik| 2^-e_i < 1,
-//    each column j of B by 2^-f_j likewise;
-//  * the scaled values are cut into seven slices of 8 bits: r_0 = A 2^-e, then
-//    a_p = rint(r_p 2^8), r_{p+1} = r_p 2^8 - a_p, so that
-//    A 2^-e = sum_p 2^-8(p+1) a_p with integer slices |a_0| <= 256, |a_p| <= 128
-//    (exact in BF16), and the same for B;
-//  * for every weight class d = p + q <= 6 the products a_p b_q are summed over
-//    K = 32 and over the (d + 1) slice pairs of the class in one FP32
-//    accumulator in tensor memory: every partial sum is an integer below 2^24,
-//    so the accumulation is exact;
-//  * the classes are combined exactly in 64-bit integers (two partial sums, each
-//    exact as a double, joined by one FMA) and scaled back with one FP64 FMA:
-//    C_ij += 2^(e_i + f_j - 16) sum_d 2^-8d D_d[i][j].
-// Dropping the classes d >= 7 leaves an error below 2^-55 of |A_i||B_j| per
-// term, i.e. FP64 accuracy.  The FP64 work per matrix element and pivot block
-// falls from 32 FMAs to two conversions and two FMAs; the tensor cores do 28 x 2 MMAs
-// (M = 128 rows, N = 32 columns, K = 16) per 128 x 32 tile.
+// Splitting.  A vector v is scaled by a power of two 2^-e so that |v_k| 2^-e < 1 and
+// rounded to the integers t_k = rint(v_k 2^(56-e)), written in seven balanced
+// 8-bit digits, t = sum_p 2^(8 (6-p)) a_p with |a_0| <= 256, |a_p| <= 128 (exact
+// in BF16).  For two such vectors and every weight class d = p + q <= 6 the
+// products a_p b_q are summed over K = 64 and over the class's d + 1 pairs in one
+// FP32 accumulator in tensor memory: every partial sum is an integer below
+// 64 (2 2^15 + 5 2^14) < 2^24, so the accumulation is exact.  The classes are
+// joined in 64-bit integers (T, exact but for a rounding below 2^-62 of the
+// largest product) and scaled back with one conversion and one FP64 FMA.
+// Dropping the classes d >= 7 leaves an error below 2^-54 of |A_i||B_j| per term:
+// FP64 accuracy.
+//
+// Symmetry.  While a set K of indices has been swept, M_ij = M_ji when both or
+// none of i, j are in K and M_ij = -M_ji otherwise, so only the lower triangle is
+// kept (k_oz_mirror fills the rest at the end), and the column panel of a pivot
+// block p is its row panel B = M[p, :] transposed up to the sign s_i = -1 for
+// swept rows, +1 otherwise.  One pivot block is three kernels:
+//   k_oz_pivot   P^-1 in FP64 (64 x 64, one CTA per matrix), its slices;
+//   k_oz_panel   slices of B; B' = -P^-1 B as a slice product; slices of B'; the
+//                row and column panels of M;
+//   k_oz_update  M_ij += s_i B_i . B'_j over the lower triangle outside p.
+// What bounds it: the update's two FP64 operations per element and pivot block
+// (GB300: two FP64 lanes per clock and SM) against 16 bytes of HBM traffic; the
+// wide pivot block and the triangle each halve both against 32-wide blocks over
+// the full square.  Measured, 40 matrices of up to 2,454 rows with their 1,229-row
+// coarse matrix: pivot 0.12, panel 0.08, update 0.38 ms per 64-wide block (mean over
+// both), against 0.51 + 0.09 (panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide
+// block over the full square; the whole factorisation 34 against 170 ms.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "dd_internal.h"
 #include "tcgen05.cuh"
@@ -31,97 +43,93 @@ namespace {
 
 constexpr int kOzS = 7;                      // slices per operand (8 bits each)
 constexpr int kOzRows = 128;                 // rows of a tile (MMA M)
-constexpr int kOzCols = 32;                  // columns of a tile (MMA N)
-constexpr int kOzK = kNB;                    // pivot block width (MMA K = 2 x 16)
-constexpr uint32_t kOzAPiece = kOzRows * kOzK * 2;   // 8 KB: one slice of a 128-row block
-constexpr uint32_t kOzBPiece = kOzCols * kOzK * 2;   // 2 KB: one slice of a 32-column block
-constexpr uint32_t kOzABytes = kOzS * kOzAPiece;     // 56 KB
-constexpr uint32_t kOzBBytes = kOzS * kOzBPiece;     // 14 KB
+constexpr int kOzCols = 32;                  // columns of one unit of the update (MMA N)
+constexpr int kOzK = kOzNB;                  // pivot block width (MMA K = 4 x 16)
+constexpr uint32_t kOzPiece = kOzRows * kOzK * 2;    // 16 KB: one slice of a 128-row block
+constexpr uint32_t kOzBlock = kOzS * kOzPiece;       // 112 KB: the slices of a 128-row block
+constexpr uint32_t kOzPPiece = kOzK * kOzK * 2;      // 8 KB: one slice of P^-1
+constexpr uint32_t kOzPBlock = kOzS * kOzPPiece;     // 56 KB
+constexpr uint32_t kOzUPiece = kOzCols * kOzK * 2;   // 4 KB: one slice of a 32-column unit
+constexpr uint32_t kOzUnit = kOzS * kOzUPiece;       // 28 KB
 constexpr unsigned kOzPolls = 1u << 22;
-static_assert(kOzK == 32, "the slice layout assumes a 32-wide pivot block");
+static_assert(kOzK == 64, "the slice layout and the exactness bound assume a 64-wide pivot block");
 
 inline cudaStream_t S(void* s) { return (cudaStream_t)s; }
 
-// Exponent e with |x| < 2^e for the largest |x| (0 for an all-zero vector).
-__device__ __forceinline__ int scale_exp(double maxabs) {
-    if (!(maxabs > 0.0)) return 0;
-    int e;
-    frexp(maxabs, &e);   // maxabs = f 2^e, f in [0.5, 1)
-    return e;
+// Exponent e with |x| < 2^e, from the high word (without its sign) of the largest
+// |x| (0 when that is zero or subnormal: its digits are then zero).
+__device__ __forceinline__ int exp_of_hi(int hi) {
+    const int f = hi >> 20;
+    return f == 0 ? 0 : f - 1022;
 }
 
-// The seven 8-bit slices of r = x 2^-e (|r| < 1) as BF16 bits.
-__device__ __forceinline__ void cut(double x, int e, uint16_t* out) {
-    double r = ldexp(x, -e);
-#pragma unroll
-    for (int p = 0; p < kOzS; ++p) {
-        const double t = r * 256.0;
-        const double a = rint(t);
-        r = t - a;
-        out[p] = __bfloat16_as_ushort(__double2bfloat16(a));
-    }
+// 2^x for any x a product's exponents give.
+__device__ __forceinline__ double pow2(int x) {
+    if (x > -1023 && x < 1024) return __longlong_as_double((long long)(x + 1023) << 52);
+    return ldexp(1.0, x);
 }
 
-// Column panel A = M[i][k0 .. k0+nb) of every matrix: one CTA per (128-row block,
-// matrix), one thread per row.  Slices in the K-major core-matrix layout of the
-// MMA's A operand (K = 32), row exponents e_i.
-__global__ void __launch_bounds__(kOzRows) k_oz_split_a(const MatDesc* __restrict__ mats, const double* __restrict__ M,
-                                                        int k0, int nblk, uint16_t* __restrict__ As,
-                                                        int32_t* __restrict__ ea, int nmax) {
-    const int m = blockIdx.y, rb = blockIdx.x;
-    const MatDesc md = mats[m];
-    if (k0 >= md.nr || rb * kOzRows >= md.ns) return;
-    const int nb = min(kOzK, md.nr - k0);
-    const int r = threadIdx.x, i = rb * kOzRows + r;
-    double v[kOzK];
-    double mx = 0.0;
-#pragma unroll
-    for (int k = 0; k < kOzK; ++k) {
-        v[k] = (i < md.ns && k < nb) ? M[md.moff + (int64_t)i * md.ld + k0 + k] : 0.0;
-        mx = fmax(mx, fabs(v[k]));
-    }
-    const int e = scale_exp(mx);
-    if (i < md.ns) ea[(int64_t)m * nmax + i] = e;
-    uint16_t* out = As + ((int64_t)m * nblk + rb) * (kOzABytes / 2);
-#pragma unroll
-    for (int k = 0; k < kOzK; ++k) {
-        uint16_t s[kOzS];
-        cut(v[k], e, s);
-        const uint32_t o = tc::kmajor_off(r, k, kOzK) / 2;
-#pragma unroll
-        for (int p = 0; p < kOzS; ++p) out[p * (kOzAPiece / 2) + o] = s[p];
-    }
+// An integer |d| <= 256 as FP32 (exact; its upper 16 bits are the BF16 value).
+__device__ __forceinline__ uint32_t small_float(int d) {
+    return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
 }
 
-// Row panel B = M[k0 .. k0+nb)[j] (already -P^-1 times the pivot rows): one CTA
-// per (32-column block, matrix), one thread per column; slices in the K-major
-// layout of the MMA's B operand (N = 32 columns, K = 32), column exponents f_j.
-__global__ void __launch_bounds__(kOzCols) k_oz_split_b(const MatDesc* __restrict__ mats, const double* __restrict__ M,
-                                                        int k0, int nblk, uint16_t* __restrict__ Bs,
-                                                        int32_t* __restrict__ fb, int nmax) {
-    const int m = blockIdx.y, cb = blockIdx.x;
-    const MatDesc md = mats[m];
-    if (k0 >= md.nr || cb * kOzCols >= md.ns) return;
-    const int nb = min(kOzK, md.nr - k0);
-    const int c = threadIdx.x, j = cb * kOzCols + c;
-    double v[kOzK];
-    double mx = 0.0;
+// Slices of eight consecutive elements v[0..7] (K direction) of a vector with
+// exponent e: one 16-byte chunk per slice, handed to put(slice, chunk).
+template <typename Put>
+__device__ __forceinline__ void cut8(const double* v, int e, Put put) {
+    const int x = 56 - e;
+    const double sc = pow2(x > 1023 ? 1023 : x);   // e < -967: v below 2^-967, digits from a smaller scale
+    uint32_t w[kOzS][4];
 #pragma unroll
-    for (int k = 0; k < kOzK; ++k) {
-        v[k] = (j < md.ns && k < nb) ? M[md.moff + (int64_t)(k0 + k) * md.ld + j] : 0.0;
-        mx = fmax(mx, fabs(v[k]));
+    for (int q = 0; q < 4; ++q) {
+        uint32_t f[2][kOzS];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long t = __double2ll_rn(v[2 * q + u] * sc);
+            const unsigned long long b = (unsigned long long)t + 0x0000808080808080ull;   // balanced digits
+            const uint32_t lo = (uint32_t)b, hi = (uint32_t)(b >> 32);
+            f[u][6] = small_float((int)(lo & 255u) - 128);
+            f[u][5] = small_float((int)((lo >> 8) & 255u) - 128);
+            f[u][4] = small_float((int)((lo >> 16) & 255u) - 128);
+            f[u][3] = small_float((int)(lo >> 24) - 128);
+            f[u][2] = small_float((int)(hi & 255u) - 128);
+            f[u][1] = small_float((int)((hi >> 8) & 255u) - 128);
+            f[u][0] = small_float((int)hi >> 16);
+        }
+#pragma unroll
+        for (int p = 0; p < kOzS; ++p) w[p][q] = __byte_perm(f[0][p], f[1][p], 0x7632);
     }
-    const int f = scale_exp(mx);
-    if (j < md.ns) fb[(int64_t)m * nmax + j] = f;
-    uint16_t* out = Bs + ((int64_t)m * nblk + cb) * (kOzBBytes / 2);
 #pragma unroll
-    for (int k = 0; k < kOzK; ++k) {
-        uint16_t s[kOzS];
-        cut(v[k], f, s);
-        const uint32_t o = tc::kmajor_off(c, k, kOzK) / 2;
-#pragma unroll
-        for (int p = 0; p < kOzS; ++p) out[p * (kOzBPiece / 2) + o] = s[p];
-    }
+    for (int p = 0; p < kOzS; ++p) put(p, make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]));
+}
+
+// Eight columns of the seven class accumulators (stride `cls` tensor-memory columns
+// apart) of the warp's 32 lanes, all loads in flight together.
+__device__ __forceinline__ void ld_classes(uint32_t t, uint32_t cls, uint32_t (&r)[kOzS][8]) {
+#define OZ_O(d) "=r"(r[d][0]), "=r"(r[d][1]), "=r"(r[d][2]), "=r"(r[d][3]), "=r"(r[d][4]), "=r"(r[d][5]), "=r"(r[d][6]), "=r"(r[d][7])
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%56];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%57];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%58];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%59];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%60];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%61];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%48,%49,%50,%51,%52,%53,%54,%55}, [%62];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : OZ_O(0), OZ_O(1), OZ_O(2), OZ_O(3), OZ_O(4), OZ_O(5), OZ_O(6)
+        : "r"(t), "r"(t + cls), "r"(t + 2 * cls), "r"(t + 3 * cls), "r"(t + 4 * cls), "r"(t + 5 * cls), "r"(t + 6 * cls)
+        : "memory");
+#undef OZ_O
+}
+
+// T of one element: sum_d D_d 2^(8 (5-d)) ... in units of 2^-40 of class 0, i.e. the
+// product is T 2^(e + f - 56) (|T| < 2^63; class 6 rounded in, see the file comment).
+__device__ __forceinline__ double join_classes(const uint32_t (&r)[kOzS][8], int c) {
+    auto I = [&](int d) { return (long long)__float2int_rn(__uint_as_float(r[d][c])); };
+    const long long H = (I(0) << 16) + (I(1) << 8) + I(2);
+    const long long L = (I(3) << 24) + (I(4) << 16) + (I(5) << 8) + I(6);
+    return (double)((H << 24) + ((L + 128) >> 8));
 }
 
 __device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity) {
@@ -137,24 +145,31 @@ __device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity) {
     return false;
 }
 
-// One CTA per (128-row block, run of kOzCb 32-column blocks, matrix) of the
-// trailing update: the row block's A slices are copied once and serve every
-// column block of the run; the B slices come through two buffers, the next
-// column block's copy in flight while the current one is combined.  Per column
-// block one thread issues the 28 slice products x 2 K-steps into the seven
-// class accumulators (224 tensor-memory columns), then the 256 threads combine
-// them: warp w reads rows 32 (w mod 4) .. + 31 (its tensor-memory lane
-// quarter) and columns 16 (w / 4) .. + 15, and adds the exact FP64 update to C
-// (the pivot rows and columns are left alone).  Every wait is bounded; a CTA
-// whose wait gives up sets the error word, lets its copies land and frees its
-// tensor memory.
-constexpr int kOzCb = 8;   // column blocks per CTA
-constexpr int kOzThreads = 256;
-constexpr size_t kOzSmem = kOzABytes + 2 * kOzBBytes + 8 * sizeof(uint64_t) + 16;
+__device__ __forceinline__ bool oz_wait_or_abort(uint64_t* bar, uint32_t parity, const volatile int* abort) {
+    for (unsigned k = 0; k < kOzPolls; ++k) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(tc::smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((k & 255u) == 255u && *abort) return false;
+    }
+    return false;
+}
 
-__device__ __forceinline__ void oz_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void oz_init(uint64_t* bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc::smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void oz_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void oz_expect(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_addr(bar)), "r"(bytes)
                  : "memory");
+}
+__device__ __forceinline__ void oz_bulk(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
             tc::smem_addr(dst)),
@@ -162,158 +177,525 @@ __device__ __forceinline__ void oz_copy(void* dst, const void* src, uint32_t byt
         : "memory");
 }
 
-__global__ void __launch_bounds__(kOzThreads, 2) k_oz_update(const MatDesc* __restrict__ mats, double* __restrict__ M,
-                                                          int k0, int nrb, int ncb, const uint16_t* __restrict__ As,
-                                                          const uint16_t* __restrict__ Bs,
-                                                          const int32_t* __restrict__ ea,
-                                                          const int32_t* __restrict__ fb, int nmax,
-                                                          int32_t* __restrict__ err) {
-    const int m = blockIdx.z, rb = blockIdx.y, cb0 = blockIdx.x * kOzCb;
+// The 28 slice products (x 4 K-steps) of A rows (slices at a0, sa bytes apart) and B
+// rows (b0, sb apart) into the class accumulators at `acc`, `cls` columns apart.
+__device__ __forceinline__ void oz_products(uint32_t acc, uint32_t cls, uint32_t a0, uint32_t sa, uint32_t b0,
+                                            uint32_t sb, uint32_t idesc) {
+    for (int d = 0; d < kOzS; ++d)
+        for (int p = 0; p <= d; ++p)
+            for (int ks = 0; ks < kOzK / 16; ++ks) {
+                const uint64_t ad = tc::smem_desc(a0 + p * sa + ks * 256, 128, (kOzK / 8) * 128);
+                const uint64_t bd = tc::smem_desc(b0 + (d - p) * sb + ks * 256, 128, (kOzK / 8) * 128);
+                tc::mma_bf16(acc + d * cls, ad, bd, idesc, (p | ks) ? 1u : 0u);
+            }
+}
+
+// ---- pivot block -------------------------------------------------------------
+// P^-1 of the pivot block by a Gauss-Jordan sweep (SPD: no pivoting) over its lower
+// triangle in registers: thread (ty, tx) of 16 x 16 holds elements (ty + 16 u, tx + 16 v),
+// v <= u.  Step k publishes the vector r (row k left of the diagonal, column k below
+// it) and 1 / d; then P_ij -= (s_i r_i) (r_j / d).  One CTA per matrix: the 64 steps
+// are a serial chain of ten FMAs per thread, FP64-ALU bound.  Writes P^-1 back into
+// M[p, p] (the panel kernel does not read that block), and its slices and exponents.
+constexpr int kOzPivThreads = 256;
+__global__ void __launch_bounds__(kOzPivThreads) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
+                                                            int k0, uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
+                                                            int32_t* __restrict__ status) {
+    const MatDesc md = mats[blockIdx.x];
+    if (k0 >= md.nr) return;
+    const int nb = min(kOzK, md.nr - k0);
+    __shared__ double Q[kOzK][kOzK + 1];
+    __shared__ double r[2][kOzK], t[kOzK], sinv[2];   // by step parity: a step's readers meet the next writers two barriers on
+    double* A = M + md.moff + (int64_t)k0 * md.ld + k0;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double a[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v <= u; ++v) {
+            const int i = ty + 16 * u, j = tx + 16 * v;
+            a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : (i == j ? 1.0 : 0.0);
+        }
+    for (int k = 0; k < nb; ++k) {
+        double* rk = r[k & 1];
+        const int uk = k >> 4, kk = k & 15;
+        // publish row k (j < k) and column k (i > k), and 1 / d
+        if (ty == kk) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    if (u != uk) continue;
+                    const int j = tx + 16 * v;
+                    if (j < k) rk[j] = a[u][v];
+                    if (j == k) {
+                        double d = a[u][v];
+                        if (!(d > 0.0) || !isfinite(d)) {
+                            atomicCAS(status, 0, DD_ERR_NOT_SPD);
+                            d = 1.0;
+                        }
+                        sinv[k & 1] = 1.0 / d;
+                    }
+                }
+        }
+        if (tx == kk) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    if (v != uk) continue;
+                    const int i = ty + 16 * u;
+                    if (i > k) rk[i] = a[u][v];
+                }
+        }
+        __syncthreads();
+        if (tid < kOzK) t[tid] = tid == k ? 0.0 : rk[tid] * sinv[k & 1];
+        __syncthreads();
+        double sr[4], tj[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = ty + 16 * u, j = tx + 16 * u;
+            sr[u] = i == k ? 0.0 : (i < k ? -rk[i] : rk[i]);
+            tj[u] = t[j];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) a[u][v] = fma(-sr[u], tj[v], a[u][v]);
+        // row and column k of the swept matrix
+        if (ty == kk || tx == kk) {
+            const double inv = sinv[k & 1];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    const int i = ty + 16 * u, j = tx + 16 * v;
+                    if (i == k && j == k) a[u][v] = inv;
+                    else if (i == k && j < k) a[u][v] = -t[j];
+                    else if (j == k && i > k) a[u][v] = t[i];
+                }
+        }
+    }
+    // full symmetric P^-1 (zero outside nb)
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v <= u; ++v) {
+            const int i = ty + 16 * u, j = tx + 16 * v;
+            if (j > i) continue;
+            const double x = i < nb ? a[u][v] : 0.0;
+            Q[i][j] = x;
+            Q[j][i] = x;
+        }
+    __syncthreads();
+    for (int p = tid; p < kOzK * kOzK; p += kOzPivThreads) {
+        const int i = p >> 6, j = p & 63;
+        if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i][j];
+    }
+    // slices: thread (row i, quarter q of the 64 columns)
+    const int i = tid >> 2, q = tid & 3;
+    int mx = 0;
+    for (int k = 0; k < 16; ++k) mx = max(mx, __double2hiint(Q[i][16 * q + k]) & 0x7fffffff);
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const int e = exp_of_hi(mx);
+    if (q == 0) ep[(int64_t)blockIdx.x * kOzK + i] = e;
+    unsigned char* out = reinterpret_cast<unsigned char*>(Ps) + (int64_t)blockIdx.x * kOzPBlock;
+    for (int g = 0; g < 2; ++g) {
+        const int k = 16 * q + 8 * g;
+        double v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = Q[i][k + c];
+        cut8(v, e, [&](int p, uint4 w) {
+            *reinterpret_cast<uint4*>(out + p * kOzPPiece + tc::kmajor_off(i, k, kOzK)) = w;
+        });
+    }
+}
+
+// ---- panel -------------------------------------------------------------------
+// One CTA per (128 indices j, matrix), thread (j, half): 32 of the 64 pivot rows each.
+// The panel's values (row-read for swept j, column-read below the block) become slices
+// in shared memory (the MMA's A operand) and in global memory (the update's rows); the
+// slice product with P^-1 gives B' = -P^-1 B, which is written back to the row panel
+// (j < k0) or, negated, to the column panel (j >= k0 + nb), and cut into slices again
+// (the update's columns).  168 KB of shared memory, 448 tensor-memory columns.
+constexpr int kOzPanThreads = 256;
+constexpr size_t kOzPanSmem = kOzBlock + kOzPBlock + 64;
+__global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __restrict__ mats, double* __restrict__ M,
+                                                               int k0, int nrb, const uint16_t* __restrict__ Ps,
+                                                               const int32_t* __restrict__ ep, uint16_t* __restrict__ Bs,
+                                                               int32_t* __restrict__ eb, uint16_t* __restrict__ Cs,
+                                                               int32_t* __restrict__ ec, int nmax,
+                                                               int32_t* __restrict__ err) {
+    const int m = blockIdx.y, rb = blockIdx.x;
     const MatDesc md = mats[m];
-    const int ncb_m = (md.ns + kOzCols - 1) / kOzCols;
-    if (k0 >= md.nr || rb * kOzRows >= md.ns || cb0 >= ncb_m) return;
-    const int nc = min(kOzCb, ncb_m - cb0);   // column blocks of this CTA
+    if (k0 >= md.nr || rb * kOzRows >= md.ns) return;
     const int nb = min(kOzK, md.nr - k0);
     extern __shared__ __align__(128) unsigned char sm[];
-    unsigned char* sA = sm;
-    unsigned char* sB = sm + kOzABytes;   // [2][kOzBBytes]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + 2 * kOzBBytes);   // [0] A, [1..2] B buffers, [3] MMAs
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint16_t* gb = Bs + ((int64_t)m * ncb + cb0) * (kOzBBytes / 2);
+    unsigned char* sB = sm;
+    unsigned char* sP = sm + kOzBlock;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sP + kOzPBlock);   // [0] P^-1 slices, [1] products
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
+    __shared__ int xmax[2][kOzRows];
+    const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
-        for (int q = 0; q < 4; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc::smem_addr(&bars[q])) : "memory");
+        oz_init(&bars[0], 1);
+        oz_init(&bars[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        oz_copy(sA, As + ((int64_t)m * nrb + rb) * (kOzABytes / 2), kOzABytes, &bars[0]);
-        oz_copy(sB, gb, kOzBBytes, &bars[1]);
+        oz_expect(&bars[0], kOzPBlock);
+        oz_bulk(sP, reinterpret_cast<const unsigned char*>(Ps) + (int64_t)m * kOzPBlock, kOzPBlock, &bars[0]);
     }
-    if (warp == 0) tc::tmem_alloc(tslot, 256);
+    if (warp == 0) tc::tmem_alloc(tslot, 512);
+    const int r = tid & (kOzRows - 1), half = tid >> 7, kb = 32 * half;
+    const int j = rb * kOzRows + r;
+    const bool on = j < md.ns && (j < k0 || j >= k0 + nb);
+    const bool row = j < k0;   // stored in the row panel
+    double* A = M + md.moff;
+    double v[32];
+    int mx = 0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const bool in = on && kb + k < nb;
+        v[k] = in ? (row ? A[(int64_t)(k0 + kb + k) * md.ld + j] : A[(int64_t)j * md.ld + k0 + kb + k]) : 0.0;
+        mx = max(mx, __double2hiint(v[k]) & 0x7fffffff);
+    }
+    xmax[half][r] = mx;
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
-    const uint32_t idesc = tc::idesc_bf16_f32(kOzRows, kOzCols);
-    const int r = 32 * (warp & 3) + lane, hcol = 16 * (warp >> 2);
-    const int i = rb * kOzRows + r;
-    const bool row_ok = i < md.ns && (i < k0 || i >= k0 + nb);
-    const int e = row_ok ? ea[(int64_t)m * nmax + i] : 0;
-    double* crow = M + md.moff + (int64_t)i * md.ld;
-    int issued_b = 1;   // B copies issued (thread 0)
-    bool good = true;
-    for (int c = 0; c < nc && good; ++c) {
-        const int buf = c & 1;
-        bool ok = true;   // thread 0: the copies of this column block arrived
-        if (tid == 0) {
-            ok = (c > 0 || oz_wait(&bars[0], 0u)) && oz_wait(&bars[1 + buf], (uint32_t)(c >> 1) & 1u);
-            if (ok) {
-                tc::fence_after_sync();
-                const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB + buf * kOzBBytes);
-                for (int d = 0; d < kOzS; ++d) {
-                    bool first = true;
-                    for (int p = 0; p <= d; ++p) {
-                        const int q = d - p;
-                        for (int ks = 0; ks < kOzK / 16; ++ks) {
-                            const uint64_t ad = tc::smem_desc(a0 + p * kOzAPiece + ks * 256, 128, (kOzK / 8) * 128);
-                            const uint64_t bd = tc::smem_desc(b0 + q * kOzBPiece + ks * 256, 128, (kOzK / 8) * 128);
-                            tc::mma_bf16(tmem + d * kOzCols, ad, bd, idesc, first ? 0u : 1u);
-                            first = false;
-                        }
-                    }
-                }
-            }
-            tc::mma_commit(&bars[3]);   // arrives once the MMAs issued above (if any) have completed
-            // the other buffer's products (column block c - 1) completed before its combination
-            if (ok && c + 1 < nc) {
-                oz_copy(sB + (buf ^ 1) * kOzBBytes, gb + (int64_t)(c + 1) * (kOzBBytes / 2), kOzBBytes,
-                        &bars[1 + (buf ^ 1)]);
-                ++issued_b;
-            }
+    const int64_t blk = ((int64_t)m * nrb + rb) * kOzBlock;
+    const int e = exp_of_hi(max(xmax[0][r], xmax[1][r]));
+    {
+        unsigned char* gB = reinterpret_cast<unsigned char*>(Bs) + blk;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const uint32_t o = tc::kmajor_off(r, kb + 8 * g, kOzK);
+            cut8(v + 8 * g, e, [&](int p, uint4 w) {
+                *reinterpret_cast<uint4*>(sB + p * kOzPiece + o) = w;
+                *reinterpret_cast<uint4*>(gB + p * kOzPiece + o) = w;
+            });
         }
-        const bool done = oz_wait(&bars[3], (uint32_t)c & 1u);
-        tc::fence_after_sync();
-        good = __syncthreads_and(done && ok) != 0;
-        if (!good) break;
-        const int cb = cb0 + c;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {   // eight columns at a time (registers)
-            float D[kOzS][8];
-#pragma unroll
-            for (int d = 0; d < kOzS; ++d)
-                tc::tmem_ld8(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + d * kOzCols + hcol + 8 * half, D[d]);
-            if (!row_ok) continue;
-            const int jb = cb * kOzCols + hcol + 8 * half;
-            bool on[8];
-            double cv[8];
-            int fe[8];
-#pragma unroll
-            for (int cc = 0; cc < 8; ++cc) {   // C and the column exponents first, all loads in flight
-                const int j = jb + cc;
-                on[cc] = j < md.ns && (j < k0 || j >= k0 + nb);
-                cv[cc] = on[cc] ? crow[j] : 0.0;
-                fe[cc] = on[cc] ? fb[(int64_t)m * nmax + j] : 0;
-            }
-#pragma unroll
-            for (int cc = 0; cc < 8; ++cc) {
-                if (!on[cc]) continue;
-                // The class sums are exact integers below 2^22: combine them in 64-bit
-                // integer arithmetic, H = D0 2^16 + D1 2^8 + D2 and L = D3 2^24 + D4 2^16 +
-                // D5 2^8 + D6, both exact as doubles, so that
-                // 2^16 sum_d D_d 2^-8d = H + L 2^-32 with one rounding.
-                const long long H = ((long long)__float2int_rn(D[0][cc]) << 16) +
-                                    ((long long)__float2int_rn(D[1][cc]) << 8) + (long long)__float2int_rn(D[2][cc]);
-                const long long L = ((long long)__float2int_rn(D[3][cc]) << 24) +
-                                    ((long long)__float2int_rn(D[4][cc]) << 16) +
-                                    ((long long)__float2int_rn(D[5][cc]) << 8) + (long long)__float2int_rn(D[6][cc]);
-                const double v = fma((double)L, 0x1p-32, (double)H);
-                // times 2^(e + f - 32) from its exponent bits when that is a normal double
-                const int x = e + fe[cc] - 32;
-                const int j = jb + cc;
-                if (x > -1023 && x < 1024) crow[j] = fma(v, __longlong_as_double((long long)(x + 1023) << 52), cv[cc]);
-                else crow[j] = cv[cc] + ldexp(v, x);
-            }
-        }
-        // every thread's tensor-memory reads complete before the next products overwrite the accumulators
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
     }
-    if (!good && tid == 0) {
+    if (half == 0 && j < md.ns) eb[(int64_t)m * nmax + j] = e;
+    tc::fence_proxy_async();
+    __syncthreads();
+    bool ok = true;
+    if (tid == 0) {
+        ok = oz_wait(&bars[0], 0u);
+        if (ok) {
+            tc::fence_after_sync();
+            oz_products(tmem, kOzK, tc::smem_addr(sB), kOzPiece, tc::smem_addr(sP), kOzPPiece,
+                        tc::idesc_bf16_f32(kOzRows, kOzK));
+        }
+        tc::mma_commit(&bars[1]);
+    }
+    const bool done = oz_wait(&bars[1], 0u);
+    tc::fence_after_sync();
+    const bool good = __syncthreads_and(done && ok) != 0;
+    if (good) {
+        mx = 0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            uint32_t D[kOzS][8];
+            ld_classes(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + kb + 8 * g, kOzK, D);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int i = kb + 8 * g + c;
+                const double y = -join_classes(D, c) * pow2(e + ep[(int64_t)m * kOzK + i] - 56);
+                v[8 * g + c] = y;
+                mx = max(mx, __double2hiint(y) & 0x7fffffff);
+            }
+        }
+        if (on) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                if (kb + k >= nb) continue;
+                if (row) A[(int64_t)(k0 + kb + k) * md.ld + j] = v[k];
+                else A[(int64_t)j * md.ld + k0 + kb + k] = -v[k];
+            }
+        }
+    }
+    xmax[half][r] = mx;   // the first exchange was read before the previous barriers
+    __syncthreads();
+    if (good) {
+        const int f = exp_of_hi(max(xmax[0][r], xmax[1][r]));
+        if (half == 0 && j < md.ns) ec[(int64_t)m * nmax + j] = f;
+        unsigned char* gC = reinterpret_cast<unsigned char*>(Cs) + blk;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const uint32_t o = tc::kmajor_off(r, kb + 8 * g, kOzK);
+            cut8(v + 8 * g, f, [&](int p, uint4 w) { *reinterpret_cast<uint4*>(gC + p * kOzPiece + o) = w; });
+        }
+    } else if (tid == 0) {
         atomicExch(err, 1);
-        // the copies issued land before the CTA ends (bounded): A, and the last one of each B buffer
-        oz_wait(&bars[0], 0u);
-        for (int q = issued_b > 2 ? issued_b - 2 : 0; q < issued_b; ++q) oz_wait(&bars[1 + (q & 1)], (uint32_t)(q >> 1) & 1u);
+        oz_wait(&bars[0], 0u);   // the copy lands before the CTA ends (bounded)
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    if (warp == 0) tc::tmem_free(tmem, 256);
+    if (warp == 0) tc::tmem_free(tmem, 512);
+}
+
+// ---- trailing update ------------------------------------------------------------
+// One CTA per (128-row block, run of kOzRun 32-column units of its lower triangle,
+// matrix): the row block's 112 KB of slices are copied once for the run; the units'
+// 28 KB come through a ring of four buffers, two units ahead.  Warp 8 issues the copies
+// and the MMAs of unit u into tensor-memory half u & 1 while warps 0..7 combine unit
+// u - 1 from the other half: warp w reads rows 32 (w mod 4) .. + 31 (its tensor-memory
+// lanes) and columns 16 (w / 4) .. + 15, and adds the exact update to C (loaded before
+// the wait).  Bound by the epilogue's two FP64 operations per element.  Every wait is
+// bounded; a CTA whose wait gives up sets the error word, lets its copies land and
+// frees its tensor memory.
+constexpr int kOzRun = 16;
+constexpr int kOzStages = 4;
+constexpr int kOzThreads = 288;
+constexpr size_t kOzSmem = kOzBlock + kOzStages * kOzUnit + (1 + 2 * kOzStages + 4) * sizeof(uint64_t) + 16;
+static_assert(kOzSmem <= 227 * 1024, "shared memory of the update");
+
+__global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __restrict__ mats, double* __restrict__ M,
+                                                             int k0, int nrb, const uint16_t* __restrict__ Bs,
+                                                             const uint16_t* __restrict__ Cs,
+                                                             const int32_t* __restrict__ eb,
+                                                             const int32_t* __restrict__ ec, int nmax,
+                                                             int32_t* __restrict__ err) {
+    const int m = blockIdx.y;
+    const MatDesc md = mats[m];
+    // blockIdx.x -> (row block, run): row block rb has ceil(4 (rb + 1) / kOzRun) runs
+    int rb = 0, run = (int)blockIdx.x;
+    for (;;) {
+        const int nrun = (4 * (rb + 1) + kOzRun - 1) / kOzRun;
+        if (run < nrun) break;
+        run -= nrun;
+        ++rb;
+    }
+    if (k0 >= md.nr || rb * kOzRows >= md.ns) return;
+    const int nb = min(kOzK, md.nr - k0);
+    const int u0 = run * kOzRun;
+    const int u1 = min(min(u0 + kOzRun, 4 * (rb + 1)), (md.ns + kOzCols - 1) / kOzCols);
+    // units inside the pivot block are left out
+    const int s0 = k0 / kOzCols, s1 = (k0 + nb) / kOzCols;   // units [s0, s1) lie wholly in it
+    auto unit = [&](int n) {   // the n-th unit of the run
+        int u = u0 + n;
+        if (u >= s0 && u0 < s1) u += u0 >= s0 ? s1 - u0 : s1 - s0;
+        return u;
+    };
+    const int skip = max(0, min(u1, s1) - max(u0, s0));
+    const int nu = u1 - u0 - skip;
+    if (nu <= 0) return;
+
+    extern __shared__ __align__(128) unsigned char sm[];
+    unsigned char* sA = sm;
+    unsigned char* sC = sm + kOzBlock;
+    uint64_t* abar = reinterpret_cast<uint64_t*>(sC + kOzStages * kOzUnit);
+    uint64_t* full = abar + 1;             // [stage] unit copied
+    uint64_t* empty = full + kOzStages;    // [stage] its products completed
+    uint64_t* tfull = empty + kOzStages;   // [half] products in tensor memory
+    uint64_t* tempty = tfull + 2;          // [half] read by the eight warps
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
+    __shared__ int abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned char* gC = reinterpret_cast<const unsigned char*>(Cs) + (int64_t)m * nrb * kOzBlock;
+    int issued = 0;   // unit copies issued (the issuing lane)
+    auto copy_unit = [&](int n) {
+        const int u = unit(n), s = n % kOzStages;
+        const unsigned char* src = gC + (int64_t)(u >> 2) * kOzBlock + (u & 3) * kOzUPiece;
+        oz_expect(&full[s], kOzUnit);
+#pragma unroll
+        for (int p = 0; p < kOzS; ++p) oz_bulk(sC + s * kOzUnit + p * kOzUPiece, src + p * kOzPiece, kOzUPiece, &full[s]);
+        ++issued;
+    };
+    if (tid == 256) {
+        abort_flag = 0;
+        oz_init(abar, 1);
+        for (int s = 0; s < kOzStages; ++s) {
+            oz_init(&full[s], 1);
+            oz_init(&empty[s], 1);
+        }
+        for (int hh = 0; hh < 2; ++hh) {
+            oz_init(&tfull[hh], 1);
+            oz_init(&tempty[hh], 8);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        oz_expect(abar, kOzBlock);
+        oz_bulk(sA, reinterpret_cast<const unsigned char*>(Bs) + ((int64_t)m * nrb + rb) * kOzBlock, kOzBlock, abar);
+        for (int n = 0; n < 2 && n < nu; ++n) copy_unit(n);
+    }
+    if (warp == 0) tc::tmem_alloc(tslot, 512);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tslot;
+
+    if (warp == 8) {
+        if (lane == 0) {
+            const uint32_t idesc = tc::idesc_bf16_f32(kOzRows, kOzCols);
+            bool ok = oz_wait(abar, 0u);
+            for (int n = 0; n < nu && ok; ++n) {
+                const int s = n % kOzStages, hh = n & 1;
+                if (n + 2 < nu) {   // unit n + 2 into the stage of unit n - 2
+                    if (n >= 2) ok = oz_wait_or_abort(&empty[(n - 2) % kOzStages], (uint32_t)((n - 2) / kOzStages) & 1u, &abort_flag);
+                    if (!ok) break;
+                    copy_unit(n + 2);
+                }
+                ok = oz_wait_or_abort(&full[s], (uint32_t)(n / kOzStages) & 1u, &abort_flag);
+                if (ok && n >= 2) ok = oz_wait_or_abort(&tempty[hh], (uint32_t)((n >> 1) - 1) & 1u, &abort_flag);
+                if (!ok) break;
+                tc::fence_after_sync();
+                oz_products(tmem + 256u * hh, kOzCols, tc::smem_addr(sA), kOzPiece, tc::smem_addr(sC + s * kOzUnit),
+                            kOzUPiece, idesc);
+                tc::mma_commit(&tfull[hh]);
+                tc::mma_commit(&empty[s]);
+            }
+            if (!ok) abort_flag = 1;
+        }
+    } else {
+        const int r = 32 * (warp & 3) + lane, hcol = 16 * (warp >> 2);
+        const int i = rb * kOzRows + r;
+        const bool row_ok = i < md.ns && (i < k0 || i >= k0 + nb);
+        const int e = row_ok ? eb[(int64_t)m * nmax + i] : 0;
+        const double sgn = i < k0 ? -1.0 : 1.0;
+        double* crow = M + md.moff + (int64_t)i * md.ld;
+        const int32_t* ecm = ec + (int64_t)m * nmax;
+        for (int n = 0; n < nu; ++n) {
+            const int hh = n & 1, j0 = unit(n) * kOzCols + hcol;
+            // columns j0 .. j0 + 15 of row i inside the lower triangle and outside the pivot block
+            const int jend = row_ok ? min(min(i + 1, md.ns), j0 + 16) : j0;
+            const bool whole = jend == j0 + 16 && (j0 + 16 <= k0 || j0 >= k0 + nb);
+            double c[16];
+            if (whole) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const double2 t = *reinterpret_cast<const double2*>(crow + j0 + 2 * q);
+                    c[2 * q] = t.x;
+                    c[2 * q + 1] = t.y;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const int j = j0 + q;
+                    c[q] = (j < jend && (j < k0 || j >= k0 + nb)) ? crow[j] : 0.0;
+                }
+            }
+            const bool ok = oz_wait_or_abort(&tfull[hh], (uint32_t)(n >> 1) & 1u, &abort_flag);
+            if (__any_sync(0xffffffffu, !ok)) {
+                abort_flag = 1;
+                break;
+            }
+            tc::fence_after_sync();
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                uint32_t D[kOzS][8];
+                ld_classes(tmem + 256u * hh + ((uint32_t)(32 * (warp & 3)) << 16) + hcol + 8 * g, kOzCols, D);
+                if (g == 1) {   // the half is read: the next products may overwrite it
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) oz_arrive(&tempty[hh]);
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int j = j0 + 8 * g + q;
+                    const int f = j < jend ? ecm[j] : 0;
+                    c[8 * g + q] = fma(join_classes(D, q), sgn * pow2(e + f - 56), c[8 * g + q]);
+                }
+            }
+            if (whole) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    *reinterpret_cast<double2*>(crow + j0 + 2 * q) = make_double2(c[2 * q], c[2 * q + 1]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const int j = j0 + q;
+                    if (j < jend && (j < k0 || j >= k0 + nb)) crow[j] = c[q];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (abort_flag && tid == 256) {   // the copies issued land before the CTA ends (bounded), then report
+        oz_wait(abar, 0u);
+        for (int n = issued > kOzStages ? issued - kOzStages : 0; n < issued; ++n)
+            oz_wait(&full[n % kOzStages], (uint32_t)(n / kOzStages) & 1u);
+        atomicExch(err, 1);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_free(tmem, 512);
+}
+
+// M[i][j] for j > i from the lower triangle: -M[j][i] when exactly one index was swept
+// (i < nr <= j), M[j][i] otherwise.  One CTA per 64 x 64 tile pair, through shared memory.
+__global__ void __launch_bounds__(256) k_oz_mirror(const MatDesc* __restrict__ mats, double* __restrict__ M) {
+    const MatDesc md = mats[blockIdx.y];
+    int a = 0, b = (int)blockIdx.x;   // tile (a, b), b <= a
+    while (b > a) b -= ++a;
+    if (a * 64 >= md.ns) return;
+    __shared__ double t[64][65];
+    double* A = M + md.moff;
+    const int lx = threadIdx.x & 63, ly = threadIdx.x >> 6;
+    for (int y = ly; y < 64; y += 4) {
+        const int i = a * 64 + y, j = b * 64 + lx;
+        if (i < md.ns && j < i) t[y][lx] = (j < md.nr && i >= md.nr) ? -A[(int64_t)i * md.ld + j] : A[(int64_t)i * md.ld + j];
+    }
+    __syncthreads();
+    for (int y = ly; y < 64; y += 4) {
+        const int j = b * 64 + y, i = a * 64 + lx;   // element (j, i) of the upper triangle
+        if (i < md.ns && j < i) A[(int64_t)j * md.ld + i] = t[lx][y];
+    }
 }
 
 }  // namespace
 
-// Workspace of the tensor-core update: slices and exponents of one pivot block.
-size_t oz_slice_elems(int nm, int nmax) {
-    const size_t nrb = (size_t)(nmax + kOzRows - 1) / kOzRows, ncb = (size_t)(nmax + kOzCols - 1) / kOzCols;
-    return (size_t)nm * (nrb * (kOzABytes / 2) + ncb * (kOzBBytes / 2));
+// Workspace of one pivot block (bytes): slices of P^-1, B and B' and their exponents.
+namespace {
+struct OzLayout {
+    size_t ps, bs, cs, ep, eb, ec, total;
+};
+OzLayout oz_layout(int nm, int nmax) {
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t nrb = (size_t)(nmax + kOzRows - 1) / kOzRows;
+    OzLayout L;
+    L.ps = 0;
+    L.bs = L.ps + up((size_t)nm * kOzPBlock);
+    L.cs = L.bs + up((size_t)nm * nrb * kOzBlock);
+    L.ep = L.cs + up((size_t)nm * nrb * kOzBlock);
+    L.eb = L.ep + up((size_t)nm * kOzK * sizeof(int32_t));
+    L.ec = L.eb + up((size_t)nm * nmax * sizeof(int32_t));
+    L.total = L.ec + up((size_t)nm * nmax * sizeof(int32_t));
+    return L;
+}
+}  // namespace
+
+size_t oz_bytes(int nm, int nmax) { return oz_layout(nm, std::max(nmax, 1)).total; }
+
+// One pivot block [k0, k0 + 64) of the sweep of nm matrices (of at most nmax rows).
+int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, unsigned char* ws, int32_t* status,
+                    int32_t* err, void* stream) {
+    const int nrb = (nmax + kOzRows - 1) / kOzRows;
+    const OzLayout L = oz_layout(nm, nmax);
+    uint16_t* Ps = reinterpret_cast<uint16_t*>(ws + L.ps);
+    uint16_t* Bs = reinterpret_cast<uint16_t*>(ws + L.bs);
+    uint16_t* Cs = reinterpret_cast<uint16_t*>(ws + L.cs);
+    int32_t* ep = reinterpret_cast<int32_t*>(ws + L.ep);
+    int32_t* eb = reinterpret_cast<int32_t*>(ws + L.eb);
+    int32_t* ec = reinterpret_cast<int32_t*>(ws + L.ec);
+    cudaError_t e = cudaFuncSetAttribute(k_oz_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzPanSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_oz_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+    if (e != cudaSuccess) return (int)e;
+    k_oz_pivot<<<(unsigned)nm, kOzPivThreads, 0, S(stream)>>>(mats, M, k0, Ps, ep, status);
+    k_oz_panel<<<dim3((unsigned)nrb, (unsigned)nm), kOzPanThreads, kOzPanSmem, S(stream)>>>(mats, M, k0, nrb, Ps, ep, Bs,
+                                                                                            eb, Cs, ec, nmax, err);
+    unsigned runs = 0;
+    for (int rb = 0; rb < nrb; ++rb) runs += (unsigned)((4 * (rb + 1) + kOzRun - 1) / kOzRun);
+    k_oz_update<<<dim3(runs, (unsigned)nm), kOzThreads, kOzSmem, S(stream)>>>(mats, M, k0, nrb, Bs, Cs, eb, ec, nmax, err);
+    return (int)cudaGetLastError();
 }
 
-int launch_oz_update(const MatDesc* mats, double* M, int nm, int nmax, int k0, uint16_t* slices, int32_t* exps,
-                     int32_t* err, void* stream) {
-    const int nrb = (nmax + kOzRows - 1) / kOzRows, ncb = (nmax + kOzCols - 1) / kOzCols;
-    uint16_t* As = slices;
-    uint16_t* Bs = slices + (size_t)nm * nrb * (kOzABytes / 2);
-    int32_t* ea = exps;
-    int32_t* fb = exps + (size_t)nm * nmax;
-    k_oz_split_a<<<dim3((unsigned)nrb, (unsigned)nm), kOzRows, 0, S(stream)>>>(mats, M, k0, nrb, As, ea, nmax);
-    k_oz_split_b<<<dim3((unsigned)ncb, (unsigned)nm), kOzCols, 0, S(stream)>>>(mats, M, k0, ncb, Bs, fb, nmax);
-    // (84 KB of shared memory: at most two CTAs per SM, whose two 256-column tensor-memory allocations
-    // fill its 512 columns)
-    static_assert(3 * (kOzSmem + 1024) > 228 * 1024 && 2 * (kOzSmem + 1024) <= 228 * 1024, "two CTAs per SM");
-    cudaError_t e = cudaFuncSetAttribute(k_oz_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
-    if (e != cudaSuccess) return (int)e;
-    const int nchunk = (ncb + kOzCb - 1) / kOzCb;
-    k_oz_update<<<dim3((unsigned)nchunk, (unsigned)nrb, (unsigned)nm), kOzThreads, kOzSmem, S(stream)>>>(
-        mats, M, k0, nrb, ncb, As, Bs, ea, fb, nmax, err);
+// The upper triangles after the last pivot block.
+int launch_oz_mirror(const MatDesc* mats, double* M, int nm, int nmax, void* stream) {
+    const unsigned nt = (unsigned)(nmax + 63) / 64;
+    k_oz_mirror<<<dim3(nt * (nt + 1) / 2, (unsigned)nm), 256, 0, S(stream)>>>(mats, M);
     return (int)cudaGetLastError();
 }
