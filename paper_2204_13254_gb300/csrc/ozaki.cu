@@ -28,15 +28,16 @@
 // (GB300: two FP64 lanes per clock and SM) against 16 bytes of HBM traffic; the
 // wide pivot block and the triangle each halve both against 32-wide blocks over
 // the full square.  Measured, 40 matrices of up to 2,454 rows with their 1,229-row
-// coarse matrix: pivot 0.12, panel 0.08, update 0.38 ms per 64-wide block (mean over
+// coarse matrix: pivot 0.17, panel 0.08, update 0.38 ms per 64-wide block (mean over
 // both), against 0.51 + 0.09 (panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide
-// block over the full square; the whole factorisation 34 against 170 ms.
+// block over the full square; the whole factorisation 37 against 170 ms.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
 #include "dd_internal.h"
+#include "fixpoint.cuh"
 #include "tcgen05.cuh"
 
 namespace {
@@ -55,19 +56,6 @@ constexpr unsigned kOzPolls = 1u << 22;
 static_assert(kOzK == 64, "the slice layout and the exactness bound assume a 64-wide pivot block");
 
 inline cudaStream_t S(void* s) { return (cudaStream_t)s; }
-
-// Exponent e with |x| < 2^e, from the high word (without its sign) of the largest
-// |x| (0 when that is zero or subnormal: its digits are then zero).
-__device__ __forceinline__ int exp_of_hi(int hi) {
-    const int f = hi >> 20;
-    return f == 0 ? 0 : f - 1022;
-}
-
-// 2^x for any x a product's exponents give.
-__device__ __forceinline__ double pow2(int x) {
-    if (x > -1023 && x < 1024) return __longlong_as_double((long long)(x + 1023) << 52);
-    return ldexp(1.0, x);
-}
 
 // An integer |d| <= 256 as FP32 (exact; its upper 16 bits are the BF16 value).
 __device__ __forceinline__ uint32_t small_float(int d) {
@@ -191,23 +179,39 @@ __device__ __forceinline__ void oz_products(uint32_t acc, uint32_t cls, uint32_t
 }
 
 // ---- pivot block -------------------------------------------------------------
-// P^-1 of the pivot block by a Gauss-Jordan sweep (SPD: no pivoting) over its lower
-// triangle in registers: thread (ty, tx) of 16 x 16 holds elements (ty + 16 u, tx + 16 v),
-// v <= u.  Step k publishes the vector r (row k left of the diagonal, column k below
-// it) and 1 / d; then P_ij -= (s_i r_i) (r_j / d).  One CTA per matrix: the 64 steps
-// are a serial chain of ten FMAs per thread, FP64-ALU bound.  Writes P^-1 back into
-// M[p, p] (the panel kernel does not read that block), and its slices and exponents.
+// P^-1 of the pivot block, one CTA per matrix.
+//  * X by a Gauss-Jordan sweep (SPD: no pivoting) over the lower triangle in registers:
+//    thread (ty, tx) of 16 x 16 holds elements (ty + 16 u, tx + 16 v), v <= u.  Step k
+//    publishes the vector r (row k left of the diagonal, column k below it) and 1 / d;
+//    then P_ij -= (s_i r_i) (r_j / d).  A serial chain of 64 steps of ten FMAs per thread,
+//    FP64-ALU bound.
+//  * The 64 roundings of every element were the largest error of the whole elimination
+//    (the products are exact to 2^-54), so X is corrected once: R = I - P X from exact
+//    57-bit fixed-point sums, X += X R in FP32 (R is of the order of FP64 rounding).  That
+//    leaves X at its own rounding.  Measured, coupled operator against an extended-precision
+//    reference, seven meshes (six bisected into 139 to 600 uneven subdomains): 2.3e-16 ..
+//    3.8e-16; without the correction 2.9e-16 .. 4.5e-16, with 32-wide pivot blocks in plain
+//    FP64 2.5e-16 .. 4.0e-16.  It costs 49 of the kernel's 173 us per block (40 matrices).
+// Writes P^-1 back into M[p, p] (the panel kernel does not read that block), and its slices
+// and exponents.
 constexpr int kOzPivThreads = 256;
-__global__ void __launch_bounds__(kOzPivThreads) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
+constexpr int kPs = kOzK + 1;   // row stride in shared memory
+constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2));
+__global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
                                                             int k0, uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
                                                             int32_t* __restrict__ status) {
     const MatDesc md = mats[blockIdx.x];
     if (k0 >= md.nr) return;
     const int nb = min(kOzK, md.nr - k0);
-    __shared__ double Q[kOzK][kOzK + 1];
+    extern __shared__ __align__(16) unsigned char smem[];
+    double* Q = reinterpret_cast<double*>(smem);         // [kOzK][kPs] the block in full; then R in FP32
+    int2* Pi = reinterpret_cast<int2*>(Q + kOzK * kPs);  // [kOzK][kPs] P, row i in units of 2^(rp_i - 57)
+    int2* Xi = Pi + kOzK * kPs;                          // [kOzK][kPs] X, column j in units of 2^(cx_j - 57)
     __shared__ double r[2][kOzK], t[kOzK], sinv[2];   // by step parity: a step's readers meet the next writers two barriers on
+    __shared__ int rp[kOzK], cx[kOzK];
     double* A = M + md.moff + (int64_t)k0 * md.ld + k0;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int ri = tid >> 2, rq = tid & 3;   // (row, quarter of its 64 columns) for row maxima and slices
     double a[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -216,6 +220,33 @@ __global__ void __launch_bounds__(kOzPivThreads) k_oz_pivot(const MatDesc* __res
             const int i = ty + 16 * u, j = tx + 16 * v;
             a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : (i == j ? 1.0 : 0.0);
         }
+    // the lower triangle in registers -> the full symmetric block in Q (zero outside nb)
+    auto spread = [&]() {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v;
+                if (j > i) continue;
+                const double x = i < nb ? a[u][v] : 0.0;
+                Q[i * kPs + j] = x;
+                Q[j * kPs + i] = x;
+            }
+        __syncthreads();
+    };
+    auto row_exp = [&]() {   // exponent of the largest element of row ri (all four lanes of the row)
+        int mx = 0;
+        for (int k = 0; k < 16; ++k) mx = max(mx, __double2hiint(Q[ri * kPs + 16 * rq + k]) & 0x7fffffff);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        return exp_of_hi(mx);
+    };
+    spread();
+    {
+        const int e = row_exp();
+        rp[ri] = e;
+        for (int k = 0; k < 16; ++k) Pi[ri * kPs + 16 * rq + k] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
+    }
     for (int k = 0; k < nb; ++k) {
         double* rk = r[k & 1];
         const int uk = k >> 4, kk = k & 15;
@@ -276,38 +307,80 @@ __global__ void __launch_bounds__(kOzPivThreads) k_oz_pivot(const MatDesc* __res
                 }
         }
     }
-    // full symmetric P^-1 (zero outside nb)
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v <= u; ++v) {
-            const int i = ty + 16 * u, j = tx + 16 * v;
-            if (j > i) continue;
-            const double x = i < nb ? a[u][v] : 0.0;
-            Q[i][j] = x;
-            Q[j][i] = x;
-        }
+    __syncthreads();   // Pi was read from Q by every thread before the first step's barriers
+    spread();
+    {
+        const int e = row_exp();   // X is symmetric: also its column exponent
+        cx[ri] = e;
+        for (int k = 0; k < 16; ++k) Xi[(16 * rq + k) * kPs + ri] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
+    }
     __syncthreads();
+    // R = I - P X: 64 products per element fit the accumulators; |R| >= 2^-20 (or exponents out of
+    // range) means that the sweep itself went wrong: X stays as it is
+    {
+        float* R = reinterpret_cast<float*>(Q);
+        long long hh[4][4] = {}, xx[4][4] = {};
+        for (int k = 0; k < nb; ++k) {
+            int2 p[4], x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                p[u] = Pi[(ty + 16 * u) * kPs + k];
+                x[u] = Xi[k * kPs + tx + 16 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) mac(hh[u][v], xx[u][v], p[u].x, p[u].y, x[v].x, x[v].y);
+        }
+        bool big = false;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v, sh = 2 * kBits - kLow - rp[i] - cx[j];   // 1 in the sums' units
+                __int128 d = -(((__int128)hh[u][v] << kLow) + xx[u][v]);
+                float f = 0.0f;
+                if (i < nb && j < nb) {
+                    if (sh < 24 || sh > 120) {
+                        big = true;
+                    } else {
+                        if (i == j) d += (__int128)1 << sh;
+                        const __int128 lim = (__int128)1 << (sh - 20);
+                        if (d > lim || d < -lim) big = true;
+                        else f = (float)(long long)(d >> (sh > 80 ? sh - 80 : 0)) * exp2f(-(float)(sh > 80 ? 80 : sh));
+                    }
+                }
+                R[i * kPs + j] = f;   // (every thread is done with Q)
+            }
+        if (!__syncthreads_or(big)) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    const int i = ty + 16 * u, j = tx + 16 * v;
+                    float s = 0.0f;
+                    for (int k = 0; k < nb; ++k) s = fmaf((float)Xi[k * kPs + i].x, R[k * kPs + j], s);
+                    if (i < nb && j <= i) a[u][v] += (double)s * pow2(cx[i] - (kBits - kLow));
+                }
+        }
+        __syncthreads();
+    }
+    spread();
     for (int p = tid; p < kOzK * kOzK; p += kOzPivThreads) {
         const int i = p >> 6, j = p & 63;
-        if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i][j];
+        if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i * kPs + j];
     }
-    // slices: thread (row i, quarter q of the 64 columns)
-    const int i = tid >> 2, q = tid & 3;
-    int mx = 0;
-    for (int k = 0; k < 16; ++k) mx = max(mx, __double2hiint(Q[i][16 * q + k]) & 0x7fffffff);
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const int e = exp_of_hi(mx);
-    if (q == 0) ep[(int64_t)blockIdx.x * kOzK + i] = e;
+    // slices
+    const int e = row_exp();
+    if (rq == 0) ep[(int64_t)blockIdx.x * kOzK + ri] = e;
     unsigned char* out = reinterpret_cast<unsigned char*>(Ps) + (int64_t)blockIdx.x * kOzPBlock;
     for (int g = 0; g < 2; ++g) {
-        const int k = 16 * q + 8 * g;
+        const int k = 16 * rq + 8 * g;
         double v[8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = Q[i][k + c];
+        for (int c = 0; c < 8; ++c) v[c] = Q[ri * kPs + k + c];
         cut8(v, e, [&](int p, uint4 w) {
-            *reinterpret_cast<uint4*>(out + p * kOzPPiece + tc::kmajor_off(i, k, kOzK)) = w;
+            *reinterpret_cast<uint4*>(out + p * kOzPPiece + tc::kmajor_off(ri, k, kOzK)) = w;
         });
     }
 }
@@ -683,8 +756,9 @@ int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, un
     int32_t* ec = reinterpret_cast<int32_t*>(ws + L.ec);
     cudaError_t e = cudaFuncSetAttribute(k_oz_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzPanSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_oz_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_oz_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzPivSmem);
     if (e != cudaSuccess) return (int)e;
-    k_oz_pivot<<<(unsigned)nm, kOzPivThreads, 0, S(stream)>>>(mats, M, k0, Ps, ep, status);
+    k_oz_pivot<<<(unsigned)nm, kOzPivThreads, kOzPivSmem, S(stream)>>>(mats, M, k0, Ps, ep, status);
     k_oz_panel<<<dim3((unsigned)nrb, (unsigned)nm), kOzPanThreads, kOzPanSmem, S(stream)>>>(mats, M, k0, nrb, Ps, ep, Bs,
                                                                                             eb, Cs, ec, nmax, err);
     unsigned runs = 0;
