@@ -127,7 +127,7 @@ struct Prof {
 
 // algorithmic bytes of one full GEMV launch of `mode` at precision `prec`
 double mb(const dd_handle* h, int mode, int prec) {
-    if (prec != DD_MIXED) return h->mode_bytes[mode];
+    if (prec != DD_MIXED) return fx_active(h, mode) ? 2.0 * h->mode_bytes_sym[mode] : h->mode_bytes[mode];
     if (h->prm.sym_fp32 && h->sym_ok && sym_active(h, mode) && h->mode_bytes_sym[mode] > 0.0) return h->mode_bytes_sym[mode];
     return h->mode_bytes32[mode];
 }
@@ -229,6 +229,15 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.M64, (size_t)h->dense_elems);
     L.take(d.M32, (size_t)h->dense_elems);
     L.take(d.Msym, (size_t)h->sym_elems);
+    L.take(d.Mfx, 256 * (size_t)h->fx_blocks);
+    L.take(d.fx_dir, h->fx_dir.size());
+    L.take(d.fx_moff, h->fx_moff.size());
+    L.take(d.fx_exps, (size_t)h->sub_ptr[h->n_sub_real]);
+    for (int m = 0; m < GEMV_NMODES; ++m)
+        if (fx_active(h, m)) {
+            L.take(d.fx_rng[m], h->fx_rng[m].size());
+            L.take(d.fx_tl[m], h->fx_tl[m].size());
+        }
     L.take(d.symd, (size_t)h->n_sub);
     L.take(d.sym_dir, h->sym_dir.size());
     L.take(d.Mtc, (size_t)h->tc_elems);
@@ -1017,6 +1026,8 @@ int dd_bind_workspace(dd_handle* h, void* dev, size_t bytes, void* stream) {
     CK(h, upload(h->d.col_dof, h->col_dof, s), "upload");
     CK(h, upload(h->d.Tval, h->Tval, s), "upload");
     CK(h, upload(h->d.symd, h->sym, s), "upload");
+    CK(h, upload(h->d.fx_dir, h->fx_dir, s), "upload");
+    CK(h, upload(h->d.fx_moff, h->fx_moff, s), "upload");
     if (!h->sym_dir.empty()) CK(h, upload(h->d.sym_dir, h->sym_dir, s), "upload");
     for (int k = 0; k < kTcKinds; ++k)
         if (!h->tcd[k].empty()) CK(h, upload(h->d.tcd[k], h->tcd[k], s), "upload");
@@ -1027,6 +1038,8 @@ int dd_bind_workspace(dd_handle* h, void* dev, size_t bytes, void* stream) {
     for (int m = 0; m < GEMV_NMODES; ++m) {
         if (!h->sym_rng[m].empty()) CK(h, upload(h->d.sym_rng[m], h->sym_rng[m], s), "upload");
         if (!h->sym_tl[m].empty()) CK(h, upload(h->d.sym_tl[m], h->sym_tl[m], s), "upload");
+        if (!h->fx_rng[m].empty()) CK(h, upload(h->d.fx_rng[m], h->fx_rng[m], s), "upload");
+        if (!h->fx_tl[m].empty()) CK(h, upload(h->d.fx_tl[m], h->fx_tl[m], s), "upload");
     }
     CK(h, upload(h->d.Sval, h->Sval, s), "upload");
     for (int p = 0; p < 2; ++p)
@@ -1113,8 +1126,9 @@ int dd_factor(dd_handle* h, double dt, void* stream) {
         CK(h, launch_corner_diag(h, s), "coarse diagonal");
     }
     {
-        Prof P(h, ST_FACTOR, s, 1);
+        Prof P(h, ST_FACTOR, s, 3);
         CK(h, launch_sym_pack(h, s), "packed symmetric tiles");
+        CK(h, launch_fx_pack(h, s), "fixed-point tiles");
         CK(h, launch_tc_pack(h, s), "tensor-core panels");
     }
     int32_t st = 0;
@@ -1230,7 +1244,10 @@ int advance(dd_handle* h, const double* u_n, const double* u_nm1, double* u_np1,
     }
     if (h->prm.precision == DD_FP64) {
         status = dd_solve(h, DD_FP64, h->prm.tol, h->prm.warm_start != 0, &iters, &resid, s);
-        if (status != DD_OK && status != DD_ERR_NO_CONVERGENCE) return status;
+        if (status != DD_OK && status != DD_ERR_NO_CONVERGENCE) {   // a wait that gave up leaves NaN behind
+            if (status != DD_ERR_CUDA && wait_err_set(h, s)) return report_timeout(h, s);
+            return status;
+        }
         Prof P(h, ST_VEC, s, 1);
         CK(h, launch_writeback(h, u_n, u_nm1, nullptr, nullptr, 1, u_np1, s), "writeback");
     } else {
@@ -1991,7 +2008,7 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
                     }
                 }
                 h->prm.sym_fp32 = 0;   // the dense tiles below time the dense kernel
-                if (h->tasks[p][m].empty()) {
+                if (h->tasks[p][m].empty() || (p == 0 && fx_active(h, m))) {   // (fixed point: nothing to choose)
                     found[{p, m}] = h->tile[p][m];
                     h->prm.sym_fp32 = sym_saved ? 1 : 0;
                     continue;
@@ -2075,6 +2092,7 @@ int dd_get_gemv_bytes(const dd_handle* h, int32_t kind, int32_t precision, doubl
     double str = alg;
     if (precision == DD_MIXED && h->prm.sym_fp32 && h->sym_ok && sym_active(h, kind) && h->mode_tile_bytes_sym[kind] > 0.0)
         str = h->mode_tile_bytes_sym[kind];
+    if (precision == DD_FP64 && fx_active(h, kind)) str = h->fx_bytes[kind];
     if (algorithmic) *algorithmic = alg;
     if (streamed) *streamed = str;
     return DD_OK;

@@ -321,6 +321,12 @@ struct DevPtrs {
     int32_t* sym_rng[GEMV_NMODES] = {};   // [n_sub * kSymCLMax * kSymRng] (list offset, tile count, end tile row,
                                           // subdomain, ensemble members served) per CTA
     uint32_t* sym_tl[GEMV_NMODES] = {};   // tiles of each packed mode, every subdomain in row order
+    int32_t* Mfx = nullptr;          // packed tiles in fixed point, blocks of 16 x 8 elements of two words
+    int32_t* fx_dir = nullptr;       // [tiles * 4], first block of every stored subdomain, tile lists
+    int64_t* fx_moff = nullptr;
+    uint32_t* fx_tl[GEMV_NMODES] = {};
+    int32_t* fx_exps = nullptr;      // row exponents of the stored subdomains, per slot
+    int32_t* fx_rng[GEMV_NMODES] = {};    // as sym_rng, for the fixed-point form
     double* K64 = nullptr;           // K~cc^-1, n_corner x ldc
     float* K32 = nullptr;
     double* Pinv = nullptr;          // [n_sub+1][NB*NB] pivot-block inverses (DD_FACTOR_FP64)
@@ -496,6 +502,15 @@ struct dd_handle {
     int32_t sym_max_tiles = 0;                     // largest tile count of one subdomain
     int64_t sym_ntiles = 0;                        // stored tiles in all (entries of sym_dir / 4)
     bool sym_ok = false;                           // the packed GEMV's shared memory fits one CTA
+    bool fx_ok = false;                            // the same for the fixed-point FP64 form (fxgemv.cu)
+    std::vector<int32_t> fx_dir;                   // its directory (as sym_dir, offsets in blocks), the first block of
+    std::vector<int64_t> fx_moff;                  // every stored subdomain, blocks in all, tile lists (order of sym_tl) and
+    int64_t fx_blocks = 0;                         // the bytes one launch streams
+    std::vector<uint32_t> fx_tl[GEMV_NMODES];
+    double fx_bytes[GEMV_NMODES] = {};
+    std::vector<int32_t> fx_rng[GEMV_NMODES];      // its CTA ranges (layout of sym_rng), CTAs per subdomain and
+    int32_t fx_cl[GEMV_NMODES] = {};               // subdomains kept in L2
+    int32_t fx_keep[GEMV_NMODES] = {};
     size_t task_cap[GEMV_NMODES] = {};             // device capacity: tasks at the smallest row count
     TileCfg tile[2][GEMV_NMODES];                  // lanes per row and rows per CTA, per precision and mode
     bool tuned = false;
@@ -624,7 +639,14 @@ int launch_faraday(const dd_handle* h, const double* e_np1, const double* e_n, d
 // symgemv.cu: packed symmetric FP32 storage and its GEMV
 void build_sym(dd_handle* h);
 void sym_ranges(dd_handle* h, int mode, int cl);
+void sym_split(const dd_handle* h, int mode, int cl, int per, std::vector<int32_t>& rng, int32_t* longest_list);
+int sym_span(const dd_handle* h, int mode);
 int launch_sym_pack(const dd_handle* h, void* stream);
+// fxgemv.cu
+void build_fx(dd_handle* h);
+bool fx_active(const dd_handle* h, int mode);
+int launch_fx_pack(const dd_handle* h, void* stream);
+int launch_fxgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);
 int launch_symgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);
 size_t sym_smem_bytes(const dd_handle* h);
 // Packed kinds in use: the recovery reads the packed tiles only for an ensemble (its I x [Gamma|c]

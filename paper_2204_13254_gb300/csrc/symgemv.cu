@@ -48,6 +48,7 @@
 #include <algorithm>
 
 #include "dd_internal.h"
+#include "symtile.cuh"
 #include "xsrc.cuh"
 
 namespace cg = cooperative_groups;
@@ -55,101 +56,8 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kT = 128;             // threads per CTA: 8 row groups x 16 column quads of a tile
-constexpr uint32_t kTileBytes = kSymTile * sizeof(float);
-constexpr unsigned kWaitLimit = 1u << 20;   // polls of one mbarrier wait before it gives up (well under a second)
 
 inline cudaStream_t S(void* s) { return (cudaStream_t)s; }
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-// L2 policies for the tile copies: evict_last keeps a subset of the operator
-// resident in L2 across the launches of one Krylov solve, evict_first streams
-// the rest past it.
-__device__ __forceinline__ uint64_t l2_policy(bool keep) {
-    uint64_t pol;
-    if (keep) asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-// One tile (bytes: a multiple of 16, at most kTileBytes) global -> shared,
-// completing on `bar` (which expects the bytes).
-__device__ __forceinline__ void load_tile(float* dst, const float* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for phase `parity` of `bar`; false if it gave up.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned limit = kWaitLimit) {
-    for (unsigned k = 0; k < limit; ++k)
-        if (mbar_test(bar, parity)) return true;
-    return false;
-}
-
-// Failure-path test (PcgScalars::wait_first > 0): the CTA's first wait polls
-// `never`, an mbarrier no thread or copy ever completes, wait_first times and
-// gives up, exercising the give-up / drain / report path with every copy issued.
-__device__ __forceinline__ bool first_wait_test(const XSrc& xs, uint64_t* never) {
-    const int n = xs.sc ? xs.sc->wait_first : 0;
-    return n > 0 ? mbar_wait(never, 0u, (unsigned)n) : true;
-}
-
-// Shape of a listed tile: rows, padded width (floats per row of a rectangle),
-// diagonal (padded triangle), bytes.
-struct TileShape {
-    int h, wp;
-    bool diag, full;
-    uint32_t bytes;
-};
-
-// Shape of the tile of list entry word e0, from the subdomain's descriptor.
-__device__ __forceinline__ TileShape tile_shape(const SymDesc& sd, uint32_t e) {
-    const int a = (int)(e >> 16), b = (int)((e >> 3) & 0x1fff);
-    const bool diag = (e & 4) != 0;
-    TileShape t;
-    t.h = sym_h(sd, a);
-    const int w = sym_h(sd, b);
-    t.wp = (w + 3) & ~3;
-    t.diag = diag;
-    t.full = !diag && t.h == kSymT && w == kSymT;
-    t.bytes = 4u * (uint32_t)sym_tile_floats(t.h, w, diag);
-    return t;
-}
-
-// First word of list entry k (the tile's rows, columns and roles): from the
-// CTA's copy in shared memory (LSM) or, read-only, from the mode's list in
-// global memory.
-template <bool LSM>
-__device__ __forceinline__ uint32_t tl_word(const uint32_t* tl, int k) {
-    return LSM ? tl[kTlW * k] : __ldg(tl + kTlW * k);
-}
-
-// Issue the bulk copy of list entry k.
-template <bool LSM = false>
-__device__ __forceinline__ void issue_tile(const uint32_t* tl, int k, const SymDesc& sd, const float* tiles, float* dst,
-                                           uint64_t* bar, uint64_t pol) {
-    const uint32_t e0 = tl_word<LSM>(tl, k), e1 = LSM ? tl[kTlW * k + 1] : __ldg(tl + kTlW * k + 1);
-    load_tile(dst, tiles + e1, tile_shape(sd, e0).bytes, bar, pol);
-}
 
 // Row `row` (0..63), column chunk cq (0..15) of a tile in a ring slot: the four
 // floats as a float4, zero outside the stored tile.
@@ -188,9 +96,6 @@ __host__ __device__ inline size_t sym_smem_ps(int span, int st, int ng) {
 
 // tile list entry: a << 16 | b << 3 | flags (a, b < 8192), then the tile's float offset
 __host__ __device__ __forceinline__ uint32_t tile_entry(int a, int b, int f) { return ((uint32_t)a << 16) | ((uint32_t)b << 3) | f; }
-
-// First padded position a mode touches (the I run only when I is in the mask).
-__host__ __device__ inline int mask_lo(const SymDesc& sd, int mask) { return (mask & 1) ? 0 : kSymT * sd.tI; }
 
 // x over the column groups of tile rows < a_end (the only ones the CTA reads),
 // eight entries per thread per pass: their index loads, then their value loads;
@@ -432,10 +337,6 @@ __global__ void __launch_bounds__(kT) k_symgemv(const SymDesc* __restrict__ desc
 
     for (int q = 0; q < nmem; ++q)
         cluster_store(cluster, ysh + q * span_max, descs[sub + q * n_real], rmask, r_lo, p_lo, np, cl, go, tid, kT);
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Bounded wait that also gives up once another role has aborted.
@@ -1083,19 +984,13 @@ static void sym_queue(dd_handle* h, int mode, int ng, int rmask, int cmask) {
 // of the subdomain's total; stored as (first entry in the mode's tile list, tile
 // count, end tile row, subdomain, members served).  Ensemble copies of a
 // subdomain follow each other (they stream the same tiles, which L2 then serves).
-void sym_ranges(dd_handle* h, int mode, int cl) {
+// `per`: ensemble copies served by one CTA.
+void sym_split(const dd_handle* h, int mode, int cl, int per, std::vector<int32_t>& rng, int32_t* longest_list) {
     int rmask, cmask;
-    h->sym_rng[mode].clear();
-    h->sym_cl[mode] = cl;
-    h->sym_nl[mode] = 0;
-    h->sym_grid[mode] = 0;
+    rng.clear();
+    *longest_list = 0;
     if (!sym_masks(mode, &rmask, &cmask)) return;
-    if (h->sym_ws[mode] == 5) {
-        sym_queue(h, mode, cl, rmask, cmask);
-        return;
-    }
     const int R = std::max(1, h->members);
-    const int per = sym_members_per_cta(h, mode);   // ensemble copies served by one CTA
     for (int s0 = 0; s0 < h->n_sub_real; ++s0) {
         const SymDesc& sd = h->sym[s0];
         const int nt = sd.nt;
@@ -1124,19 +1019,18 @@ void sym_ranges(dd_handle* h, int mode, int cl) {
                 }
                 int64_t n = 0;
                 for (int q = begin; q < a; ++q) n += cnt_row[q];
-                h->sym_rng[mode].push_back((int32_t)first);
-                h->sym_rng[mode].push_back((int32_t)n);
-                h->sym_rng[mode].push_back(n ? a : 0);
-                h->sym_rng[mode].push_back(sub);
-                h->sym_rng[mode].push_back(nmem);
+                rng.push_back((int32_t)first);
+                rng.push_back((int32_t)n);
+                rng.push_back(n ? a : 0);
+                rng.push_back(sub);
+                rng.push_back(nmem);
                 first += n;
-                h->sym_nl[mode] = std::max<int32_t>(h->sym_nl[mode], (int32_t)n);
+                *longest_list = std::max<int32_t>(*longest_list, (int32_t)n);
             }
         }
     }
     // Largest clusters first (longest CTA tile list, stable): when the grid is larger than
     // one wave, the short clusters fill the slots the long ones leave at the end.
-    std::vector<int32_t>& rng = h->sym_rng[mode];
     const size_t per_cluster = (size_t)cl * kSymRng, ncl = rng.size() / per_cluster;
     std::vector<int32_t> longest(ncl, 0);
     std::vector<size_t> order(ncl);
@@ -1149,7 +1043,21 @@ void sym_ranges(dd_handle* h, int mode, int cl) {
     sorted.reserve(rng.size());
     for (size_t q : order) sorted.insert(sorted.end(), rng.begin() + q * per_cluster, rng.begin() + (q + 1) * per_cluster);
     rng.swap(sorted);
-    h->sym_grid[mode] = (int32_t)(rng.size() / kSymRng);
+}
+
+void sym_ranges(dd_handle* h, int mode, int cl) {
+    int rmask, cmask;
+    h->sym_rng[mode].clear();
+    h->sym_cl[mode] = cl;
+    h->sym_nl[mode] = 0;
+    h->sym_grid[mode] = 0;
+    if (!sym_masks(mode, &rmask, &cmask)) return;
+    if (h->sym_ws[mode] == 5) {
+        sym_queue(h, mode, cl, rmask, cmask);
+        return;
+    }
+    sym_split(h, mode, cl, sym_members_per_cta(h, mode), h->sym_rng[mode], &h->sym_nl[mode]);
+    h->sym_grid[mode] = (int32_t)(h->sym_rng[mode].size() / kSymRng);
 }
 
 int launch_sym_pack(const dd_handle* h, void* stream) {

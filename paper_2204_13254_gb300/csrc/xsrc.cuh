@@ -115,42 +115,70 @@ __device__ __forceinline__ float xsrc_value_f(const XSrc& xs, int64_t slot, int6
 // null), 0 when a is null.  Lets a caller issue the index loads of several
 // slots, then their value loads, without a dependent chain per slot; the
 // values equal xsrc_value_f's bit for bit (the sign is a multiplication by +-1).
-struct XRef {
-    const float* a;
-    const float* b;
+template <typename T>
+struct XRefT {
+    const T* a;
+    const T* b;
     int64_t i;
-    float sgn;
+    T sgn;
+};
+using XRef = XRefT<float>;
+
+// The three vectors of an XSrc at precision T.
+template <typename T>
+struct XVecs;
+template <>
+struct XVecs<float> {
+    const float *v, *v2, *v3;
+    __device__ __forceinline__ explicit XVecs(const XSrc& xs) : v(xs.vf), v2(xs.v2f), v3(xs.v3f) {}
+};
+template <>
+struct XVecs<double> {
+    const double *v, *v2, *v3;
+    __device__ __forceinline__ explicit XVecs(const XSrc& xs) : v(xs.v), v2(xs.v2), v3(xs.v3) {}
 };
 
-__device__ __forceinline__ XRef xsrc_ref_f(const XSrc& xs, int m, int c, int64_t slot, int64_t j) {
-    const XRef none{nullptr, nullptr, 0, 1.0f};
+template <typename T>
+__device__ __forceinline__ XRefT<T> xsrc_ref(const XSrc& xs, int m, int c, int64_t slot, int64_t j) {
+    using R = XRefT<T>;
+    const XVecs<T> q(xs);
+    const R none{nullptr, nullptr, 0, (T)1};
     const int mi = (m > 0 ? m : -m) - 1;
-    const float ms = m > 0 ? 1.0f : -1.0f;
+    const T ms = m > 0 ? (T)1 : (T)-1;
     switch (xs.kind) {
-        case X_FLAT: return {xs.vf, nullptr, slot, 1.0f};
-        case X_LAMBDA: return m != 0 ? XRef{xs.vf, nullptr, mi, ms} : none;
-        case X_PCG: return m != 0 ? XRef{xs.vf, xs.v2f, mi, ms} : none;
-        case X_CORNER: return c >= 0 ? XRef{xs.vf, nullptr, c, 1.0f} : none;
+        case X_FLAT: return {q.v, nullptr, slot, (T)1};
+        case X_LAMBDA: return m != 0 ? R{q.v, nullptr, mi, ms} : none;
+        case X_PCG: return m != 0 ? R{q.v, q.v2, mi, ms} : none;
+        case X_CORNER: return c >= 0 ? R{q.v, nullptr, c, (T)1} : none;
         case X_RECOVER:
-            if (m != 0) return {xs.vf, nullptr, mi, -ms};
-            return c >= 0 ? XRef{xs.v2f, nullptr, c, 1.0f} : none;
+            if (m != 0) return {q.v, nullptr, mi, -ms};
+            return c >= 0 ? R{q.v2, nullptr, c, (T)1} : none;
         case X_PCG_CV:
-            if (m != 0) return {xs.vf, xs.v2f, mi, ms};
-            return c >= 0 ? XRef{xs.v3f, nullptr, c, -1.0f} : none;
+            if (m != 0) return {q.v, q.v2, mi, ms};
+            return c >= 0 ? R{q.v3, nullptr, c, (T)-1} : none;
         case X_LAMBDA_CV:
-            if (m != 0) return {xs.vf, nullptr, mi, ms};
-            return c >= 0 ? XRef{xs.v3f, nullptr, c, -1.0f} : none;
+            if (m != 0) return {q.v, nullptr, mi, ms};
+            return c >= 0 ? R{q.v3, nullptr, c, (T)-1} : none;
         case X_SIDE_CP:
-            if (m != 0) return m > 0 ? XRef{xs.vf, nullptr, mi, 1.0f} : XRef{xs.v2f, nullptr, mi, 1.0f};
-            return c >= 0 ? XRef{xs.v3f, nullptr, c, 1.0f} : none;
-        default: return {xs.vf, nullptr, j, 1.0f};
+            if (m != 0) return m > 0 ? R{q.v, nullptr, mi, (T)1} : R{q.v2, nullptr, mi, (T)1};
+            return c >= 0 ? R{q.v3, nullptr, c, (T)1} : none;
+        default: return {q.v, nullptr, j, (T)1};
     }
+}
+
+__device__ __forceinline__ XRef xsrc_ref_f(const XSrc& xs, int m, int c, int64_t slot, int64_t j) {
+    return xsrc_ref<float>(xs, m, c, slot, j);
 }
 
 __device__ __forceinline__ float xref_value(const XRef& r, float beta) {
     if (!r.a) return 0.0f;
     const float v = r.b ? fmaf(beta, r.b[r.i], r.a[r.i]) : r.a[r.i];
     return r.sgn * v;
+}
+__device__ __forceinline__ double xref_value(const XRefT<double>& r, double beta) {
+    if (!r.a) return 0.0;
+    const double v = r.b ? r.a[r.i] + beta * r.b[r.i] : r.a[r.i];
+    return r.sgn < 0.0 ? -v : v;
 }
 
 }  // namespace
