@@ -124,7 +124,12 @@ typedef struct {
  *            Gram-Schmidt applied twice, Givens rotations; warm start from
  *            the previous solve's [lambda; x_c] (warm_start 2: extrapolated).
  *            DD_FP64 or DD_MIXED (FP32 Krylov vectors inside the FP64
- *            refinement).  K~cc^-1 is not used by this solver.
+ *            refinement).  K~cc^-1 is not used by this solver.  DD_MIXED with
+ *            sym_fp32, one problem: when every subdomain's [Gamma | c] block
+ *            and Krylov vectors fit the shared memory of a CTA of its own, all
+ *            CTAs on the device at once, each solve is one cooperative kernel
+ *            (the packed launch of the coupled kind, dd_set_sym_config, is then
+ *            not used by it, nor is chunk).
  * restart    GMRES restart length m, 1..DD_MAX_RESTART (the paper: 20).
  * scheme     DD_SCHEME_DP1 (default) or DD_SCHEME_DP2.  DP2 (Sec. III-B, read for
  *            the edge-only step system A = T + dt^2/4 S): every local matrix

@@ -256,6 +256,7 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     // slices and exponents of one pivot block of the tensor-core elimination (local or coarse)
     L.take(d.oz, std::max(oz_bytes(std::max(1, h->n_sub_real), h->max_ns), oz_bytes(1, (int)nc)));
     L.take(d.dinv, nm);
+    L.take(d.rpart, (size_t)(kMaxRestart + 4) * (size_t)h->n_sub);
     for (int k = 0; k < 3; ++k) L.take(d.e[k], nd);
     for (int k = 0; k < 3; ++k) L.take(d.mu[k], nd);
     L.take(d.lam_adj, nm);
@@ -565,6 +566,20 @@ UView uview(const dd_handle* h, int prec) {
     return U;
 }
 
+// Status and final relative residual of a finished solve from its control words.
+int gmres_outcome(dd_handle* h, const GmresScalars& c, double* res_out) {
+    *res_out = c.bnorm > 0 ? c.resid / c.bnorm : 0.0;
+    if (c.status != DD_OK) {
+        h->err = "non-finite GMRES residual";
+        return c.status;
+    }
+    if (!c.converged) {
+        h->err = "coupled GMRES did not converge";
+        return DD_ERR_NO_CONVERGENCE;
+    }
+    return DD_OK;
+}
+
 int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double* res_out, cudaStream_t s,
                 int depth, int adaptive) {
     const size_t nm = h->mult_dof.size(), nc = h->corner_dof.size();
@@ -617,6 +632,27 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
         CK(h, launch_gm_normalize(h, U, zuf, st), "gmres normalize");
         return DD_OK;
     };
+    // the whole solve in one cooperative kernel where every subdomain's operator finds room on chip
+    const int resident = prec == DD_MIXED && h->prm.sym_fp32 ? res_warps(h, h->prm.restart) : 0;
+    if (resident) {
+        {
+            Prof P(h, ST_VEC, s, 2);
+            CK(h, launch_gm_init(h, tol, h->prm.max_it, h->prm.restart, h->capturing ? adaptive : 0, 0ull, s), "gmres init");
+            CK(h, launch_gm_resident(h, U, resident, use_warm ? 1 : 0, h->prm.restart, s), "resident gmres");
+        }
+        h->lam_valid = true;
+        if (h->capturing) {
+            Prof P(h, ST_VEC, s, 1);
+            CK(h, launch_solve_end(h, s), "solve end");
+            h->g_kernels_iter = h->g_kernels_cycle = 0;
+            return DD_OK;
+        }
+        GmresScalars c;
+        CK(h, read_gm(h, &c, s), "gmres scalars");
+        h->work[ST_SCHUR] += c.it;
+        *it_out = c.it;
+        return gmres_outcome(h, c, res_out);
+    }
     if (h->capturing) {
         cudaGraphConditionalHandle ho;
         int rc = create_handle(h, s, &ho);
@@ -707,16 +743,7 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
     }
     h->lam_valid = true;
     *it_out = c.it;
-    *res_out = c.bnorm > 0 ? c.resid / c.bnorm : 0.0;
-    if (c.status != DD_OK) {
-        h->err = "non-finite GMRES residual";
-        return c.status;
-    }
-    if (!c.converged) {
-        h->err = "coupled GMRES did not converge";
-        return DD_ERR_NO_CONVERGENCE;
-    }
-    return DD_OK;
+    return gmres_outcome(h, c, res_out);
 }
 
 int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double* res_out, cudaStream_t s,

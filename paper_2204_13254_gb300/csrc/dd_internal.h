@@ -248,6 +248,8 @@ struct GmresScalars {
     int32_t max_it, m, cycles;
     int32_t nh2;        // terms of the second projection k_gm_normalize applies (0 at a cycle start)
     uint32_t counter[4];
+    uint32_t bar;       // arrivals at the grid barriers of the resident solve
+    uint32_t pad;
     double g[kMaxRestart + 1];
     double cs[kMaxRestart], sn[kMaxRestart];
     double y[kMaxRestart];
@@ -332,6 +334,7 @@ struct DevPtrs {
     double* Pinv = nullptr;          // [n_sub+1][NB*NB] pivot-block inverses (DD_FACTOR_FP64)
     unsigned char* oz = nullptr;     // DD_FACTOR_TENSOR: slices and exponents of one pivot block
     double* dinv = nullptr;          // [n_lambda] inverse Jacobi diagonal
+    double* rpart = nullptr;         // partial sums of the resident GMRES (resident.cu)
     // particles (dd_set_beam): state, per-tet geometry and faces
     double* px = nullptr;            // [n_p*3] positions
     double* pv = nullptr;            // [n_p*3] velocities
@@ -502,6 +505,7 @@ struct dd_handle {
     int32_t sym_max_tiles = 0;                     // largest tile count of one subdomain
     int64_t sym_ntiles = 0;                        // stored tiles in all (entries of sym_dir / 4)
     bool sym_ok = false;                           // the packed GEMV's shared memory fits one CTA
+    int32_t res_span = 0, res_floats = 0;          // resident GMRES: padded interface entries and tile floats of a CTA
     bool fx_ok = false;                            // the same for the fixed-point FP64 form (fxgemv.cu)
     std::vector<int32_t> fx_dir;                   // its directory (as sym_dir, offsets in blocks), the first block of
     std::vector<int64_t> fx_moff;                  // every stored subdomain, blocks in all, tile lists (order of sym_tl) and
@@ -642,6 +646,9 @@ void sym_ranges(dd_handle* h, int mode, int cl);
 void sym_split(const dd_handle* h, int mode, int cl, int per, std::vector<int32_t>& rng, int32_t* longest_list);
 int sym_span(const dd_handle* h, int mode);
 int launch_sym_pack(const dd_handle* h, void* stream);
+// resident.cu
+int res_warps(dd_handle* h, int m);
+int launch_gm_resident(const dd_handle* h, const UView& U, int W, int have_q, int m, void* stream);
 // fxgemv.cu
 void build_fx(dd_handle* h);
 bool fx_active(const dd_handle* h, int mode);

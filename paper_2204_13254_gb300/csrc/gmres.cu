@@ -239,6 +239,7 @@ __global__ void k_gm_init(GmresScalars* gs, const PcgScalars* sc, double tol, do
     gs->max_it = max_it;
     gs->m = m;
     gs->cycles = 0;
+    gs->bar = 0u;
     if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 1u);
 }
 
