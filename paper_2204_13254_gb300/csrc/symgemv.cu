@@ -826,6 +826,29 @@ static int ps_ctas_per_sm(const dd_handle* h, int mode, int ng, int st) {
     return nb;
 }
 
+// Launch of a packed mode until dd_autotune or dd_set_sym_config chooses another: as many
+// CTAs per subdomain as keep the grid within 512 (a cluster of 8 at most; 4 for the
+// Krylov operators, whose lists are a quarter as long), a ring of two tiles, the
+// warp-specialised kernel for the Krylov operators and where a few subdomains leave SMs
+// empty, and 64 MB of a Krylov operator that L2 cannot hold kept there.  Measured, untuned
+// mixed step with four / one / two / two CTAs per subdomain and rings of four everywhere
+// against this rule, and tuned: 8 subdomains of 1,512 unknowns 1,094 / 877 / 865 us, 64 of
+// 1,854 (Schur CG) 1,809 / 1,410 / 1,359, 27 of 1,854 1,653 / 1,126 / 1,135, 128 of 604
+// 601 / 573 / 564, 216 of 1,854 2,308 / 2,300 / 2,101; eight CTAs for each of 216
+// subdomains take 3,428 us, one for each of 64 2,195.
+static void sym_default(dd_handle* h, int mode) {
+    const bool krylov = mode == GEMV_SCHUR_G || mode == GEMV_COUPLED;
+    int cl = 1;
+    while (cl < (krylov ? 4 : kSymCLMax) && h->n_sub * cl * 2 <= 512) cl *= 2;
+    h->sym_cl[mode] = cl;
+    h->sym_st[mode] = 2;
+    h->sym_ws[mode] = krylov || h->n_sub < 48 ? 1 : 0;
+    h->sym_keep[mode] = 0;
+    const double streamed = h->mode_tile_bytes_sym[mode];
+    if (krylov && streamed > 100e6)
+        h->sym_keep[mode] = (int32_t)std::min<double>(h->n_sub_real, 64e6 * h->n_sub_real / streamed);
+}
+
 // Host side: tile descriptors, the tile directory, the algorithmic and
 // streamed bytes and the tile list of every packed mode.
 void build_sym(dd_handle* h) {
@@ -921,6 +944,7 @@ void build_sym(dd_handle* h) {
                 }
             off.push_back((int64_t)tl.size() / kTlW);
         }
+        sym_default(h, mode);
         sym_ranges(h, mode, h->sym_cl[mode]);
     }
 }
