@@ -241,6 +241,7 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.symd, (size_t)h->n_sub);
     L.take(d.sym_dir, h->sym_dir.size());
     L.take(d.Mtc, (size_t)h->tc_elems);
+    L.take(d.xtc, h->members > 1 ? tc_x_elems(h) : 0);
     for (int k = 0; k < kTcKinds; ++k) L.take(d.tcd[k], h->tcd[k].size());
     L.take(d.tc_dir, h->tc_dir.size());
     for (int m = 0; m < GEMV_NMODES; ++m) {

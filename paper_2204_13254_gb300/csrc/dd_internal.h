@@ -329,6 +329,7 @@ struct DevPtrs {
     uint32_t* fx_tl[GEMV_NMODES] = {};
     int32_t* fx_exps = nullptr;      // row exponents of the stored subdomains, per slot
     int32_t* fx_rng[GEMV_NMODES] = {};    // as sym_rng, for the fixed-point form
+    uint16_t* xtc = nullptr;         // tensor-core GEMV: x in BF16 pieces by subdomain, member group and column block
     double* K64 = nullptr;           // K~cc^-1, n_corner x ldc
     float* K32 = nullptr;
     double* Pinv = nullptr;          // [n_sub+1][NB*NB] pivot-block inverses (DD_FACTOR_FP64)
@@ -666,6 +667,7 @@ int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, un
 int launch_oz_mirror(const MatDesc* mats, double* M, int nm, int nmax, void* stream);
 // tensor.cu
 void build_tc(dd_handle* h);
+size_t tc_x_elems(const dd_handle* h);
 int launch_tc_pack(const dd_handle* h, void* stream);
 int launch_tc_gemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);
 bool tc_available(const dd_handle* h, int mode);

@@ -172,11 +172,54 @@ __device__ __forceinline__ uint16_t bf16_split(float& v) {
     return __bfloat16_as_ushort(b);
 }
 
-// One CTA: stored subdomain `sub` (blockIdx.x % n_real) and the ensemble copies
-// m0 .. m0 + nmem - 1 (group blockIdx.x / n_real).
+// x of every member of a group over one column block (64 local columns of the stored
+// subdomain), split into three BF16 pieces in the layout of the MMA's B operand (members as
+// N): thread (member n, eight columns).  Staged once per launch, by CTAs enough to fill the
+// chip: two warps of the GEMV's own CTAs gathering it block by block took 16 us a block (three
+// dependent loads each) and set the pace of the whole product.
+constexpr int kTcStageT = kTcN * kTcK / 8;   // 128
+__global__ void __launch_bounds__(kTcStageT) k_tc_stage(const TcDesc* __restrict__ tcd, const SymDesc* __restrict__ descs,
+                                                        int n_real, int members, int qmax, XSrc xs,
+                                                        uint16_t* __restrict__ xt, const int32_t* __restrict__ skip) {
+    if (skip && *skip) return;
+    const int sub = blockIdx.x % n_real, m0 = (blockIdx.x / n_real) * kTcN, q = blockIdx.y;
+    const TcDesc td = tcd[sub];
+    if (q >= td.Q) return;
+    const float beta = (xs.kind == X_PCG || xs.kind == X_PCG_CV) ? (float)xs.sc->beta : 0.0f;
+    const int n = threadIdx.x >> 3, k = 8 * (threadIdx.x & 7), lj = td.c0 + q * kTcK + k;
+    const bool on = m0 + n < members;
+    const int64_t slot = on ? descs[sub + (m0 + n) * n_real].voff + lj : 0;
+    int mm[8], cc[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const bool need = on && lj + u < td.c1;
+        mm[u] = need ? xs.slot_mult[slot + u] : 0;
+        cc[u] = need ? xs.slot_corner[slot + u] : -1;
+    }
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        v[u] = on && lj + u < td.c1 ? xref_value(xsrc_ref_f(xs, mm[u], cc[u], slot + u, lj + u), beta) : 0.0f;
+    unsigned char* out = reinterpret_cast<unsigned char*>(xt) + ((int64_t)blockIdx.x * qmax + q) * kTcXBuf + tc::kmajor_off(n, k, kTcK);
+#pragma unroll
+    for (int piece = 0; piece < 3; ++piece) {
+        uint32_t w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t lo = bf16_split(v[2 * u]), hi = bf16_split(v[2 * u + 1]);
+            w[u] = lo | (hi << 16);
+        }
+        *reinterpret_cast<uint4*>(out + piece * kTcXPiece) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// One CTA: stored subdomain `sub` (blockIdx.x % n_real), the ensemble copies
+// m0 .. m0 + nmem - 1 (group blockIdx.x / n_real) and the row panels [p0, p0 + P) of the
+// rectangle (part blockIdx.y of gridDim.y); an accumulator's products keep their order
+// whatever the parts.
 __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd, const SymDesc* __restrict__ descs,
-                                                 const uint16_t* __restrict__ Mtc, int n_real, int members, XSrc xs,
-                                                 GemvOut go, const int32_t* __restrict__ skip, int32_t* __restrict__ err) {
+                                                 const uint16_t* __restrict__ Mtc, int n_real, int members,
+                                                 const uint16_t* __restrict__ xt, int qmax, GemvOut go, const int32_t* __restrict__ skip, int32_t* __restrict__ err) {
     if (skip && *skip) return;
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* ring = smem;
@@ -184,7 +227,7 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
     uint64_t* bars = reinterpret_cast<uint64_t*>(xbuf + 2 * kTcXBuf);
     uint64_t* full = bars;              // [kTcST] block landed
     uint64_t* empty = bars + kTcST;     // [kTcST] its MMAs done
-    uint64_t* xfull = bars + 2 * kTcST; // [2] x pieces written
+    uint64_t* xfull = bars + 2 * kTcST; // [2] x pieces landed
     uint64_t* xfree = xfull + 2;        // [2] their MMAs done
     uint64_t* done = xfree + 2;         // every MMA done
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
@@ -193,7 +236,9 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
     const int sub = blockIdx.x % n_real, m0 = (blockIdx.x / n_real) * kTcN;
     const int nmem = min(kTcN, members - m0);
     const TcDesc td = tcd[sub];
-    const int P = td.P, Q = td.Q, nblk = P * Q;
+    const int p0 = td.P * (int)blockIdx.y / (int)gridDim.y, P = td.P * ((int)blockIdx.y + 1) / (int)gridDim.y - p0;
+    const int Q = td.Q, nblk = P * Q;
+    if (P == 0) return;
     const uint32_t ncols = P * kTcN <= 32 ? 32 : (P * kTcN <= 64 ? 64 : (P * kTcN <= 128 ? 128 : 256));
     if (tid == 0) {
         for (int i = 0; i < kTcST; ++i) {
@@ -201,7 +246,7 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
             tc_bar_init(&empty[i], 1);
         }
         for (int i = 0; i < 2; ++i) {
-            tc_bar_init(&xfull[i], 64);
+            tc_bar_init(&xfull[i], 1);
             tc_bar_init(&xfree[i], 1);
         }
         tc_bar_init(done, 1);
@@ -214,17 +259,27 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
     const uint16_t* blocks = Mtc + td.off;
-    int issued = 0;   // producer lane
+    const unsigned char* xsrc = reinterpret_cast<const unsigned char*>(xt) + (int64_t)blockIdx.x * qmax * kTcXBuf;
+    int issued = 0, xissued = 0;   // producer lane: panel blocks and x blocks
 
     if (warp == 0) {
-        if (lane == 0) {   // producer: panel blocks in (q, p) order
+        if (lane == 0) {   // producer: panel blocks in (q, p) order, before each column block its x
             for (int b = 0; b < nblk; ++b) {
-                const int slot = b % kTcST;
+                const int slot = b % kTcST, q = b / P;
+                if (b == q * P) {
+                    if (q >= 2 && !tc_wait(&xfree[q & 1], (uint32_t)((q >> 1) - 1) & 1u, &abort_flag)) {
+                        abort_flag = 1;
+                        break;
+                    }
+                    tc_load(xbuf + (q & 1) * kTcXBuf, xsrc + (int64_t)q * kTcXBuf, kTcXBuf, &xfull[q & 1]);
+                    ++xissued;
+                }
                 if (b >= kTcST && !tc_wait(&empty[slot], (uint32_t)((b / kTcST) - 1) & 1u, &abort_flag)) {
                     abort_flag = 1;
                     break;
                 }
-                tc_load(ring + slot * kTcBlockBytes, blocks + (int64_t)b * kTcBlockElems, kTcBlockBytes, &full[slot]);
+                tc_load(ring + slot * kTcBlockBytes, blocks + ((int64_t)q * td.P + p0 + b % P) * kTcBlockElems, kTcBlockBytes,
+                        &full[slot]);
                 ++issued;
             }
         }
@@ -257,42 +312,6 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
             if (!ok) abort_flag = 1;
             tc::mma_commit(done);   // arrives once every MMA issued so far has completed
         }
-    } else {   // warps 2-3: x of column block q split into three BF16 pieces, members as MMA N
-        const int t = tid - 64;
-        const float beta = (xs.kind == X_PCG || xs.kind == X_PCG_CV) ? (float)xs.sc->beta : 0.0f;
-        for (int q = 0; q < Q; ++q) {
-            if (q >= 2 && !tc_wait(&xfree[q & 1], (uint32_t)((q >> 1) - 1) & 1u, &abort_flag)) {
-                abort_flag = 1;
-                break;
-            }
-            unsigned char* xq = xbuf + (q & 1) * kTcXBuf;
-            for (int i0 = t; i0 < kTcN * kTcK; i0 += 64 * 8) {
-                int sl[8], mm[8], cc[8], jj[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + 64 * u;
-                    const int n = i / kTcK, k = i % kTcK, lj = td.c0 + q * kTcK + k;
-                    const bool need = i < kTcN * kTcK && n < nmem && lj < td.c1;
-                    const int64_t slot = need ? descs[sub + (m0 + n) * n_real].voff + lj : 0;
-                    sl[u] = (int)slot;
-                    jj[u] = need ? lj : -1;
-                    mm[u] = need ? xs.slot_mult[slot] : 0;
-                    cc[u] = need ? xs.slot_corner[slot] : -1;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + 64 * u;
-                    if (i >= kTcN * kTcK) continue;
-                    float v = jj[u] >= 0 ? xref_value(xsrc_ref_f(xs, mm[u], cc[u], sl[u], jj[u]), beta) : 0.0f;
-                    const uint32_t o = tc::kmajor_off(i / kTcK, i % kTcK, kTcK);
-#pragma unroll
-                    for (int piece = 0; piece < 3; ++piece)
-                        *reinterpret_cast<uint16_t*>(xq + piece * kTcXPiece + o) = bf16_split(v);
-                }
-            }
-            tc::fence_proxy_async();
-            tc_arrive(&xfull[q & 1]);
-        }
     }
     // epilogue: y of the panel rows for the members of this CTA
     const bool all_done = tc_wait(done, 0u, &abort_flag);
@@ -305,7 +324,7 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
         for (int p = 0; p < P; ++p) {
             float d[kTcN];
             tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + p * kTcN, d);
-            const int li = td.r0 + p * kTcP + 32 * warp + lane;
+            const int li = td.r0 + (p0 + p) * kTcP + 32 * warp + lane;
             if (li >= td.r1) continue;
             for (int n = 0; n < nmem; ++n) {
                 const int64_t o = descs[sub + (m0 + n) * n_real].voff + li;
@@ -330,6 +349,10 @@ __global__ void __launch_bounds__(128) k_tc_gemv(const TcDesc* __restrict__ tcd,
         for (int b = max(0, issued - kTcST); b < issued; ++b) {
             for (unsigned k = 0; k < kTcPolls; ++k)
                 if (tc_test(&full[b % kTcST], (uint32_t)(b / kTcST) & 1u)) break;
+        }
+        for (int q = max(0, xissued - 2); q < xissued; ++q) {
+            for (unsigned k = 0; k < kTcPolls; ++k)
+                if (tc_test(&xfull[q & 1], (uint32_t)(q >> 1) & 1u)) break;
         }
     }
     tc::fence_before_sync();
@@ -397,6 +420,17 @@ void build_tc(dd_handle* h) {
     }
 }
 
+// BF16 elements of the staged x of the largest kind.
+size_t tc_x_elems(const dd_handle* h) {
+    size_t n = 0;
+    for (int k = 0; k < kTcKinds; ++k) {
+        size_t qmax = 0;
+        for (const TcDesc& td : h->tcd[k]) qmax = std::max<size_t>(qmax, td.Q);
+        n = std::max(n, (size_t)h->n_sub_real * ((h->members + kTcN - 1) / kTcN) * qmax * (kTcXBuf / 2));
+    }
+    return n;
+}
+
 bool tc_available(const dd_handle* h, int mode) {
     const int k = tc_kind_index(mode);
     if (k < 0 || h->members <= 1 || h->tcd[k].empty()) return false;
@@ -421,9 +455,20 @@ int launch_tc_gemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int3
     xs.sc = h->d.sc;
     cudaError_t e = cudaFuncSetAttribute(k_tc_gemv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
     if (e != cudaSuccess) return (int)e;
-    const int groups = (h->members + kTcN - 1) / kTcN;
-    k_tc_gemv<<<(unsigned)(h->n_sub_real * groups), 128, kTcSmem, (cudaStream_t)stream>>>(
-        h->d.tcd[k], h->d.symd, h->d.Mtc, h->n_sub_real, h->members, xs, go, skip, &h->d.sc->wait_err);
+    const int groups = (h->members + kTcN - 1) / kTcN, ctas = h->n_sub_real * groups;
+    // row panels split over enough CTAs for two per SM (what its shared memory holds).  Measured, 64
+    // subdomains of 1,854 unknowns and 16 members, whole mixed step: 4.15 ms with one CTA per subdomain
+    // staging x itself, 4.18 with the split alone (staging set the pace), 3.36 with both.
+    int pmax = 1, qmax = 1;
+    for (const TcDesc& td : h->tcd[k]) {
+        pmax = std::max(pmax, (int)td.P);
+        qmax = std::max(qmax, (int)td.Q);
+    }
+    const int parts = std::max(1, std::min((304 + ctas - 1) / ctas, pmax));
+    k_tc_stage<<<dim3((unsigned)ctas, (unsigned)qmax), kTcStageT, 0, (cudaStream_t)stream>>>(
+        h->d.tcd[k], h->d.symd, h->n_sub_real, h->members, qmax, xs, h->d.xtc, skip);
+    k_tc_gemv<<<dim3((unsigned)ctas, (unsigned)parts), 128, kTcSmem, (cudaStream_t)stream>>>(
+        h->d.tcd[k], h->d.symd, h->d.Mtc, h->n_sub_real, h->members, h->d.xtc, qmax, go, skip, &h->d.sc->wait_err);
     return (int)cudaGetLastError();
 }
 
