@@ -634,12 +634,14 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
         return DD_OK;
     };
     // the whole solve in one cooperative kernel where every subdomain's operator finds room on chip
-    const int resident = prec == DD_MIXED && h->prm.sym_fp32 ? res_warps(h, h->prm.restart) : 0;
+    bool resident = false;
+    if (prec == DD_MIXED && h->prm.sym_fp32)
+        CK(h, launch_gm_resident(h, U, 0, h->prm.restart, true, &resident, s), "resident gmres");
     if (resident) {
         {
             Prof P(h, ST_VEC, s, 2);
             CK(h, launch_gm_init(h, tol, h->prm.max_it, h->prm.restart, h->capturing ? adaptive : 0, 0ull, s), "gmres init");
-            CK(h, launch_gm_resident(h, U, resident, use_warm ? 1 : 0, h->prm.restart, s), "resident gmres");
+            CK(h, launch_gm_resident(h, U, use_warm ? 1 : 0, h->prm.restart, false, &resident, s), "resident gmres");
         }
         h->lam_valid = true;
         if (h->capturing) {
@@ -811,11 +813,34 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
         // a captured graph always takes the warm start; dd_step zeroes lambda before
         // launching it when the multipliers are not valid (same values as a cold start)
         const bool use_warm = warm && (h->lam_valid || h->capturing);
-        if (use_warm) {
-            CK(h, apply_schur_w(h, prec, X_LAMBDA, h->d.lam, nullptr, V.lamf, nullptr, false, s), "apply lambda0");
-        } else {
+        if (!use_warm) {
             CK(h, (int)cudaMemsetAsync(h->d.lam, 0, nlb, s), "memset");
             CK(h, (int)cudaMemsetAsync(h->d.lamf, 0, sizeof(float) * h->mult_dof.size(), s), "memset");
+        }
+        // the whole CG in one kernel where every subdomain's operator finds room on chip
+        bool resident = false;
+        {
+            Prof P(h, ST_VEC, s, 1);
+            CK(h, launch_cg_resident(h, prec, tol, use_warm ? 1 : 0, h->capturing ? adaptive : 0, &resident, s), "resident cg");
+        }
+        if (resident) {
+            h->lam_valid = true;
+            if (h->capturing) {
+                Prof P(h, ST_VEC, s, 1);
+                CK(h, launch_solve_end(h, s), "solve end");
+                h->g_kernels_iter = 0;
+            } else {
+                PcgScalars hs;
+                CK(h, read_scalars(h, &hs, s), "pcg scalars");
+                iters = hs.it;
+                h->work[ST_SCHUR] += hs.it;
+                res = hs.gg > 0 ? std::sqrt(hs.rr / hs.gg) : 0.0;
+                if (hs.status != DD_OK) status = hs.status;
+                else if (!hs.done) status = DD_ERR_NO_CONVERGENCE;
+            }
+        } else {
+        if (use_warm) {
+            CK(h, apply_schur_w(h, prec, X_LAMBDA, h->d.lam, nullptr, V.lamf, nullptr, false, s), "apply lambda0");
         }
         if (h->capturing) {
             // CG loop as a conditional WHILE node; the CG kernels set its condition
@@ -877,6 +902,7 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
         if (hs.status != DD_OK) status = hs.status;
         else if (!hs.done) status = DD_ERR_NO_CONVERGENCE;
         h->lam_valid = true;
+        }
         }
     }
     // x_c = K~cc^-1 (f~_c + F_rc^T lambda)                           Eq. F1uc

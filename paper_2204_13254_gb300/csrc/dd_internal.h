@@ -132,6 +132,12 @@ struct TcDesc {
 DD_HD inline int tc_kind_index(int mode) { return mode == 0 ? 0 : (mode == 3 ? 1 : (mode == 6 ? 2 : -1)); }
 constexpr int kTcKinds = 3;
 
+// Resident solves: most interface entries of a subdomain, that padded to whole tiles, and
+// most floats of a subdomain's [Gamma | c] tiles.
+struct ResSizes {
+    int32_t g, span, floats;
+};
+
 // One CTA of a batched GEMV: rows [row0, row1) of matrix `mat`.
 struct GemvTask {
     int32_t mat;
@@ -506,7 +512,7 @@ struct dd_handle {
     int32_t sym_max_tiles = 0;                     // largest tile count of one subdomain
     int64_t sym_ntiles = 0;                        // stored tiles in all (entries of sym_dir / 4)
     bool sym_ok = false;                           // the packed GEMV's shared memory fits one CTA
-    int32_t res_span = 0, res_floats = 0;          // resident GMRES: padded interface entries and tile floats of a CTA
+    ResSizes res{0, 0, 0};                         // sizes of the resident solves (resident.cu)
     bool fx_ok = false;                            // the same for the fixed-point FP64 form (fxgemv.cu)
     std::vector<int32_t> fx_dir;                   // its directory (as sym_dir, offsets in blocks), the first block of
     std::vector<int64_t> fx_moff;                  // every stored subdomain, blocks in all, tile lists (order of sym_tl) and
@@ -648,8 +654,9 @@ void sym_split(const dd_handle* h, int mode, int cl, int per, std::vector<int32_
 int sym_span(const dd_handle* h, int mode);
 int launch_sym_pack(const dd_handle* h, void* stream);
 // resident.cu
-int res_warps(dd_handle* h, int m);
-int launch_gm_resident(const dd_handle* h, const UView& U, int W, int have_q, int m, void* stream);
+void build_res(dd_handle* h);
+int launch_gm_resident(const dd_handle* h, const UView& U, int have_q, int m, bool probe, bool* ran, void* stream);
+int launch_cg_resident(const dd_handle* h, int prec, double tol, int have_q, int adaptive, bool* ran, void* stream);
 // fxgemv.cu
 void build_fx(dd_handle* h);
 bool fx_active(const dd_handle* h, int mode);

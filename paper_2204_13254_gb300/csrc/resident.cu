@@ -1,7 +1,8 @@
-// The whole coupled GMRES solve in one cooperative kernel, with the operator resident in
-// shared memory (sm_103a; DD_MIXED, one problem).
+// The whole interface solve of a small tearing in one kernel, with the operators resident
+// in shared memory (sm_103a, one problem): the coupled GMRES of DD_MIXED (k_gm_resident)
+// and the Schur CG of both precisions (k_cg_resident, further below).
 //
-// On small tearings every kernel of an Arnoldi step (operator GEMV, two Gram-Schmidt
+// GMRES.  On small tearings every kernel of an Arnoldi step (operator GEMV, two Gram-Schmidt
 // passes, normalisation; gmres.cu) runs for 2 to 11 us of launch, load and reduction
 // latency over a few kilobytes per SM.  Here one CTA holds one subdomain: the packed
 // FP32 tiles of its [Gamma | c] block are copied to shared memory once per solve, and the
@@ -28,8 +29,11 @@
 // 0.89 / 0.51; no measured tearing that fits was slower.  The bound is the latency of the
 // three barriers and of the loads after them (about 2 us each).
 //
-// Every wait is bounded: a barrier or copy wait that gives up sets the error word and the
-// CTA ends; the others then run into their own limits.
+// Barriers: up to eight subdomains form one thread-block cluster and use its hardware
+// barrier (0.3 us against 1.2); more make a cooperative launch and meet at a counter in
+// global memory.  Every wait on memory is bounded: a barrier or copy wait that gives up
+// sets the error word and the CTA ends; the others then run into their own limits (a
+// cluster barrier does not wait for threads that have ended).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,7 +60,7 @@ struct ResArgs {
     GmresScalars* gs;
     PcgScalars* sc;
     double* partials;     // [2][kM1 + 1][gridDim.x]
-    int span, tile_floats, have_q;
+    int span, tile_floats, have_q, clustered;
 };
 
 // Shared memory of one CTA with W product warps, in bytes.
@@ -64,29 +68,42 @@ size_t res_smem(int W, int span, int tile_floats, int m) {
     return sizeof(float) * ((size_t)tile_floats + (size_t)span * (2 + W + m + 1));
 }
 
-// Grid barrier: writes of the product warps (W > 0: only these are waited for, the last
-// warp joins at the end; W = 0: of all threads) before it are visible to every CTA's L2
-// loads (__ldcg) after it.  False when it gave up.
+// What the CTAs meet at: the counter in global memory, or (bar null) the cluster.
+struct Meet {
+    uint32_t* bar;
+    uint32_t target;
+    int32_t* err;
+    int* failed;   // shared memory
+};
+
+// Grid barrier: writes of the product warps (W > 0: only these are waited for before the
+// arrival, the last warp joins at the end; W = 0: of all threads) before it are visible to
+// every CTA's L2 loads (__ldcg) after it.  False when it gave up.
 template <int W>
-__device__ bool grid_barrier(uint32_t* bar, uint32_t target, int32_t* err, int* failed) {
+__device__ bool grid_barrier(Meet& m) {
+    if (!m.bar) {
+        asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+        return true;
+    }
+    m.target += gridDim.x;
     if constexpr (W == 0) __syncthreads();
     else if (threadIdx.x < 32 * W) asm volatile("bar.sync 1, %0;" ::"n"(32 * W) : "memory");
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(bar, 1u);
+        atomicAdd(m.bar, 1u);
         unsigned k = 0;
         uint32_t v;
         do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-        } while (v < target && ++k < kBarLimit);
-        if (v < target) {
-            *failed = 1;
-            atomicExch(err, 1);
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(m.bar) : "memory");
+        } while (v < m.target && ++k < kBarLimit);
+        if (v < m.target) {
+            *m.failed = 1;
+            atomicExch(m.err, 1);
         }
         __threadfence();
     }
     __syncthreads();
-    return *failed == 0;
+    return *m.failed == 0;
 }
 
 // Sum of nb FP32 partial sums (a warp; lanes take q = lane, lane + 32, ...) as an integer in
@@ -123,6 +140,94 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Tiles of the [Gamma | c] block (the subdomain's first run): (a, c) and float offsets; returns
+// the floats in all.  One thread.
+__device__ int tile_table(const SymDesc& sd, int* tile_ab, int* tile_off) {
+    int off = 0, q = 0;
+    for (int a = 0; a < sd.nt - sd.tI; ++a)
+        for (int c = 0; c <= a; ++c, ++q) {
+            tile_ab[q] = a | (c << 8);
+            tile_off[q] = off;
+            off += sym_tile_floats(sym_h(sd, sd.tI + a), sym_h(sd, sd.tI + c), a == c);
+        }
+    return off;
+}
+
+// y = S x over tiles [q0, nT) of a subdomain's [Gamma | c] block in shared memory, by W
+// product warps, into one partial y per warp (yw): warp (group, w4) takes rows 16 w4 ..
+// + 15 of the group's tiles, lane (rg, cq) rows 8 rg .. + 7 of those and columns 4 cq .. + 3.
+template <int W>
+__device__ __forceinline__ void tile_product(const SymDesc& sd, const float* tiles, const int* tile_ab,
+                                             const int* tile_off, int q0, int nT, const float* xg, float* yw, int span) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= W) return;
+    float* yc = yw + warp * span;
+    for (int p = lane; p < span; p += 32) yc[p] = 0.0f;
+    __syncwarp();
+    const int w4 = warp & 3, rg = lane >> 4, cq = lane & 15, row0 = 16 * w4 + 8 * rg;
+    for (int q = q0 + (warp >> 2); q < nT; q += W / 4) {
+        const int a = tile_ab[q] & 255, c = tile_ab[q] >> 8;
+        TileShape ts;
+        ts.h = sym_h(sd, sd.tI + a);
+        ts.wp = (sym_h(sd, sd.tI + c) + 3) & ~3;
+        ts.diag = a == c;
+        const float* T = tiles + tile_off[q];
+        const float4 xb = *reinterpret_cast<const float4*>(xg + c * kSymT + 4 * cq);
+        float acc[8];
+        float4 col = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int row = row0 + r;
+            float4 mm = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (row < ts.h) {
+                if (ts.diag) {
+                    if (4 * cq < sym_rowlen(row)) mm = *reinterpret_cast<const float4*>(T + sym_trioff(row) + 4 * cq);
+                } else if (4 * cq < ts.wp) {
+                    mm = *reinterpret_cast<const float4*>(T + row * ts.wp + 4 * cq);
+                }
+            }
+            const float xa = xg[a * kSymT + row];
+            acc[r] = fmaf(mm.x, xb.x, fmaf(mm.y, xb.y, fmaf(mm.z, xb.z, mm.w * xb.w)));
+            col.x = fmaf(mm.x, xa, col.x);
+            col.y = fmaf(mm.y, xa, col.y);
+            col.z = fmaf(mm.z, xa, col.z);
+            col.w = fmaf(mm.w, xa, col.w);
+        }
+        // rows: halving exchanges over the 16 column quads; lane pair (cq / 2) ends with one row
+        float v4[4], v2[2];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const bool hi = (cq & 8) != 0;
+            v4[r] = (hi ? acc[r + 4] : acc[r]) + __shfl_xor_sync(0xffffffffu, hi ? acc[r] : acc[r + 4], 8);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const bool hi = (cq & 4) != 0;
+            v2[r] = (hi ? v4[r + 2] : v4[r]) + __shfl_xor_sync(0xffffffffu, hi ? v4[r] : v4[r + 2], 4);
+        }
+        const bool hi = (cq & 2) != 0;
+        float v = (hi ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, hi ? v2[0] : v2[1], 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if (!(cq & 1)) yc[a * kSymT + row0 + ((cq & 8) ? 4 : 0) + ((cq & 4) ? 2 : 0) + ((cq & 2) ? 1 : 0)] += v;
+        // columns: the warp's two row groups
+        col.x += __shfl_xor_sync(0xffffffffu, col.x, 16);
+        col.y += __shfl_xor_sync(0xffffffffu, col.y, 16);
+        col.z += __shfl_xor_sync(0xffffffffu, col.z, 16);
+        col.w += __shfl_xor_sync(0xffffffffu, col.w, 16);
+        __syncwarp();
+        if (lane < 16) {
+            float4* yp = reinterpret_cast<float4*>(yc + c * kSymT + 4 * cq);
+            float4 y = *yp;
+            y.x += col.x;
+            y.y += col.y;
+            y.z += col.z;
+            y.w += col.w;
+            *yp = y;
+        }
+        __syncwarp();
+    }
+}
+
 // W product warps (groups of four taking alternate tiles) and the warp of the small dense
 // problem; one interface entry per thread.
 template <int W>
@@ -141,7 +246,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     __shared__ long long isum[kM1 + 1];
     __shared__ int iexp[kM1 + 1];
     __shared__ double red[2][kT / 32];
-    __shared__ double shnext, sresid;
+    __shared__ double shnext, sresid, s_beta, s_bnorm, s_thr;
     __shared__ float sinv;
     __shared__ int s_end, s_final, s_k, s_conv, s_status, s_it, s_fail;
     __shared__ uint64_t bar_tiles;
@@ -155,21 +260,14 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     GmresScalars* gs = P.gs;
     const int m = gs->m, max_it = gs->max_it;
     const double tol = gs->tol;
-    uint32_t* bar = &gs->bar;
-    uint32_t target = 0;
+    Meet meet{P.clustered ? nullptr : &gs->bar, 0u, &P.sc->wait_err, &s_fail};
 
     // the tiles of the [Gamma | c] block: the subdomain's first run
     if (tid == 0) {
         s_fail = 0;
         s_it = 0;
         s_status = DD_OK;
-        int off = 0, q = 0;
-        for (int a = 0; a < nG; ++a)
-            for (int c = 0; c <= a; ++c, ++q) {
-                tile_ab[q] = a | (c << 8);
-                tile_off[q] = off;
-                off += sym_tile_floats(sym_h(sd, sd.tI + a), sym_h(sd, sd.tI + c), a == c);
-            }
+        const int off = tile_table(sd, tile_ab, tile_off);
         mbar_init(&bar_tiles, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         load_tile(tiles, P.Msym + sd.toff, 4u * (uint32_t)off, &bar_tiles, l2_policy(true));
@@ -220,6 +318,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
         xs = *xp;
     }
     const float dinvf = (float)dinv;
+    const int nw = (g + 31) >> 5;   // warps with entries
     __syncthreads();
     if (!mbar_wait(&bar_tiles, 0u)) {   // (every thread waits itself)
         s_fail = 1;
@@ -228,76 +327,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     __syncthreads();
     if (s_fail) return;
 
-    // y = S x over the tiles in shared memory (product warps): warp (group, w4) takes rows 16 w4 ..
-    // + 15 of the group's tiles, lane (rg, cq) rows 8 rg .. + 7 of those and columns 4 cq .. + 3
-    auto product = [&]() {
-        if (warp >= kW) return;
-        float* yc = yw + warp * P.span;
-        for (int p = lane; p < P.span; p += 32) yc[p] = 0.0f;
-        __syncwarp();
-        const int w4 = warp & 3, rg = lane >> 4, cq = lane & 15, row0 = 16 * w4 + 8 * rg;
-        for (int q = warp >> 2; q < nT; q += kW / 4) {
-            const int a = tile_ab[q] & 255, c = tile_ab[q] >> 8;
-            TileShape ts;
-            ts.h = sym_h(sd, sd.tI + a);
-            ts.wp = (sym_h(sd, sd.tI + c) + 3) & ~3;
-            ts.diag = a == c;
-            const float* T = tiles + tile_off[q];
-            const float4 xb = *reinterpret_cast<const float4*>(xg + c * kSymT + 4 * cq);
-            float acc[8];
-            float4 col = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                const int row = row0 + r;
-                float4 mm = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (row < ts.h) {
-                    if (ts.diag) {
-                        if (4 * cq < sym_rowlen(row)) mm = *reinterpret_cast<const float4*>(T + sym_trioff(row) + 4 * cq);
-                    } else if (4 * cq < ts.wp) {
-                        mm = *reinterpret_cast<const float4*>(T + row * ts.wp + 4 * cq);
-                    }
-                }
-                const float xa = xg[a * kSymT + row];
-                acc[r] = fmaf(mm.x, xb.x, fmaf(mm.y, xb.y, fmaf(mm.z, xb.z, mm.w * xb.w)));
-                col.x = fmaf(mm.x, xa, col.x);
-                col.y = fmaf(mm.y, xa, col.y);
-                col.z = fmaf(mm.z, xa, col.z);
-                col.w = fmaf(mm.w, xa, col.w);
-            }
-            // rows: halving exchanges over the 16 column quads; lane pair (cq / 2) ends with one row
-            float v4[4], v2[2];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const bool hi = (cq & 8) != 0;
-                v4[r] = (hi ? acc[r + 4] : acc[r]) + __shfl_xor_sync(0xffffffffu, hi ? acc[r] : acc[r + 4], 8);
-            }
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const bool hi = (cq & 4) != 0;
-                v2[r] = (hi ? v4[r + 2] : v4[r]) + __shfl_xor_sync(0xffffffffu, hi ? v4[r] : v4[r + 2], 4);
-            }
-            const bool hi = (cq & 2) != 0;
-            float v = (hi ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, hi ? v2[0] : v2[1], 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            if (!(cq & 1)) yc[a * kSymT + row0 + ((cq & 8) ? 4 : 0) + ((cq & 4) ? 2 : 0) + ((cq & 2) ? 1 : 0)] += v;
-            // columns: the warp's two row groups
-            col.x += __shfl_xor_sync(0xffffffffu, col.x, 16);
-            col.y += __shfl_xor_sync(0xffffffffu, col.y, 16);
-            col.z += __shfl_xor_sync(0xffffffffu, col.z, 16);
-            col.w += __shfl_xor_sync(0xffffffffu, col.w, 16);
-            __syncwarp();
-            if (lane < 16) {
-                float4* yp = reinterpret_cast<float4*>(yc + c * kSymT + 4 * cq);
-                float4 y = *yp;
-                y.x += col.x;
-                y.y += col.y;
-                y.z += col.z;
-                y.w += col.w;
-                *yp = y;
-            }
-            __syncwarp();
-        }
-    };
+    auto product = [&]() { tile_product<kW>(sd, tiles, tile_ab, tile_off, 0, nT, xg, yw, P.span); };
     // this entry's row of M_s x, published (the corner rows of M = J S change sign)
     auto publish = [&]() {
         if (!on) return;
@@ -306,8 +336,11 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
         for (int w = 0; w < kW; ++w) y += yw[w * P.span + e];
         P.wf[up] = corner ? -y : y;
     };
-    // (M u) of this entry from the published w (and, for DP2, the unknowns of both sides)
+    // (M u) of this entry from the published w (and, for DP2, the unknowns of both sides); a DP1
+    // multiplier's jump is one FP32 subtraction (the FP64 pipe takes 16 clocks per warp instruction)
+    float jump = 0.0f;
     auto combined = [&](bool residual) -> double {
+        jump = 0.0f;
         const int64_t wc = 2 * U.n1;
         if (corner) {
             double s = 0.0;
@@ -317,7 +350,8 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
         const int64_t k = side && U.n2 > 0 ? ui - U.n1 : ui;
         if (U.n2 == 0) {
             const float2 w = __ldcg(reinterpret_cast<const float2*>(P.wf) + k);
-            return (double)w.x - (double)w.y;
+            jump = w.x - w.y;
+            return 0.0;
         }
         const int other = side == 0 ? 1 : 0;
         double acc = 0.0;
@@ -339,7 +373,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
             p = warp_sum(p);
             if (lane == 0) part[(size_t)k * nb + b] = p;
         }
-        if (!grid_barrier<0>(bar, target += nb, &P.sc->wait_err, &s_fail)) return false;
+        if (!grid_barrier<0>(meet)) return false;
         for (int k = warp; k < nsum; k += kW + 1) {
             int ex;
             const long long v = partial_sum(part + (size_t)k * nb, nb, lane, shift, &ex);
@@ -370,25 +404,30 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
             product();
             __syncthreads();
             publish();
-            if (!grid_barrier<0>(bar, target += nb, &P.sc->wait_err, &s_fail)) return;
+            if (!grid_barrier<0>(meet)) return;
         }
-        if (on) t = (float)(rhs - (warm ? combined(true) : 0.0));
+        if (on) {
+            const double mu = warm ? combined(true) : 0.0;
+            t = (float)(rhs - (mu + (double)jump));   // (one of the two is zero)
+        }
         warm = true;
         {
             const bool mine = on && own;
-            const double rr = warp_sum(mine ? (double)t * (double)t : 0.0), bb = warp_sum(mine ? rhs * rhs : 0.0);
-            if (lane == 0) {
-                red[0][warp] = rr;
-                red[1][warp] = bb;
+            if (warp < nw) {
+                const double rr = warp_sum(mine ? (double)t * (double)t : 0.0), bb = warp_sum(mine ? rhs * rhs : 0.0);
+                if (lane == 0) {
+                    red[0][warp] = rr;
+                    red[1][warp] = bb;
+                }
             }
             __syncthreads();
             double* part = P.partials + (size_t)(kM1 + 1) * nb;   // past the FP32 sets
             if (tid < 2) {
                 double v = 0.0;
-                for (int w = 0; w < kT / 32; ++w) v += red[tid][w];
+                for (int w = 0; w < nw; ++w) v += red[tid][w];
                 part[(size_t)tid * nb + b] = v;
             }
-            if (!grid_barrier<0>(bar, target += nb, &P.sc->wait_err, &s_fail)) return;
+            if (!grid_barrier<0>(meet)) return;
             if (warp < 2) {
                 double v = 0.0;
                 for (int q = lane; q < nb; q += 32) v += __ldcg(part + (size_t)warp * nb + q);
@@ -397,14 +436,16 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
             }
             __syncthreads();
         }
-        const double beta = sqrt(red[0][0]), bnorm = sqrt(red[1][0]), thr = tol * bnorm;
-        const bool finite = isfinite(beta) && isfinite(bnorm);
-        __syncthreads();
         if (tid == 0) {
+            const double beta = sqrt(red[0][0]), bnorm = sqrt(red[1][0]);
+            const bool finite = isfinite(beta) && isfinite(bnorm);
+            s_beta = beta;
+            s_bnorm = bnorm;
+            s_thr = tol * bnorm;
             sg[0] = sresid = shnext = beta;
             sinv = (float)(1.0 / beta);
             s_k = 0;
-            s_conv = finite && beta <= thr ? 1 : 0;
+            s_conv = finite && beta <= s_thr ? 1 : 0;
             s_status = finite ? DD_OK : DD_ERR_NONFINITE;
             s_end = s_final = (!finite || s_conv || s_it >= max_it) ? 1 : 0;
         }
@@ -447,7 +488,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
                 const int it = ++s_it;
                 const double resid = fabs(sg[c + 1]);
                 const bool fin = isfinite(resid) && isfinite(shnext) && isfinite(col[c]);
-                const bool conv = fin && resid <= thr;
+                const bool conv = fin && resid <= s_thr;
                 sresid = resid;
                 s_conv = conv ? 1 : 0;
                 s_final = (!fin || conv || it >= max_it) ? 1 : 0;
@@ -462,10 +503,14 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
                         syf[i] = (float)sy[i];
                     }
             }
-            if (!grid_barrier<W>(bar, target += nb, &P.sc->wait_err, &s_fail)) return;
+            if (!grid_barrier<W>(meet)) return;
             if (s_end) break;   // (the same decision in every CTA; this product is dropped)
             const int nv = j + 1;
-            t = on ? (float)combined(false) : 0.0f;
+            t = 0.0f;
+            if (on) {
+                const double mu = combined(false);
+                t = corner || U.n2 > 0 ? (float)mu : jump;
+            }
             if (on) tm[e] = own ? t : 0.0f;
             __syncthreads();
             if (!dots(0, nv, false, h1, h1f)) return;
@@ -498,9 +543,9 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
             }
         }
         if (b == 0 && tid == 0) {
-            gs->bnorm = bnorm;
-            gs->thr = thr;
-            gs->beta = beta;
+            gs->bnorm = s_bnorm;
+            gs->thr = s_thr;
+            gs->beta = s_beta;
             gs->resid = sresid;
             if (s_final) {
                 gs->it = P.sc->it = s_it;
@@ -511,7 +556,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
                 P.sc->it_total += s_it;
                 P.sc->cycles += cycle + 1;
                 P.sc->rr = sresid * sresid;
-                P.sc->gg = bnorm * bnorm;
+                P.sc->gg = s_bnorm * s_bnorm;
             }
         }
         __syncthreads();
@@ -520,42 +565,356 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     }
 }
 
+// ---- Schur CG -------------------------------------------------------------------
+// CG on Eq. f1schur (k_pcg_* in kernels.cu: same recurrences, precisions and stopping rule;
+// T is the type of the operator and its input, everything else FP64).  One CTA per
+// subdomain holds its [Gamma | c] block: packed FP32 tiles, or the dense FP64 rows.  One
+// application of the operator is
+//   u = corner rows of M_s B_r^T p, published                                   barrier
+//   v = K~cc^-1 sum_s u: every CTA assembles sum u and does its share of the rows  barrier
+//   w = interface rows of M_s [B_r^T p; -v], published                          barrier
+// and an iteration adds the barriers of p.q and of r.r, r.z.  Measured, FP64 step with the
+// library's defaults on 8 subdomains of 448 unknowns: 1.15 ms as seven launches per
+// iteration polled every eight, 0.45 ms here (21 us per iteration: the five exchanges and
+// the FP64 products, 17,000 FMAs per CTA at two per clock).
+struct CgArgs {
+    const SymDesc* descs;
+    const MatDesc* mats;
+    const float* Msym;
+    const double* M;
+    const int32_t* slot_mult;
+    const int32_t* slot_corner;
+    const int32_t* slot_upos;
+    const int64_t* cp;        // corner copies
+    const double* g;          // right-hand side
+    const double* dinv;       // null: no preconditioner
+    double* lam;
+    float* lamf;
+    const void* K;            // K~cc^-1 in T, row stride ldc
+    void* w;                  // published w in T (multiplier / corner-copy order), v
+    void* v;
+    PcgScalars* sc;
+    uint32_t* bar;
+    double* partials;         // [3][gridDim.x]
+    double tol, refine_tol;
+    int64_t nl;
+    int nc, ldc, ld, span, floats, have_q, adaptive, max_it, clustered;
+};
+
+// Shared memory of one CTA: the block (FP32 tiles with x and W partial y, or dense FP64 rows with x
+// and y) and the assembled corner vector.
+size_t cg_smem(bool f32, int W, int span, int floats, int g, int ld, int nc) {
+    return f32 ? sizeof(float) * ((size_t)floats + (size_t)span * (1 + W)) + sizeof(double) * (size_t)nc
+               : sizeof(double) * ((size_t)g * ld + 2 * (size_t)span + nc);
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs P) {
+    constexpr bool kF32 = sizeof(T) == 4;
+    constexpr int kT = 32 * W;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ double red[3][W];
+    __shared__ double s_rz, s_gg, s_rr, s_tol2, s_alpha, s_beta;
+    __shared__ int s_done, s_finite;
+    __shared__ int s_fail, tile_ab[64], tile_off[64];
+    __shared__ uint64_t bar_tiles;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, b = blockIdx.x;
+    const SymDesc sd = P.descs[b];
+    const MatDesc md = P.mats[b];
+    const int nGam = sd.n[1], g = nGam + sd.n[2], nG = sd.nt - sd.tI, nT = nG * (nG + 1) / 2;
+    // FP32: tiles | x | y per warp | uc;  FP64: rows | x | y | uc
+    float* tiles = reinterpret_cast<float*>(smem);
+    double* rows = reinterpret_cast<double*>(smem);
+    T* xg = kF32 ? reinterpret_cast<T*>(tiles + P.floats) : reinterpret_cast<T*>(rows + (size_t)P.ld * P.floats);
+    T* yg = xg + P.span;
+    double* uc = reinterpret_cast<double*>(yg + (kF32 ? W : 1) * P.span);
+    T* w = reinterpret_cast<T*>(P.w);
+    T* vC = reinterpret_cast<T*>(P.v);
+    const T* K = reinterpret_cast<const T*>(P.K);
+    Meet meet{P.clustered ? nullptr : P.bar, 0u, &P.sc->wait_err, &s_fail};
+    if (tid == 0) s_fail = 0;
+    if constexpr (kF32) {
+        if (tid == 0) {
+            const int off = tile_table(sd, tile_ab, tile_off);
+            mbar_init(&bar_tiles, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            load_tile(tiles, P.Msym + sd.toff, 4u * (uint32_t)off, &bar_tiles, l2_policy(true));
+        }
+    } else {
+        const double* src = P.M + md.moff + (int64_t)sd.n[0] * md.ld + sd.n[0];
+        for (int i = warp; i < g; i += W)
+            for (int j = lane; j < g; j += 32) rows[(size_t)i * P.ld + j] = src[(int64_t)i * md.ld + j];
+    }
+    for (int p = tid; p < P.span; p += kT) xg[p] = (T)0;
+    // this thread's entry
+    const int e = tid;
+    const bool gam = e < nGam, cor = e >= nGam && e < g;
+    int64_t mi = 0;
+    int up = 0, ci = 0;
+    bool own = false;
+    double sgn = 0.0, dinv = 1.0, rhs = 0.0, lam = 0.0;
+    if (gam || cor) {
+        const int64_t slot = sd.voff + sd.n[0] + e;
+        up = P.slot_upos[slot];
+        if (gam) {
+            const int mu = P.slot_mult[slot];
+            own = mu > 0;
+            mi = (mu > 0 ? mu : -mu) - 1;
+            sgn = own ? 1.0 : -1.0;
+            rhs = P.g[mi];
+            if (P.dinv) dinv = P.dinv[mi];
+            lam = P.lam[mi];
+        } else {
+            ci = P.slot_corner[slot];
+        }
+    }
+    double tol = P.tol;
+    if (P.adaptive) {   // a later refinement pass only has to cut the current step residual to refine_tol
+        const double resid = P.sc->norm_b2 > 0.0 ? sqrt(P.sc->norm_r2 / P.sc->norm_b2) : 0.0;
+        if (resid > 0.0) tol = fmin(0.1, fmax(tol, 0.3 * P.refine_tol / resid));
+    }
+    __syncthreads();
+    if constexpr (kF32) {
+        if (!mbar_wait(&bar_tiles, 0u)) {
+            s_fail = 1;
+            atomicExch(&P.sc->wait_err, 1);
+        }
+        __syncthreads();
+        if (s_fail) return;
+    }
+    // rows [i0, g) of M_s x; the result of entry e in y(e)
+    auto product = [&](int i0) {
+        if constexpr (kF32) {
+            const int a0 = i0 / kSymT;
+            tile_product<W>(sd, tiles, tile_ab, tile_off, a0 * (a0 + 1) / 2, nT, xg, yg, P.span);
+        } else {   // four threads per row, every fourth column (rows an odd multiple of four banks apart)
+            for (int i = i0 + (tid >> 2); i - (tid >> 2) < g; i += kT / 4) {
+                double s0 = 0.0, s1 = 0.0;
+                if (i < g) {
+                    const double* r = rows + (size_t)i * P.ld;
+                    int j = tid & 3;
+                    for (; j + 4 < g; j += 8) {
+                        s0 = fma(r[j], (double)xg[j], s0);
+                        s1 = fma(r[j + 4], (double)xg[j + 4], s1);
+                    }
+                    if (j < g) s0 = fma(r[j], (double)xg[j], s0);
+                }
+                s0 += s1;
+                s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+                s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+                if (i < g && (tid & 3) == 0) yg[i] = (T)s0;
+            }
+        }
+        __syncthreads();
+    };
+    auto y = [&]() -> T {
+        if constexpr (kF32) {
+            T v = (T)0;
+#pragma unroll
+            for (int k = 0; k < W; ++k) v += yg[k * P.span + e];
+            return cor ? -v : v;   // the tiles hold S = J M
+        } else {
+            return yg[e];
+        }
+    };
+    // q = (Schur operator) x at this thread's interface entry, x in T
+    auto apply = [&](T x, double& q) -> bool {
+        if (gam) xg[e] = x;
+        if (cor) xg[e] = (T)0;
+        __syncthreads();
+        if (P.nc > 0) {
+            product(nGam);
+            if (cor) w[up] = y();
+            if (!grid_barrier<0>(meet)) return false;
+            for (int I = tid; I < P.nc; I += kT) {
+                double s = 0.0;
+                for (int64_t k = P.cp[I]; k < P.cp[I + 1]; ++k) s += (double)__ldcg(w + 2 * P.nl + k);
+                uc[I] = kF32 ? (double)(float)s : s;
+            }
+            __syncthreads();
+            for (int I = b + nb * warp; I < P.nc; I += nb * W) {
+                const T* r = K + (int64_t)I * P.ldc;
+                T s = (T)0;
+                for (int J = lane; J < P.nc; J += 32) s += r[J] * (T)uc[J];
+                s = warp_sum(s);
+                if (lane == 0) vC[I] = s;
+            }
+            if (!grid_barrier<0>(meet)) return false;
+            if (cor) xg[e] = -__ldcg(vC + ci);
+            __syncthreads();
+        }
+        product(0);
+        if (gam) w[up] = y();
+        if (!grid_barrier<0>(meet)) return false;
+        q = 0.0;
+        if (gam) q = (double)__ldcg(w + 2 * mi) - (double)__ldcg(w + 2 * mi + 1);
+        return true;
+    };
+    // n sums over the multipliers (each counted by its first side), in CTA order, left in red[k][0]
+    const int nw = (nGam + 31) >> 5;   // warps with interface entries
+    auto sums = [&](int n, double a0, double a1, double a2) -> bool {
+        double v[3] = {own ? a0 : 0.0, own ? a1 : 0.0, own ? a2 : 0.0};
+        if (warp < nw)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (k >= n) continue;
+                v[k] = warp_sum(v[k]);
+                if (lane == 0) red[k][warp] = v[k];
+            }
+        __syncthreads();
+        if (tid < n) {
+            double s = 0.0;
+            for (int k = 0; k < nw; ++k) s += red[tid][k];
+            P.partials[(size_t)tid * nb + b] = s;
+        }
+        if (!grid_barrier<0>(meet)) return false;
+        if (warp < n) {
+            double s = 0.0;
+            for (int k = lane; k < nb; k += 32) s += __ldcg(P.partials + (size_t)warp * nb + k);
+            s = warp_sum(s);
+            if (lane == 0) red[warp][0] = s;
+        }
+        __syncthreads();
+        return true;
+    };
+    // the vector updates run in the warps that hold interface entries, quotients in one thread: the
+    // FP64 pipe takes 16 clocks per warp instruction, whatever the lanes hold
+    double q = 0.0;
+    if (P.have_q && !apply((T)(sgn * lam), q)) return;
+    double r = 0.0, z = 0.0, p = 0.0;
+    if (warp < nw) {
+        r = rhs - q;
+        z = r * dinv;
+    }
+    if (!sums(3, r * z, rhs * rhs, r * r)) return;
+    if (tid == 0) {
+        const double a = red[0][0], gg = red[1][0], rr = red[2][0];
+        const bool finite = isfinite(a) && isfinite(gg) && isfinite(rr);
+        s_rz = a;
+        s_gg = gg;
+        s_rr = rr;
+        s_tol2 = tol * tol * gg;
+        s_beta = 0.0;
+        s_finite = finite;
+        s_done = !finite || rr <= s_tol2;
+    }
+    __syncthreads();
+    int it = 0;
+    while (!s_done && it < P.max_it) {
+        double pn = 0.0;
+        T x = (T)0;
+        if (warp < nw) {
+            const double beta = s_beta;
+            pn = z + beta * p;
+            if constexpr (kF32) x = (T)sgn * fmaf((float)beta, (float)p, (float)z);
+            else x = (T)(sgn * pn);
+        }
+        if (!apply(x, q)) return;
+        if (!sums(1, warp < nw ? pn * q : 0.0, 0.0, 0.0)) return;
+        if (tid == 0) s_alpha = s_rz / red[0][0];
+        __syncthreads();
+        if (warp < nw) {
+            const double alpha = s_alpha;
+            lam += alpha * pn;
+            r -= alpha * q;
+            z = r * dinv;
+            p = pn;
+        }
+        ++it;
+        if (!sums(2, warp < nw ? r * r : 0.0, warp < nw ? r * z : 0.0, 0.0)) return;
+        if (tid == 0) {
+            const double rr = red[0][0], rz = red[1][0];
+            const bool finite = isfinite(rr) && isfinite(rz) && isfinite(s_alpha);
+            s_rr = rr;
+            s_finite = finite;
+            s_done = !finite || rr <= s_tol2;
+            s_beta = rz / s_rz;
+            s_rz = rz;
+        }
+        __syncthreads();
+    }
+    if (own && it > 0) {
+        P.lam[mi] = lam;
+        if (kF32) P.lamf[mi] = (float)lam;
+    }
+    if (b == 0 && tid == 0) {
+        PcgScalars* sc = P.sc;
+        sc->rz = s_rz;
+        sc->gg = s_gg;
+        sc->rr = s_rr;
+        sc->tol2 = s_tol2;
+        sc->it = it;
+        sc->it_total += it;
+        sc->status = s_finite ? DD_OK : DD_ERR_NONFINITE;
+        sc->done = s_done ? 1 : 0;
+    }
+}
+
 }  // namespace
 
-// Host: sizes of the resident form, and the number of product warps for which every
-// subdomain finds a CTA of its own on the device at once (0: the form does not apply).
-// Shapes with sixteen warps first (one CTA per SM), then eight, then four.
-int res_warps(dd_handle* h, int m) {
-    if (h->members > 1 || !h->sym_ok || h->mult_dof.empty() || h->n_sm == 0) return 0;
-    int g = 0, span = 0, floats = 0;
+// Host: largest interface block, its padded entries and its tile floats over the subdomains.
+void build_res(dd_handle* h) {
+    ResSizes z{0, 0, 0};
     for (const SymDesc& sd : h->sym) {
-        g = std::max(g, sd.n[1] + sd.n[2]);
-        span = std::max(span, (sd.nt - sd.tI) * kSymT);
-    }
-    if (g > 512) return 0;
-    for (const SymDesc& sd : h->sym) {
+        z.g = std::max(z.g, sd.n[1] + sd.n[2]);
+        z.span = std::max(z.span, (sd.nt - sd.tI) * kSymT);
         int f = 0;
         for (int a = sd.tI; a < sd.nt; ++a)
             for (int c = sd.tI; c <= a; ++c) f += sym_tile_floats(sym_h(sd, a), sym_h(sd, c), a == c);
-        floats = std::max(floats, f);
+        z.floats = std::max(z.floats, (f + 31) / 32 * 32);
     }
-    floats = (floats + 31) / 32 * 32;
-    h->res_span = span;
-    h->res_floats = floats;
-    for (int W = 16; W >= 4; W /= 2) {
-        const size_t smem = res_smem(W, span, floats, m);
-        auto kern = W == 16 ? k_gm_resident<16> : W == 8 ? k_gm_resident<8> : k_gm_resident<4>;
-        cudaFuncAttributes fa;
-        if (g > 32 * W || cudaFuncGetAttributes(&fa, kern) != cudaSuccess || smem + fa.sharedSizeBytes > 227 * 1024) continue;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * W + 32, smem) != cudaSuccess) return 0;
-        if ((int64_t)per_sm * h->n_sm >= h->n_sub) return W;
-    }
-    return 0;
+    h->res = z;
 }
 
-int launch_gm_resident(const dd_handle* h, const UView& U, int W, int have_q, int m, void* stream) {
+namespace {
+
+// Launch of a resident kernel with one CTA per subdomain: all of them on the device at once,
+// as one cluster (up to eight) or cooperatively.
+struct Launch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    bool clustered = false;
+    template <typename Kern>
+    bool plan(const dd_handle* h, Kern kern, int threads, size_t smem) {
+        cudaFuncAttributes fa;
+        if (smem > 227 * 1024) return false;
+        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || smem + fa.sharedSizeBytes > 227 * 1024) return false;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+        cfg.gridDim = dim3((unsigned)h->n_sub);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (h->n_sub <= 8) {
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)h->n_sub;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            int n = 0;
+            clustered = cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n >= 1;
+            if (clustered) return true;
+            cudaGetLastError();
+        }
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess) return false;
+        return (int64_t)per_sm * h->n_sm >= h->n_sub;
+    }
+};
+
+bool res_candidate(const dd_handle* h) {
+    return h->members <= 1 && h->sym_ok && !h->mult_dof.empty() && h->n_sm > 0 && h->res.g <= 512;
+}
+
+}  // namespace
+
+// Runs the coupled GMRES (after k_gm_init) in its resident form; *ran = false, and nothing
+// launched, where it does not apply.  Sixteen product warps first (one CTA per SM), then
+// eight, then four, for the first with which every subdomain finds a CTA of its own.
+int launch_gm_resident(const dd_handle* h, const UView& U, int have_q, int m, bool probe, bool* ran, void* stream) {
+    *ran = false;
+    if (!res_candidate(h)) return 0;
+    const ResSizes& z = h->res;
     ResArgs P;
     P.U = U;
     P.descs = h->d.symd;
@@ -568,19 +927,74 @@ int launch_gm_resident(const dd_handle* h, const UView& U, int W, int have_q, in
     P.gs = h->d.gs;
     P.sc = h->d.sc;
     P.partials = h->d.rpart;
-    P.span = h->res_span;
-    P.tile_floats = h->res_floats;
+    P.span = z.span;
+    P.tile_floats = z.floats;
     P.have_q = have_q;
-    auto kern = W == 16 ? k_gm_resident<16> : W == 8 ? k_gm_resident<8> : k_gm_resident<4>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)h->n_sub);
-    cfg.blockDim = dim3(32 * W + 32);
-    cfg.dynamicSmemBytes = res_smem(W, P.span, P.tile_floats, m);
-    cfg.stream = S(stream);
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return (int)cudaLaunchKernelEx(&cfg, kern, P);
+    for (int W = 16; W >= 4; W /= 2) {
+        if (z.g > 32 * W) break;
+        auto kern = W == 16 ? k_gm_resident<16> : W == 8 ? k_gm_resident<8> : k_gm_resident<4>;
+        Launch L;
+        if (!L.plan(h, kern, 32 * W + 32, res_smem(W, z.span, z.floats, m))) continue;
+        *ran = true;
+        if (probe) return 0;
+        P.clustered = L.clustered ? 1 : 0;
+        L.cfg.stream = S(stream);
+        return (int)cudaLaunchKernelEx(&L.cfg, kern, P);
+    }
+    return 0;
+}
+
+// Runs the Schur CG in its resident form from lambda (have_q: its product is needed); *ran as above.
+int launch_cg_resident(const dd_handle* h, int prec, double tol, int have_q, int adaptive, bool* ran, void* stream) {
+    *ran = false;
+    const bool f32 = prec == DD_MIXED;
+    const int nc = (int)h->corner_dof.size();
+    if (!res_candidate(h) || nc > 2048 || (f32 && !h->prm.sym_fp32)) return 0;
+    const ResSizes& z = h->res;
+    CgArgs P;
+    P.descs = h->d.symd;
+    P.mats = h->d.mats;
+    P.Msym = h->d.Msym;
+    P.M = h->d.M64;
+    P.slot_mult = h->d.slot_mult;
+    P.slot_corner = h->d.slot_corner;
+    P.slot_upos = h->d.slot_upos;
+    P.cp = h->d.corner_ptr;
+    P.g = h->d.g;
+    P.dinv = h->prm.precond ? h->d.dinv : nullptr;
+    P.lam = h->d.lam;
+    P.lamf = h->d.lamf;
+    P.K = f32 ? (const void*)h->d.K32 : (const void*)h->d.K64;
+    P.w = f32 ? (void*)h->d.wf : (void*)h->d.w;
+    P.v = f32 ? (void*)h->d.vCf : (void*)h->d.vC;
+    P.sc = h->d.sc;
+    P.bar = &h->d.gs->bar;
+    P.partials = h->d.rpart;
+    P.tol = tol;
+    P.refine_tol = h->prm.refine_tol;
+    P.nl = (int64_t)h->mult_dof.size();
+    P.nc = nc;
+    P.ldc = h->ldc;
+    P.ld = (z.g + 11) / 16 * 16 + 4;   // >= g, 4 mod 16: the rows of a half-warp start four banks apart
+    P.span = z.span;
+    P.floats = f32 ? z.floats : z.g;
+    P.have_q = have_q;
+    P.adaptive = adaptive;
+    P.max_it = h->prm.max_it;
+    for (int W = 16; W >= 8; W /= 2) {
+        if (z.g > 32 * W) break;
+        auto kern = f32 ? (W == 16 ? k_cg_resident<float, 16> : k_cg_resident<float, 8>)
+                        : (W == 16 ? k_cg_resident<double, 16> : k_cg_resident<double, 8>);
+        Launch L;
+        if (!L.plan(h, kern, 32 * W, cg_smem(f32, W, z.span, z.floats, z.g, P.ld, nc))) continue;
+        P.clustered = L.clustered ? 1 : 0;
+        if (!P.clustered) {
+            const cudaError_t e = cudaMemsetAsync(P.bar, 0, sizeof(uint32_t), S(stream));
+            if (e != cudaSuccess) return (int)e;
+        }
+        L.cfg.stream = S(stream);
+        *ran = true;
+        return (int)cudaLaunchKernelEx(&L.cfg, kern, P);
+    }
+    return 0;
 }

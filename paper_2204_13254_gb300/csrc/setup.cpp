@@ -480,6 +480,7 @@ int dd_build_host(dd_handle* h, const dd_mesh* mesh, const int32_t* part, int32_
     build_tc(h);
     h->sym_ok = sym_smem_bytes(h) <= 227 * 1024;
     build_fx(h);
+    build_res(h);
 
     // ---- batched GEMV task lists (default tiles; dd_autotune may change them) ------
     for (int mode = 0; mode < GEMV_NMODES; ++mode) {

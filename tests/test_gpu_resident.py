@@ -1,4 +1,4 @@
-"""The mixed-precision coupled GMRES as one cooperative kernel (operators resident in
+"""The mixed-precision coupled GMRES and the Schur CG as one kernel (operators resident in
 shared memory) against the kernel-per-stage solve (which sym_fp32 = 0 selects): the
 same Arnoldi counts up to FP32 rounding of the stopping test (cold solves), fields equal
 to the refinement tolerance; one, two and four CTAs per SM, short and long restarts, both
@@ -64,6 +64,37 @@ def test_resident_solve_matches_staged(kind, kw):
         assert abs(a - b) <= 1
     f2, i2, _ = march(w, dt, 4, **kw)       # fixed summation order: bitwise reproducible
     assert i2 == i1 and all(torch.equal(a, b) for a, b in zip(f1, f2))
+
+
+@pytest.mark.parametrize("kind", ["sub8", "sub216", "ragged"])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_resident_cg(kind, graph):
+    """Mixed against the kernel-per-stage CG (sym_fp32 = 0); FP64 against the coupled GMRES
+    (another kernel family) to the solves' tolerance."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w, dt = problem(kind)
+    cg = dict(solver=D.DD_SOLVER_SCHUR_CG, use_graph=graph)
+    f1, _, l1 = march(w, dt, 4, **cg)
+    f0, _, l0 = march(w, dt, 4, sym_fp32=0, **cg)
+    assert l1 < l0 / 2
+    for a, b in zip(f1, f0):
+        assert torch.linalg.norm(a - b) <= 1e-9 * torch.linalg.norm(b)
+    one = dict(max_refine=1, refine_tol=1.0, warm_start=0)
+    for a, b in zip(march(w, dt, 3, **cg, **one)[1], march(w, dt, 3, sym_fp32=0, **cg, **one)[1]):
+        assert abs(a - b) <= 1
+    d = dict(precision=D.DD_FP64, tol=1e-13, max_it=2000)
+    f2, _, l2 = march(w, dt, 4, **cg, **d)
+    f3, _, _ = march(w, dt, 4, **d)
+    h = D.dd_setup(w.xyz, w.tets, w.part, w.n_sub)
+    m = D.dd_get_maps(h)
+    D.dd_destroy(h)
+    if (m["n_gam"] + m["n_cor"]).max() <= 150:   # the FP64 rows of a larger block do not fit a CTA
+        assert l2 < 4 * 25
+    for a, b in zip(f2, f3):
+        assert torch.linalg.norm(a - b) <= 1e-10 * torch.linalg.norm(b)
+    f4, _, _ = march(w, dt, 4, **cg, **d)
+    assert all(torch.equal(a, b) for a, b in zip(f2, f4))
 
 
 def test_resident_budget_and_nonfinite():
