@@ -28,9 +28,9 @@
 // (GB300: two FP64 lanes per clock and SM) against 16 bytes of HBM traffic; the
 // wide pivot block and the triangle each halve both against 32-wide blocks over
 // the full square.  Measured, 40 matrices of up to 2,454 rows with their 1,229-row
-// coarse matrix: pivot 0.17, panel 0.08, update 0.38 ms per 64-wide block (mean over
+// coarse matrix: pivot 0.15, panel 0.07, update 0.26 ms per 64-wide block (mean over
 // both), against 0.51 + 0.09 (panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide
-// block over the full square; the whole factorisation 37 against 170 ms.
+// block over the full square; the whole factorisation 33 against 170 ms.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -111,6 +111,27 @@ __device__ __forceinline__ void ld_classes(uint32_t t, uint32_t cls, uint32_t (&
 #undef OZ_O
 }
 
+// The same for the update: eight columns of 32 lanes in the 16 x 256-bit shape, by which a thread
+// gets columns 2 (lane % 4), + 1 of rows lane / 4 + 8 k in r[.][2 k], r[.][2 k + 1]: four lanes
+// cover 64 contiguous bytes of a row of doubles.
+__device__ __forceinline__ void ld_classes_pairs(uint32_t t, uint32_t cls, uint32_t (&r)[kOzS][8]) {
+#pragma unroll
+    for (int d = 0; d < kOzS; ++d) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];\n"
+                         : "=r"(r[d][4 * h]), "=r"(r[d][4 * h + 1]), "=r"(r[d][4 * h + 2]), "=r"(r[d][4 * h + 3])
+                         : "r"(t + d * cls + ((uint32_t)(16 * h) << 16))
+                         : "memory");
+    }
+    // the registers pass through the wait so that no use moves above it
+#define OZ_P(d) "+r"(r[d][0]), "+r"(r[d][1]), "+r"(r[d][2]), "+r"(r[d][3]), "+r"(r[d][4]), "+r"(r[d][5]), "+r"(r[d][6]), "+r"(r[d][7])
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" : OZ_P(0), OZ_P(1), OZ_P(2) : : "memory");
+    asm volatile("" : OZ_P(3), OZ_P(4), OZ_P(5) : : "memory");
+    asm volatile("" : OZ_P(6) : : "memory");
+#undef OZ_P
+}
+
 // T of one element: sum_d D_d 2^(8 (5-d)) ... in units of 2^-40 of class 0, i.e. the
 // product is T 2^(e + f - 56) (|T| < 2^63; class 6 rounded in, see the file comment).
 __device__ __forceinline__ double join_classes(const uint32_t (&r)[kOzS][8], int c) {
@@ -165,38 +186,120 @@ __device__ __forceinline__ void oz_bulk(void* dst, const void* src, uint32_t byt
         : "memory");
 }
 
-// The 28 slice products (x 4 K-steps) of A rows (slices at a0, sa bytes apart) and B
-// rows (b0, sb apart) into the class accumulators at `acc`, `cls` columns apart.
-__device__ __forceinline__ void oz_products(uint32_t acc, uint32_t cls, uint32_t a0, uint32_t sa, uint32_t b0,
-                                            uint32_t sb, uint32_t idesc) {
-    for (int d = 0; d < kOzS; ++d)
-        for (int p = 0; p <= d; ++p)
+// The 28 slice products of A rows (slices at a0, kOzPiece bytes apart) and `cls` B rows (slices
+// at b0, one after the other) into the class accumulators at `acc`, `cls` columns apart.
+// For one slice p of A the classes p + q lie side by side, and so do the slices q of B: one
+// MMA takes as many q as N = 256 columns allow.  An MMA reads its 128 x 16 A operand from
+// shared memory whatever N is, which at N = 32 takes four times the product itself (measured,
+// per-block means: update 384 -> 367 us, panel 77 -> 72 us against 112 MMAs of N = 32 per unit).
+__device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, uint32_t b0) {
+    const int qmax = 256 / cls;
+    const uint32_t sb = (uint32_t)cls * kOzK * 2;
+    for (int p = 0; p < kOzS; ++p)
+        for (int q = 0; q < kOzS - p; q += qmax) {
+            const int nq = min(qmax, kOzS - p - q);
+            const uint32_t idesc = tc::idesc_bf16_f32(kOzRows, nq * cls);
             for (int ks = 0; ks < kOzK / 16; ++ks) {
-                const uint64_t ad = tc::smem_desc(a0 + p * sa + ks * 256, 128, (kOzK / 8) * 128);
-                const uint64_t bd = tc::smem_desc(b0 + (d - p) * sb + ks * 256, 128, (kOzK / 8) * 128);
-                tc::mma_bf16(acc + d * cls, ad, bd, idesc, (p | ks) ? 1u : 0u);
+                const uint64_t ad = tc::smem_desc(a0 + p * kOzPiece + ks * 256, 128, (kOzK / 8) * 128);
+                const uint64_t bd = tc::smem_desc(b0 + q * sb + ks * 256, 128, (kOzK / 8) * 128);
+                tc::mma_bf16(acc + (p + q) * cls, ad, bd, idesc, (p | ks) ? 1u : 0u);
             }
+        }
 }
 
 // ---- pivot block -------------------------------------------------------------
 // P^-1 of the pivot block, one CTA per matrix.
-//  * X by a Gauss-Jordan sweep (SPD: no pivoting) over the lower triangle in registers:
-//    thread (ty, tx) of 16 x 16 holds elements (ty + 16 u, tx + 16 v), v <= u.  Step k
-//    publishes the vector r (row k left of the diagonal, column k below it) and 1 / d;
-//    then P_ij -= (s_i r_i) (r_j / d).  A serial chain of 64 steps of ten FMAs per thread,
-//    FP64-ALU bound.
-//  * The 64 roundings of every element were the largest error of the whole elimination
-//    (the products are exact to 2^-54), so X is corrected once: R = I - P X from exact
-//    57-bit fixed-point sums, X += X R in FP32 (R is of the order of FP64 rounding).  That
-//    leaves X at its own rounding.  Measured, coupled operator against an extended-precision
-//    reference, seven meshes (six bisected into 139 to 600 uneven subdomains): 2.3e-16 ..
-//    3.8e-16; without the correction 2.9e-16 .. 4.5e-16, with 32-wide pivot blocks in plain
-//    FP64 2.5e-16 .. 4.0e-16.  It costs 49 of the kernel's 173 us per block (40 matrices).
+//  * A first X by a Gauss-Jordan sweep in FP32 (SPD: no pivoting; the block scaled by powers of
+//    two to a diagonal in [1/4, 1)) over the lower triangle in registers: thread (ty, tx) of
+//    16 x 16 holds elements (ty + 16 u, tx + 16 v), v <= u.  Step k publishes the vector r (row
+//    k left of the diagonal, column k below it) and 1 / d; then P_ij -= (s_i r_i) (r_j / d).
+//  * Newton: R = I - P X from exact 57-bit fixed-point sums, X += X R in FP32, until |R| was
+//    below 2^-34 (twice as a rule: 2^-19, then 2^-38): X ends at its own FP64 rounding.
+//  * Where the FP32 sweep meets a pivot that is not positive or leaves |R| >= 2^-5, the sweep
+//    is done in FP64 (it decides whether the matrix is positive definite) and corrected once.
+// The FP64 sweep is 64 steps of ten FMAs per thread, FP64-ALU bound at 124 us per block; with
+// one correction 173 us, in FP32 with two corrections 147 us (40 matrices).  Its 64
+// roundings per element would be the largest error of the elimination (the products are
+// exact to 2^-54).  Measured, coupled operator against an extended-precision reference, seven
+// meshes (six bisected into 139 to 600 uneven subdomains): 2.3e-16 .. 3.8e-16; with the FP64
+// sweep alone 2.9e-16 .. 4.5e-16, with 32-wide pivot blocks in plain FP64 2.5e-16 .. 4.0e-16.
 // Writes P^-1 back into M[p, p] (the panel kernel does not read that block), and its slices
 // and exponents.
 constexpr int kOzPivThreads = 256;
 constexpr int kPs = kOzK + 1;   // row stride in shared memory
 constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2));
+
+// The sweep in type T; r [2][kOzK], t [kOzK], sinv [2], bad in shared memory (r and sinv by
+// step parity: a step's readers meet the next writers two barriers on).  False, in every
+// thread, if a pivot was not positive (it counts as 1 then).
+template <typename T>
+__device__ __forceinline__ bool gauss_jordan(T (&a)[4][4], T* r, T* t, T* sinv, int* bad, int nb, int tid) {
+    const int tx = tid & 15, ty = tid >> 4;
+    if (tid == 0) *bad = 0;
+    for (int k = 0; k < nb; ++k) {
+        T* rk = r + (k & 1) * kOzK;
+        const int uk = k >> 4, kk = k & 15;
+        // publish row k (j < k) and column k (i > k), and 1 / d
+        if (ty == kk) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    if (u != uk) continue;
+                    const int j = tx + 16 * v;
+                    if (j < k) rk[j] = a[u][v];
+                    if (j == k) {
+                        T d = a[u][v];
+                        if (!(d > (T)0) || !isfinite(d)) {
+                            *bad = 1;
+                            d = (T)1;
+                        }
+                        sinv[k & 1] = (T)1 / d;
+                    }
+                }
+        }
+        if (tx == kk) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    if (v != uk) continue;
+                    const int i = ty + 16 * u;
+                    if (i > k) rk[i] = a[u][v];
+                }
+        }
+        __syncthreads();
+        if (tid < kOzK) t[tid] = tid == k ? (T)0 : rk[tid] * sinv[k & 1];
+        __syncthreads();
+        T sr[4], tj[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = ty + 16 * u, j = tx + 16 * u;
+            sr[u] = i == k ? (T)0 : (i < k ? -rk[i] : rk[i]);
+            tj[u] = t[j];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) a[u][v] = fma(-sr[u], tj[v], a[u][v]);
+        // row and column k of the swept matrix
+        if (ty == kk || tx == kk) {
+            const T inv = sinv[k & 1];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) {
+                    const int i = ty + 16 * u, j = tx + 16 * v;
+                    if (i == k && j == k) a[u][v] = inv;
+                    else if (i == k && j < k) a[u][v] = -t[j];
+                    else if (j == k && i > k) a[u][v] = t[i];
+                }
+        }
+    }
+    __syncthreads();
+    return *bad == 0;
+}
+
 __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
                                                             int k0, uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
                                                             int32_t* __restrict__ status) {
@@ -207,19 +310,21 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
     double* Q = reinterpret_cast<double*>(smem);         // [kOzK][kPs] the block in full; then R in FP32
     int2* Pi = reinterpret_cast<int2*>(Q + kOzK * kPs);  // [kOzK][kPs] P, row i in units of 2^(rp_i - 57)
     int2* Xi = Pi + kOzK * kPs;                          // [kOzK][kPs] X, column j in units of 2^(cx_j - 57)
-    __shared__ double r[2][kOzK], t[kOzK], sinv[2];   // by step parity: a step's readers meet the next writers two barriers on
-    __shared__ int rp[kOzK], cx[kOzK];
+    __shared__ double sw[2 * kOzK + kOzK + 2];           // the sweep's r, t, sinv
+    __shared__ int rp[kOzK], cx[kOzK], sd[kOzK], s_bad;
     double* A = M + md.moff + (int64_t)k0 * md.ld + k0;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int ri = tid >> 2, rq = tid & 3;   // (row, quarter of its 64 columns) for row maxima and slices
     double a[4][4];
+    auto load = [&]() {
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v <= u; ++v) {
-            const int i = ty + 16 * u, j = tx + 16 * v;
-            a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : (i == j ? 1.0 : 0.0);
-        }
+            for (int v = 0; v <= u; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v;
+                a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : (i == j ? 1.0 : 0.0);
+            }
+    };
     // the lower triangle in registers -> the full symmetric block in Q (zero outside nb)
     auto spread = [&]() {
 #pragma unroll
@@ -241,83 +346,39 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         return exp_of_hi(mx);
     };
+    load();
     spread();
     {
         const int e = row_exp();
         rp[ri] = e;
         for (int k = 0; k < 16; ++k) Pi[ri * kPs + 16 * rq + k] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
+        if (rq == 0) sd[ri] = ri < nb ? (exp_of_hi(__double2hiint(Q[ri * kPs + ri]) & 0x7fffffff) + 1) >> 1 : 0;
     }
-    for (int k = 0; k < nb; ++k) {
-        double* rk = r[k & 1];
-        const int uk = k >> 4, kk = k & 15;
-        // publish row k (j < k) and column k (i > k), and 1 / d
-        if (ty == kk) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    if (u != uk) continue;
-                    const int j = tx + 16 * v;
-                    if (j < k) rk[j] = a[u][v];
-                    if (j == k) {
-                        double d = a[u][v];
-                        if (!(d > 0.0) || !isfinite(d)) {
-                            atomicCAS(status, 0, DD_ERR_NOT_SPD);
-                            d = 1.0;
-                        }
-                        sinv[k & 1] = 1.0 / d;
-                    }
-                }
-        }
-        if (tx == kk) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    if (v != uk) continue;
-                    const int i = ty + 16 * u;
-                    if (i > k) rk[i] = a[u][v];
-                }
-        }
-        __syncthreads();
-        if (tid < kOzK) t[tid] = tid == k ? 0.0 : rk[tid] * sinv[k & 1];
-        __syncthreads();
-        double sr[4], tj[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = ty + 16 * u, j = tx + 16 * u;
-            sr[u] = i == k ? 0.0 : (i < k ? -rk[i] : rk[i]);
-            tj[u] = t[j];
-        }
+    __syncthreads();
+    {   // X = D (D P D)^-1 D with D = diag(2^-sd)
+        float f[4][4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v <= u; ++v) a[u][v] = fma(-sr[u], tj[v], a[u][v]);
-        // row and column k of the swept matrix
-        if (ty == kk || tx == kk) {
-            const double inv = sinv[k & 1];
+            for (int v = 0; v <= u; ++v)
+                f[u][v] = (float)scale2(a[u][v], -sd[ty + 16 * u] - sd[tx + 16 * v]);
+        float* fs = reinterpret_cast<float*>(sw);
+        const bool ok = gauss_jordan(f, fs, fs + 2 * kOzK, fs + 3 * kOzK, &s_bad, nb, tid);
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    const int i = ty + 16 * u, j = tx + 16 * v;
-                    if (i == k && j == k) a[u][v] = inv;
-                    else if (i == k && j < k) a[u][v] = -t[j];
-                    else if (j == k && i > k) a[u][v] = t[i];
-                }
+            for (int v = 0; v <= u; ++v) a[u][v] = ok ? scale2((double)f[u][v], -sd[ty + 16 * u] - sd[tx + 16 * v]) : 0.0;
+    }
+    bool swept = false;   // in FP64
+    for (int pass = 0; pass < 4; ++pass) {
+        spread();
+        {
+            const int e = row_exp();   // X is symmetric: also its column exponent
+            cx[ri] = e;
+            for (int k = 0; k < 16; ++k) Xi[(16 * rq + k) * kPs + ri] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
         }
-    }
-    __syncthreads();   // Pi was read from Q by every thread before the first step's barriers
-    spread();
-    {
-        const int e = row_exp();   // X is symmetric: also its column exponent
-        cx[ri] = e;
-        for (int k = 0; k < 16; ++k) Xi[(16 * rq + k) * kPs + ri] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
-    }
-    __syncthreads();
-    // R = I - P X: 64 products per element fit the accumulators; |R| >= 2^-20 (or exponents out of
-    // range) means that the sweep itself went wrong: X stays as it is
-    {
+        __syncthreads();
+        // R = I - P X: 64 products per element fit the accumulators
         float* R = reinterpret_cast<float*>(Q);
         long long hh[4][4] = {}, xx[4][4] = {};
         for (int k = 0; k < nb; ++k) {
@@ -332,7 +393,7 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
 #pragma unroll
                 for (int v = 0; v < 4; ++v) mac(hh[u][v], xx[u][v], p[u].x, p[u].y, x[v].x, x[v].y);
         }
-        bool big = false;
+        int big = 0;   // 2: |R| >= 2^-5 (or exponents out of range), 1: |R| >= 2^-34
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -341,30 +402,41 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
                 __int128 d = -(((__int128)hh[u][v] << kLow) + xx[u][v]);
                 float f = 0.0f;
                 if (i < nb && j < nb) {
-                    if (sh < 24 || sh > 120) {
-                        big = true;
+                    if (sh < 40 || sh > 120) {
+                        big = 2;
                     } else {
                         if (i == j) d += (__int128)1 << sh;
-                        const __int128 lim = (__int128)1 << (sh - 20);
-                        if (d > lim || d < -lim) big = true;
-                        else f = (float)(long long)(d >> (sh > 80 ? sh - 80 : 0)) * exp2f(-(float)(sh > 80 ? 80 : sh));
+                        const __int128 m = d < 0 ? -d : d;
+                        if (m >= (__int128)1 << (sh - 5)) big = 2;
+                        else if (m >= (__int128)1 << (sh - 34)) big = max(big, 1);
+                        f = (float)(long long)(d >> (sh > 60 ? sh - 60 : 0)) * exp2f(-(float)(sh > 60 ? 60 : sh));
                     }
                 }
                 R[i * kPs + j] = f;   // (every thread is done with Q)
             }
-        if (!__syncthreads_or(big)) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    const int i = ty + 16 * u, j = tx + 16 * v;
-                    float s = 0.0f;
-                    for (int k = 0; k < nb; ++k) s = fmaf((float)Xi[k * kPs + i].x, R[k * kPs + j], s);
-                    if (i < nb && j <= i) a[u][v] += (double)s * pow2(cx[i] - (kBits - kLow));
-                }
+        const int any2 = __syncthreads_or(big == 2), any1 = __syncthreads_or(big >= 1);
+        if (any2) {
+            if (swept) break;   // nothing to correct: the status says why, or the block is beyond FP64
+            load();
+            double(&ad)[4][4] = a;
+            if (!gauss_jordan(ad, sw, sw + 2 * kOzK, sw + 3 * kOzK, &s_bad, nb, tid) && tid == 0)
+                atomicCAS(status, 0, DD_ERR_NOT_SPD);
+            swept = true;
+            continue;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v;
+                float s = 0.0f;
+                for (int k = 0; k < nb; ++k) s = fmaf((float)Xi[k * kPs + i].x, R[k * kPs + j], s);
+                if (i < nb && j <= i) a[u][v] += (double)s * pow2(cx[i] - (kBits - kLow));
+            }
         __syncthreads();
+        if (!any1) break;
     }
+    __syncthreads();
     spread();
     for (int p = tid; p < kOzK * kOzK; p += kOzPivThreads) {
         const int i = p >> 6, j = p & 63;
@@ -458,8 +530,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
         ok = oz_wait(&bars[0], 0u);
         if (ok) {
             tc::fence_after_sync();
-            oz_products(tmem, kOzK, tc::smem_addr(sB), kOzPiece, tc::smem_addr(sP), kOzPPiece,
-                        tc::idesc_bf16_f32(kOzRows, kOzK));
+            oz_products(tmem, kOzK, tc::smem_addr(sB), tc::smem_addr(sP));
         }
         tc::mma_commit(&bars[1]);
     }
@@ -513,16 +584,21 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
 // ---- trailing update ------------------------------------------------------------
 // One CTA per (128-row block, run of kOzRun 32-column units of its lower triangle,
 // matrix): the row block's 112 KB of slices are copied once for the run; the units'
-// 28 KB come through a ring of four buffers, two units ahead.  Warp 8 issues the copies
-// and the MMAs of unit u into tensor-memory half u & 1 while warps 0..7 combine unit
-// u - 1 from the other half: warp w reads rows 32 (w mod 4) .. + 31 (its tensor-memory
-// lanes) and columns 16 (w / 4) .. + 15, and adds the exact update to C (loaded before
-// the wait).  Bound by the epilogue's two FP64 operations per element.  Every wait is
-// bounded; a CTA whose wait gives up sets the error word, lets its copies land and
-// frees its tensor memory.
+// 28 KB come through a ring of four buffers, two units ahead.  Warp 8 issues the copies and
+// the MMAs; warps 0..7 (rows 32 (w mod 4) .. + 31, columns 16 (w / 4) .. + 15) combine unit
+// n from one tensor-memory half while the MMAs of unit n + 1 run into the other.
+// What bounds it: latency and the path to L2 rather than the two FP64 operations per element.
+// C is loaded a unit ahead (367 -> 350 us, mean over the blocks of 40 matrices of up to 2,454
+// rows and their coarse matrix), and a thread holds column pairs of four rows so that a warp's
+// access is whole 64-byte pieces of rows: with a row per lane every 16-byte access was half a
+// sector, and the copies leave too little L1 to join them (350 -> 260 us).  Sixteen warps of
+// eight columns with warp 0 issuing were slower in both layouts (398, 309 us).
+// Every wait is bounded; a CTA whose wait gives up sets the error word, lets its copies land
+// and frees its tensor memory.
 constexpr int kOzRun = 16;
 constexpr int kOzStages = 4;
 constexpr int kOzThreads = 288;
+constexpr int kOzWCols = 16;   // columns of a unit per warp
 constexpr size_t kOzSmem = kOzBlock + kOzStages * kOzUnit + (1 + 2 * kOzStages + 4) * sizeof(uint64_t) + 16;
 static_assert(kOzSmem <= 227 * 1024, "shared memory of the update");
 
@@ -600,55 +676,80 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
 
+    // the issuing lane: the copy of unit n + 2 and the MMAs of unit n
+    auto issue = [&](int n) {
+        const int s = n % kOzStages, hh = n & 1;
+        bool ok = true;
+        if (n + 2 < nu) {   // unit n + 2 into the stage of unit n - 2
+            if (n >= 2) ok = oz_wait_or_abort(&empty[(n - 2) % kOzStages], (uint32_t)((n - 2) / kOzStages) & 1u, &abort_flag);
+            if (ok) copy_unit(n + 2);
+        }
+        if (ok) ok = oz_wait_or_abort(&full[s], (uint32_t)(n / kOzStages) & 1u, &abort_flag);
+        if (ok && n >= 2) ok = oz_wait_or_abort(&tempty[hh], (uint32_t)((n >> 1) - 1) & 1u, &abort_flag);
+        if (!ok) {
+            abort_flag = 1;
+            return;
+        }
+        tc::fence_after_sync();
+        oz_products(tmem + 256u * hh, kOzCols, tc::smem_addr(sA), tc::smem_addr(sC + s * kOzUnit));
+        tc::mma_commit(&tfull[hh]);
+        tc::mma_commit(&empty[s]);
+    };
     if (warp == 8) {
         if (lane == 0) {
-            const uint32_t idesc = tc::idesc_bf16_f32(kOzRows, kOzCols);
-            bool ok = oz_wait(abar, 0u);
-            for (int n = 0; n < nu && ok; ++n) {
-                const int s = n % kOzStages, hh = n & 1;
-                if (n + 2 < nu) {   // unit n + 2 into the stage of unit n - 2
-                    if (n >= 2) ok = oz_wait_or_abort(&empty[(n - 2) % kOzStages], (uint32_t)((n - 2) / kOzStages) & 1u, &abort_flag);
-                    if (!ok) break;
-                    copy_unit(n + 2);
-                }
-                ok = oz_wait_or_abort(&full[s], (uint32_t)(n / kOzStages) & 1u, &abort_flag);
-                if (ok && n >= 2) ok = oz_wait_or_abort(&tempty[hh], (uint32_t)((n >> 1) - 1) & 1u, &abort_flag);
-                if (!ok) break;
-                tc::fence_after_sync();
-                oz_products(tmem + 256u * hh, kOzCols, tc::smem_addr(sA), kOzPiece, tc::smem_addr(sC + s * kOzUnit),
-                            kOzUPiece, idesc);
-                tc::mma_commit(&tfull[hh]);
-                tc::mma_commit(&empty[s]);
-            }
-            if (!ok) abort_flag = 1;
+            if (!oz_wait(abar, 0u)) abort_flag = 1;
+            for (int n = 0; n < nu && !abort_flag; ++n) issue(n);
         }
     } else {
-        const int r = 32 * (warp & 3) + lane, hcol = 16 * (warp >> 2);
-        const int i = rb * kOzRows + r;
-        const bool row_ok = i < md.ns && (i < k0 || i >= k0 + nb);
-        const int e = row_ok ? eb[(int64_t)m * nmax + i] : 0;
-        const double sgn = i < k0 ? -1.0 : 1.0;
-        double* crow = M + md.moff + (int64_t)i * md.ld;
+        // rows i0 + 8 k, columns j0 .. j0 + 1 of every group of eight
+        const int i0 = rb * kOzRows + 32 * (warp & 3) + (lane >> 2);
+        const int hcol = kOzWCols * (warp >> 2) + 2 * (lane & 3);
         const int32_t* ecm = ec + (int64_t)m * nmax;
+        double* crow = M + md.moff + (int64_t)i0 * md.ld;
+        const int64_t step = 8 * (int64_t)md.ld;
+        int e[4], jend[4], sg[4];   // exponent, end of the row in the lower triangle, sign bit
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + 8 * k;
+            const bool row_ok = i < md.ns && (i < k0 || i >= k0 + nb);
+            e[k] = row_ok ? eb[(int64_t)m * nmax + i] : 0;
+            jend[k] = row_ok ? i + 1 : 0;
+            sg[k] = i < k0 ? (int)0x80000000 : 0;
+        }
+        auto in = [&](int k, int j) { return j < jend[k] && (j < k0 || j >= k0 + nb); };
+        auto load_c = [&](int n, double (&c)[kOzWCols], int (&f)[kOzWCols / 4]) {
+#pragma unroll
+            for (int g = 0; g < kOzWCols / 8; ++g) {
+                const int j = unit(n) * kOzCols + hcol + 8 * g;
+                f[2 * g] = j < md.ns ? ecm[j] : 0;
+                f[2 * g + 1] = j + 1 < md.ns ? ecm[j + 1] : 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    double* const p = crow + k * step + j;
+                    double2 t = make_double2(0.0, 0.0);
+                    if (in(k, j) && in(k, j + 1)) t = *reinterpret_cast<const double2*>(p);
+                    else {
+                        if (in(k, j)) t.x = p[0];
+                        if (in(k, j + 1)) t.y = p[1];
+                    }
+                    c[8 * g + 2 * k] = t.x;
+                    c[8 * g + 2 * k + 1] = t.y;
+                }
+            }
+        };
+        double cn[kOzWCols];
+        int fn[kOzWCols / 4];
+        load_c(0, cn, fn);
         for (int n = 0; n < nu; ++n) {
             const int hh = n & 1, j0 = unit(n) * kOzCols + hcol;
-            // columns j0 .. j0 + 15 of row i inside the lower triangle and outside the pivot block
-            const int jend = row_ok ? min(min(i + 1, md.ns), j0 + 16) : j0;
-            const bool whole = jend == j0 + 16 && (j0 + 16 <= k0 || j0 >= k0 + nb);
-            double c[16];
-            if (whole) {
+            double c[kOzWCols];
+            int f[kOzWCols / 4];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const double2 t = *reinterpret_cast<const double2*>(crow + j0 + 2 * q);
-                    c[2 * q] = t.x;
-                    c[2 * q + 1] = t.y;
-                }
-            } else {
+            for (int q = 0; q < kOzWCols; ++q) c[q] = cn[q];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int j = j0 + q;
-                    c[q] = (j < jend && (j < k0 || j >= k0 + nb)) ? crow[j] : 0.0;
-                }
+            for (int q = 0; q < kOzWCols / 4; ++q) f[q] = fn[q];
+            if (n + 1 < nu) {
+                load_c(n + 1, cn, fn);   // in flight while this unit is combined
             }
             const bool ok = oz_wait_or_abort(&tfull[hh], (uint32_t)(n >> 1) & 1u, &abort_flag);
             if (__any_sync(0xffffffffu, !ok)) {
@@ -657,30 +758,32 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
             }
             tc::fence_after_sync();
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {
+            for (int g = 0; g < kOzWCols / 8; ++g) {
                 uint32_t D[kOzS][8];
-                ld_classes(tmem + 256u * hh + ((uint32_t)(32 * (warp & 3)) << 16) + hcol + 8 * g, kOzCols, D);
-                if (g == 1) {   // the half is read: the next products may overwrite it
+                ld_classes_pairs(tmem + 256u * hh + ((uint32_t)(32 * (warp & 3)) << 16) + kOzWCols * (warp >> 2) + 8 * g,
+                                 kOzCols, D);
+                if (g == kOzWCols / 8 - 1) {   // the half is read: later products may overwrite it
                     tc::fence_before_sync();
                     __syncwarp();
                     if (lane == 0) oz_arrive(&tempty[hh]);
                 }
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int j = j0 + 8 * g + q;
-                    const int f = j < jend ? ecm[j] : 0;
-                    c[8 * g + q] = fma(join_classes(D, q), sgn * pow2(e + f - 56), c[8 * g + q]);
-                }
-            }
-            if (whole) {
+                for (int k = 0; k < 4; ++k) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<double2*>(crow + j0 + 2 * q) = make_double2(c[2 * q], c[2 * q + 1]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int j = j0 + q;
-                    if (j < jend && (j < k0 || j >= k0 + nb)) crow[j] = c[q];
+                    for (int u = 0; u < 2; ++u) {
+                        const double sc = pow2(e[k] + f[2 * g + u] - 56);   // its sign set without an FP64 operation
+                        c[8 * g + 2 * k + u] =
+                            fma(join_classes(D, 2 * k + u),
+                                __hiloint2double(__double2hiint(sc) ^ sg[k], __double2loint(sc)), c[8 * g + 2 * k + u]);
+                    }
+                    const int j = j0 + 8 * g;
+                    double* const p = crow + k * step + j;
+                    if (in(k, j) && in(k, j + 1))
+                        *reinterpret_cast<double2*>(p) = make_double2(c[8 * g + 2 * k], c[8 * g + 2 * k + 1]);
+                    else {
+                        if (in(k, j)) p[0] = c[8 * g + 2 * k];
+                        if (in(k, j + 1)) p[1] = c[8 * g + 2 * k + 1];
+                    }
                 }
             }
         }
