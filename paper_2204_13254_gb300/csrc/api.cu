@@ -1136,7 +1136,7 @@ int eliminate(dd_handle* h, bool coarse, cudaStream_t s) {
     const int n = coarse ? (int)h->corner_dof.size() : h->max_nr;
     const bool tensor = h->prm.factor_mode == DD_FACTOR_TENSOR;
     for (int k0 = 0; k0 < n; k0 += tensor ? kOzNB : kNB) {
-        Prof P(h, ST_FACTOR, s, 3);
+        Prof P(h, ST_FACTOR, s, tensor && k0 > 0 ? 2 : 3);
         const int rc = launch_sweep(h, coarse, k0, s);
         if (rc) return rc;
     }

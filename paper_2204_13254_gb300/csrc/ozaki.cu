@@ -227,7 +227,8 @@ __device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, 
 // and exponents.
 constexpr int kOzPivThreads = 256;
 constexpr int kPs = kOzK + 1;   // row stride in shared memory
-constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2));
+constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2)) + (3 * kOzK + 2) * sizeof(double) +
+                              (3 * kOzK + 1) * sizeof(int);
 
 // The sweep in type T; r [2][kOzK], t [kOzK], sinv [2], bad in shared memory (r and sinv by
 // step parity: a step's readers meet the next writers two barriers on).  False, in every
@@ -300,18 +301,19 @@ __device__ __forceinline__ bool gauss_jordan(T (&a)[4][4], T* r, T* t, T* sinv, 
     return *bad == 0;
 }
 
-__global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
-                                                            int k0, uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
-                                                            int32_t* __restrict__ status) {
-    const MatDesc md = mats[blockIdx.x];
-    if (k0 >= md.nr) return;
+// Threads 0 .. kOzPivThreads - 1 of the CTA (the others have exited); smem kOzPivSmem bytes.
+__device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restrict__ M, int m, int k0,
+                                            uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
+                                            int32_t* __restrict__ status, unsigned char* smem) {
     const int nb = min(kOzK, md.nr - k0);
-    extern __shared__ __align__(16) unsigned char smem[];
     double* Q = reinterpret_cast<double*>(smem);         // [kOzK][kPs] the block in full; then R in FP32
     int2* Pi = reinterpret_cast<int2*>(Q + kOzK * kPs);  // [kOzK][kPs] P, row i in units of 2^(rp_i - 57)
     int2* Xi = Pi + kOzK * kPs;                          // [kOzK][kPs] X, column j in units of 2^(cx_j - 57)
-    __shared__ double sw[2 * kOzK + kOzK + 2];           // the sweep's r, t, sinv
-    __shared__ int rp[kOzK], cx[kOzK], sd[kOzK], s_bad;
+    double* sw = reinterpret_cast<double*>(Xi + kOzK * kPs);   // the sweep's r, t, sinv
+    int* rp = reinterpret_cast<int*>(sw + 3 * kOzK + 2);
+    int* cx = rp + kOzK;
+    int* sd = cx + kOzK;
+    int* s_bad = sd + kOzK;
     double* A = M + md.moff + (int64_t)k0 * md.ld + k0;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int ri = tid >> 2, rq = tid & 3;   // (row, quarter of its 64 columns) for row maxima and slices
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
             for (int v = 0; v <= u; ++v)
                 f[u][v] = (float)scale2(a[u][v], -sd[ty + 16 * u] - sd[tx + 16 * v]);
         float* fs = reinterpret_cast<float*>(sw);
-        const bool ok = gauss_jordan(f, fs, fs + 2 * kOzK, fs + 3 * kOzK, &s_bad, nb, tid);
+        const bool ok = gauss_jordan(f, fs, fs + 2 * kOzK, fs + 3 * kOzK, s_bad, nb, tid);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
             if (swept) break;   // nothing to correct: the status says why, or the block is beyond FP64
             load();
             double(&ad)[4][4] = a;
-            if (!gauss_jordan(ad, sw, sw + 2 * kOzK, sw + 3 * kOzK, &s_bad, nb, tid) && tid == 0)
+            if (!gauss_jordan(ad, sw, sw + 2 * kOzK, sw + 3 * kOzK, s_bad, nb, tid) && tid == 0)
                 atomicCAS(status, 0, DD_ERR_NOT_SPD);
             swept = true;
             continue;
@@ -444,8 +446,8 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
     }
     // slices
     const int e = row_exp();
-    if (rq == 0) ep[(int64_t)blockIdx.x * kOzK + ri] = e;
-    unsigned char* out = reinterpret_cast<unsigned char*>(Ps) + (int64_t)blockIdx.x * kOzPBlock;
+    if (rq == 0) ep[(int64_t)m * kOzK + ri] = e;
+    unsigned char* out = reinterpret_cast<unsigned char*>(Ps) + (int64_t)m * kOzPBlock;
     for (int g = 0; g < 2; ++g) {
         const int k = 16 * rq + 8 * g;
         double v[8];
@@ -455,6 +457,16 @@ __global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __
             *reinterpret_cast<uint4*>(out + p * kOzPPiece + tc::kmajor_off(ri, k, kOzK)) = w;
         });
     }
+}
+
+// The first pivot block, one CTA per matrix; the later ones are formed by k_oz_update.
+__global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
+                                                               uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
+                                                               int32_t* __restrict__ status) {
+    const MatDesc md = mats[blockIdx.x];
+    if (md.nr <= 0) return;
+    extern __shared__ __align__(16) unsigned char smem[];
+    pivot_block(md, M, (int)blockIdx.x, 0, Ps, ep, status, smem);
 }
 
 // ---- panel -------------------------------------------------------------------
@@ -600,28 +612,40 @@ constexpr int kOzStages = 4;
 constexpr int kOzThreads = 288;
 constexpr int kOzWCols = 16;   // columns of a unit per warp
 constexpr size_t kOzSmem = kOzBlock + kOzStages * kOzUnit + (1 + 2 * kOzStages + 4) * sizeof(uint64_t) + 16;
-static_assert(kOzSmem <= 227 * 1024, "shared memory of the update");
+static_assert(kOzSmem <= 227 * 1024 && kOzPivSmem <= kOzBlock, "shared memory of the update");
 
 __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __restrict__ mats, double* __restrict__ M,
                                                              int k0, int nrb, const uint16_t* __restrict__ Bs,
                                                              const uint16_t* __restrict__ Cs,
                                                              const int32_t* __restrict__ eb,
                                                              const int32_t* __restrict__ ec, int nmax,
+                                                             uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
+                                                             int nm, int runs, int32_t* __restrict__ status,
                                                              int32_t* __restrict__ err) {
-    const int m = blockIdx.y;
+    const bool ahead = (int)blockIdx.x < nm;
+    const int m = ahead ? (int)blockIdx.x : ((int)blockIdx.x - nm) / runs;
     const MatDesc md = mats[m];
-    // blockIdx.x -> (row block, run): row block rb has ceil(4 (rb + 1) / kOzRun) runs
-    int rb = 0, run = (int)blockIdx.x;
-    for (;;) {
-        const int nrun = (4 * (rb + 1) + kOzRun - 1) / kOzRun;
-        if (run < nrun) break;
-        run -= nrun;
-        ++rb;
-    }
-    if (k0 >= md.nr || rb * kOzRows >= md.ns) return;
+    if (k0 >= md.nr) return;
     const int nb = min(kOzK, md.nr - k0);
-    const int u0 = run * kOzRun;
-    const int u1 = min(min(u0 + kOzRun, 4 * (rb + 1)), (md.ns + kOzCols - 1) / kOzCols);
+    const int k1 = k0 + kOzK, nb1 = max(0, min(kOzK, md.nr - k1));   // the next pivot block
+    int rb = 0, u0, u1;
+    if (ahead) {
+        if (nb1 == 0) return;
+        rb = k1 / kOzRows;
+        u0 = k1 / kOzCols;
+        u1 = u0 + (nb1 + kOzCols - 1) / kOzCols;
+    } else {   // (row block, run): row block rb has ceil(4 (rb + 1) / kOzRun) runs
+        int run = ((int)blockIdx.x - nm) % runs;
+        for (;;) {
+            const int nrun = (4 * (rb + 1) + kOzRun - 1) / kOzRun;
+            if (run < nrun) break;
+            run -= nrun;
+            ++rb;
+        }
+        if (rb * kOzRows >= md.ns) return;
+        u0 = run * kOzRun;
+        u1 = min(min(u0 + kOzRun, 4 * (rb + 1)), (md.ns + kOzCols - 1) / kOzCols);
+    }
     // units inside the pivot block are left out
     const int s0 = k0 / kOzCols, s1 = (k0 + nb) / kOzCols;   // units [s0, s1) lie wholly in it
     auto unit = [&](int n) {   // the n-th unit of the run
@@ -711,9 +735,10 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + 8 * k;
-            const bool row_ok = i < md.ns && (i < k0 || i >= k0 + nb);
+            const bool next = i >= k1 && i < k1 + nb1;   // rows of the next pivot block
+            const bool row_ok = ahead ? next : i < md.ns && (i < k0 || i >= k0 + nb);
             e[k] = row_ok ? eb[(int64_t)m * nmax + i] : 0;
-            jend[k] = row_ok ? i + 1 : 0;
+            jend[k] = row_ok ? (next && !ahead ? k1 : i + 1) : 0;
             sg[k] = i < k0 ? (int)0x80000000 : 0;
         }
         auto in = [&](int k, int j) { return j < jend[k] && (j < k0 || j >= k0 + nb); };
@@ -799,6 +824,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
     __syncthreads();
     tc::fence_after_sync();
     if (warp == 0) tc::tmem_free(tmem, 512);
+    if (!ahead || abort_flag || warp == 8) return;
+    pivot_block(md, M, m, k1, Ps, ep, status, sm);   // written by this CTA, before the barrier above
 }
 
 // M[i][j] for j > i from the lower triangle: -M[j][i] when exactly one index was swept
@@ -846,7 +873,8 @@ OzLayout oz_layout(int nm, int nmax) {
 
 size_t oz_bytes(int nm, int nmax) { return oz_layout(nm, std::max(nmax, 1)).total; }
 
-// One pivot block [k0, k0 + 64) of the sweep of nm matrices (of at most nmax rows).
+// One pivot block [k0, k0 + 64) of the sweep of nm matrices (of at most nmax rows), and the
+// inverse of the next one; called for k0 = 0, 64, ... in turn.
 int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, unsigned char* ws, int32_t* status,
                     int32_t* err, void* stream) {
     const int nrb = (nmax + kOzRows - 1) / kOzRows;
@@ -861,12 +889,13 @@ int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, un
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_oz_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_oz_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzPivSmem);
     if (e != cudaSuccess) return (int)e;
-    k_oz_pivot<<<(unsigned)nm, kOzPivThreads, kOzPivSmem, S(stream)>>>(mats, M, k0, Ps, ep, status);
+    if (k0 == 0) k_oz_pivot<<<(unsigned)nm, kOzPivThreads, kOzPivSmem, S(stream)>>>(mats, M, Ps, ep, status);
     k_oz_panel<<<dim3((unsigned)nrb, (unsigned)nm), kOzPanThreads, kOzPanSmem, S(stream)>>>(mats, M, k0, nrb, Ps, ep, Bs,
                                                                                             eb, Cs, ec, nmax, err);
     unsigned runs = 0;
     for (int rb = 0; rb < nrb; ++rb) runs += (unsigned)((4 * (rb + 1) + kOzRun - 1) / kOzRun);
-    k_oz_update<<<dim3(runs, (unsigned)nm), kOzThreads, kOzSmem, S(stream)>>>(mats, M, k0, nrb, Bs, Cs, eb, ec, nmax, err);
+    k_oz_update<<<(unsigned)nm * (1 + runs), kOzThreads, kOzSmem, S(stream)>>>(mats, M, k0, nrb, Bs, Cs, eb, ec, nmax, Ps,
+                                                                              ep, nm, (int)runs, status, err);
     return (int)cudaGetLastError();
 }
 
