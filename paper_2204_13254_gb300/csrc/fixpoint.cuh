@@ -15,8 +15,9 @@ __device__ __forceinline__ int exp_of_hi(int hi) {
     const int f = hi >> 20;
     return f == 0 ? 0 : f - 1022;
 }
+__device__ __forceinline__ double pow2n(int x) { return __hiloint2double((x + 1023) << 20, 0); }   // |x| <= 1022
 __device__ __forceinline__ double pow2(int x) {
-    if (x > -1023 && x < 1024) return __longlong_as_double((long long)(x + 1023) << 52);
+    if (x > -1023 && x < 1024) return pow2n(x);
     return ldexp(1.0, x);
 }
 // v 2^x without an intermediate overflow of the factor.
@@ -24,12 +25,12 @@ __device__ __forceinline__ double scale2(double v, int x) {
     if (x > -1000 && x < 1000) return v * pow2(x);
     return ldexp(v, x);
 }
-// Integer of v 2^x (|v| 2^x <= 2^57) in its two words.
-__device__ __forceinline__ int2 split57(double v, int x) {
-    const long long t = __double2ll_rn(scale2(v, x));
+// The two words of an integer |t| <= 2^57, and of v 2^x.
+__device__ __forceinline__ int2 split57(long long t) {
     const int hi = (int)((t + (1ll << (kLow - 1))) >> kLow);
     return make_int2(hi, (int)(t - ((long long)hi << kLow)));
 }
+__device__ __forceinline__ int2 split57(double v, int x) { return split57(__double2ll_rn(scale2(v, x))); }
 
 // acc += a b, one 32 x 32 + 64 bit multiply-add.
 __device__ __forceinline__ void imad(long long& acc, int a, int b) {

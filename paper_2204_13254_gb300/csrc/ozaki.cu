@@ -227,78 +227,97 @@ __device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, 
 // and exponents.
 constexpr int kOzPivThreads = 256;
 constexpr int kPs = kOzK + 1;   // row stride in shared memory
-constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2)) + (3 * kOzK + 2) * sizeof(double) +
-                              (3 * kOzK + 1) * sizeof(int);
 
-// The sweep in type T; r [2][kOzK], t [kOzK], sinv [2], bad in shared memory (r and sinv by
-// step parity: a step's readers meet the next writers two barriers on).  False, in every
-// thread, if a pivot was not positive (it counts as 1 then).
-template <typename T>
-__device__ __forceinline__ bool gauss_jordan(T (&a)[4][4], T* r, T* t, T* sinv, int* bad, int nb, int tid) {
+// The FP32 sweep, the inverse in place: thread (ty, tx) holds elements (ty + 16 u, 4 tx + v) of
+// the full square.  Step k publishes row and column k and the pivot d; with p = 1 / d and the
+// pivot's own entries published as d + 1 (row) and d - 1 (column), a_ij -= c_i (r_j p) is the
+// whole exchange, row and column k included (d < 1 by the scaling, so 1 +- d costs no accuracy).
+// buf [2][kSwBuf] by step parity, so that one barrier a step is enough (a step's readers meet
+// the next writers of its half one barrier on).  The reciprocal may be approximate, as the
+// result is corrected.  One loop body and no selection by register index: the code is run
+// once per launch, and with bodies unrolled over the registers its instruction fetches beside
+// the update took longer than the steps.  False, in every thread, if a pivot was not positive.
+constexpr int kSwBuf = 2 * kOzK + 4;
+constexpr size_t kOzPivSmem = kOzK * kPs * (sizeof(double) + 2 * sizeof(int2)) + 2 * kSwBuf * sizeof(float) + 3 * kOzK * sizeof(int);
+__device__ __forceinline__ bool sweep32(float (&a)[4][4], float* buf, int nb, int tid) {
     const int tx = tid & 15, ty = tid >> 4;
-    if (tid == 0) *bad = 0;
+    bool good = true;
+#pragma unroll 1
     for (int k = 0; k < nb; ++k) {
-        T* rk = r + (k & 1) * kOzK;
-        const int uk = k >> 4, kk = k & 15;
-        // publish row k (j < k) and column k (i > k), and 1 / d
-        if (ty == kk) {
+        float* row = buf + (k & 1) * kSwBuf;
+        float* col = row + kOzK;
+        if (ty == (k & 15)) {
+            const int uk = k >> 4;
+            float4 w = make_float4(a[0][0], a[0][1], a[0][2], a[0][3]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    if (u != uk) continue;
-                    const int j = tx + 16 * v;
-                    if (j < k) rk[j] = a[u][v];
-                    if (j == k) {
-                        T d = a[u][v];
-                        if (!(d > (T)0) || !isfinite(d)) {
-                            *bad = 1;
-                            d = (T)1;
-                        }
-                        sinv[k & 1] = (T)1 / d;
-                    }
-                }
+            for (int u = 1; u < 4; ++u)
+                if (uk == u) w = make_float4(a[u][0], a[u][1], a[u][2], a[u][3]);
+            *reinterpret_cast<float4*>(row + 4 * tx) = w;
         }
-        if (tx == kk) {
+        if (tx == (k >> 2)) {
+            const int q = k & 3;
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    if (v != uk) continue;
-                    const int i = ty + 16 * u;
-                    if (i > k) rk[i] = a[u][v];
+            for (int u = 0; u < 4; ++u) {
+                const float x = q < 2 ? (q == 0 ? a[u][0] : a[u][1]) : (q == 2 ? a[u][2] : a[u][3]);
+                const bool own = ty + 16 * u == k;
+                col[ty + 16 * u] = own ? x - 1.0f : x;
+                if (own) {
+                    row[k] = x + 1.0f;
+                    col[kOzK] = x;
                 }
+            }
         }
         __syncthreads();
-        if (tid < kOzK) t[tid] = tid == k ? (T)0 : rk[tid] * sinv[k & 1];
-        __syncthreads();
-        T sr[4], tj[4];
+        float d = col[kOzK];
+        if (!(d > 0.0f) || !isfinite(d)) {
+            good = false;
+            d = 1.0f;
+        }
+        const float p = __fdividef(1.0f, d);
+        const float4 r = *reinterpret_cast<const float4*>(row + 4 * tx);
+        const float rp[4] = {r.x * p, r.y * p, r.z * p, r.w * p};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = ty + 16 * u, j = tx + 16 * u;
-            sr[u] = i == k ? (T)0 : (i < k ? -rk[i] : rk[i]);
-            tj[u] = t[j];
-        }
+            const float c = col[ty + 16 * u];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v <= u; ++v) a[u][v] = fma(-sr[u], tj[v], a[u][v]);
-        // row and column k of the swept matrix
-        if (ty == kk || tx == kk) {
-            const T inv = sinv[k & 1];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) {
-                    const int i = ty + 16 * u, j = tx + 16 * v;
-                    if (i == k && j == k) a[u][v] = inv;
-                    else if (i == k && j < k) a[u][v] = -t[j];
-                    else if (j == k && i > k) a[u][v] = t[i];
-                }
+            for (int v = 0; v < 4; ++v) a[u][v] = fmaf(-c, rp[v], a[u][v]);
         }
     }
     __syncthreads();
-    return *bad == 0;
+    return good;
+}
+
+// The FP64 sweep, for the blocks that the FP32 one leaves: the same in shared memory, Q [.][kPs].
+__device__ __forceinline__ bool sweep64(double* Q, int nb, int tid) {
+    const int tx = tid & 15, ty = tid >> 4;
+    bool good = true;
+    for (int k = 0; k < nb; ++k) {
+        double d = Q[k * kPs + k];
+        if (!(d > 0.0) || !isfinite(d)) {
+            good = false;
+            d = 1.0;
+        }
+        const double p = 1.0 / d;
+        double r[4], c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            r[u] = Q[k * kPs + tx + 16 * u] * p;
+            c[u] = Q[(ty + 16 * u) * kPs + k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = ty + 16 * u;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int j = tx + 16 * v;
+                double* q = Q + i * kPs + j;
+                *q = i == k ? (j == k ? p : r[v]) : (j == k ? -c[u] * p : fma(-c[u], r[v], *q));
+            }
+        }
+        __syncthreads();
+    }
+    return good;
 }
 
 // Threads 0 .. kOzPivThreads - 1 of the CTA (the others have exited); smem kOzPivSmem bytes.
@@ -309,14 +328,15 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
     double* Q = reinterpret_cast<double*>(smem);         // [kOzK][kPs] the block in full; then R in FP32
     int2* Pi = reinterpret_cast<int2*>(Q + kOzK * kPs);  // [kOzK][kPs] P, row i in units of 2^(rp_i - 57)
     int2* Xi = Pi + kOzK * kPs;                          // [kOzK][kPs] X, column j in units of 2^(cx_j - 57)
-    double* sw = reinterpret_cast<double*>(Xi + kOzK * kPs);   // the sweep's r, t, sinv
-    int* rp = reinterpret_cast<int*>(sw + 3 * kOzK + 2);
+    float* sw = reinterpret_cast<float*>(Xi + kOzK * kPs);   // the sweep's rows and columns
+    int* rp = reinterpret_cast<int*>(sw + 2 * kSwBuf);
     int* cx = rp + kOzK;
     int* sd = cx + kOzK;
-    int* s_bad = sd + kOzK;
     double* A = M + md.moff + (int64_t)k0 * md.ld + k0;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int ri = tid >> 2, rq = tid & 3;   // (row, quarter of its 64 columns) for row maxima and slices
+    // the k-th column of the quarter, rotated so that a half warp's 16 elements lie in 16 bank pairs
+    auto qc = [&](int k) { return 16 * rq + ((k + 4 * rq) & 15); };
     double a[4][4];
     auto load = [&]() {
 #pragma unroll
@@ -324,7 +344,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 #pragma unroll
             for (int v = 0; v <= u; ++v) {
                 const int i = ty + 16 * u, j = tx + 16 * v;
-                a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : (i == j ? 1.0 : 0.0);
+                a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : 0.0;
             }
     };
     // the lower triangle in registers -> the full symmetric block in Q (zero outside nb)
@@ -343,33 +363,63 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
     };
     auto row_exp = [&]() {   // exponent of the largest element of row ri (all four lanes of the row)
         int mx = 0;
-        for (int k = 0; k < 16; ++k) mx = max(mx, __double2hiint(Q[ri * kPs + 16 * rq + k]) & 0x7fffffff);
+        for (int k = 0; k < 16; ++k) mx = max(mx, __double2hiint(Q[ri * kPs + qc(k)]) & 0x7fffffff);
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         return exp_of_hi(mx);
+    };
+    // row ri of Q in 57-bit units of 2^(e - 57), handed to put(column, words)
+    auto split_row = [&](int e, auto put) {
+        const int x = kBits - e;
+        if (x > -1000 && x < 1000) {   // (scale2's range, outside the loop)
+            const double f = pow2(x);
+#pragma unroll 4
+            for (int k = 0; k < 16; ++k) put(qc(k), split57(__double2ll_rn(Q[ri * kPs + qc(k)] * f)));
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < 16; ++k) put(qc(k), split57(Q[ri * kPs + qc(k)], x));
+        }
     };
     load();
     spread();
     {
         const int e = row_exp();
         rp[ri] = e;
-        for (int k = 0; k < 16; ++k) Pi[ri * kPs + 16 * rq + k] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
-        if (rq == 0) sd[ri] = ri < nb ? (exp_of_hi(__double2hiint(Q[ri * kPs + ri]) & 0x7fffffff) + 1) >> 1 : 0;
+        split_row(e, [&](int c, int2 w) { Pi[ri * kPs + c] = w; });
+        sd[ri] = ri < nb ? (exp_of_hi(__double2hiint(Q[ri * kPs + ri]) & 0x7fffffff) + 1) >> 1 : 0;
     }
-    __syncthreads();
-    {   // X = D (D P D)^-1 D with D = diag(2^-sd)
+    // X = D (D P D)^-1 D with D = diag(2^-sd); zero, so that the FP64 sweep follows, where an
+    // exponent is far out or a pivot was not positive
+    const int far = __syncthreads_or(abs(sd[ri]) > 500);
+    float* F = reinterpret_cast<float*>(Xi);   // [kOzK][kPs]
+    if (!far) {
         float f[4][4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v <= u; ++v)
-                f[u][v] = (float)scale2(a[u][v], -sd[ty + 16 * u] - sd[tx + 16 * v]);
-        float* fs = reinterpret_cast<float*>(sw);
-        const bool ok = gauss_jordan(f, fs, fs + 2 * kOzK, fs + 3 * kOzK, s_bad, nb, tid);
+            for (int v = 0; v < 4; ++v) {
+                const int i = ty + 16 * u, j = 4 * tx + v;
+                f[u][v] = (float)(Q[i * kPs + j] * pow2n(-sd[i] - sd[j]));
+                if (i == j && i >= nb) f[u][v] = 1.0f;
+            }
+        const bool ok = sweep32(f, sw, nb, tid);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v <= u; ++v) a[u][v] = ok ? scale2((double)f[u][v], -sd[ty + 16 * u] - sd[tx + 16 * v]) : 0.0;
+            for (int v = 0; v < 4; ++v) F[(ty + 16 * u) * kPs + 4 * tx + v] = ok ? f[u][v] : 0.0f;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v;
+                a[u][v] = (double)F[i * kPs + j] * pow2n(-sd[i] - sd[j]);
+            }
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) a[u][v] = 0.0;
     }
     bool swept = false;   // in FP64
     for (int pass = 0; pass < 4; ++pass) {
@@ -377,7 +427,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
         {
             const int e = row_exp();   // X is symmetric: also its column exponent
             cx[ri] = e;
-            for (int k = 0; k < 16; ++k) Xi[(16 * rq + k) * kPs + ri] = split57(Q[ri * kPs + 16 * rq + k], kBits - e);
+            split_row(e, [&](int c, int2 w) { Xi[c * kPs + ri] = w; });
         }
         __syncthreads();
         // R = I - P X: 64 products per element fit the accumulators
@@ -400,40 +450,51 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
         for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                const int i = ty + 16 * u, j = tx + 16 * v, sh = 2 * kBits - kLow - rp[i] - cx[j];   // 1 in the sums' units
-                __int128 d = -(((__int128)hh[u][v] << kLow) + xx[u][v]);
-                float f = 0.0f;
-                if (i < nb && j < nb) {
-                    if (sh < 40 || sh > 120) {
-                        big = 2;
-                    } else {
-                        if (i == j) d += (__int128)1 << sh;
-                        const __int128 m = d < 0 ? -d : d;
-                        if (m >= (__int128)1 << (sh - 5)) big = 2;
-                        else if (m >= (__int128)1 << (sh - 34)) big = max(big, 1);
-                        f = (float)(long long)(d >> (sh > 60 ? sh - 60 : 0)) * exp2f(-(float)(sh > 60 ? 60 : sh));
-                    }
-                }
+                // the sums hold P X in units of 2^-sh; the 1 is taken off before the low words join
+                const int i = ty + 16 * u, j = tx + 16 * v, sh = 2 * kBits - kLow - rp[i] - cx[j];
+                const bool one = u == v && tx == ty && i < nb;
+                const bool fit = sh >= 40 && sh <= (one ? kLow + 62 : 120);
+                const long long t = (one && fit ? 1ll << (sh - kLow) : 0ll) - hh[u][v] - (xx[u][v] >> kLow);
+                const float lo = (float)((int)xx[u][v] & ((1 << kLow) - 1)) * (1.0f / (1 << kLow));
+                const float f = fit ? ((float)t - lo) * __int_as_float((127 + kLow - sh) << 23) : 0.0f;
+                const float g = fabsf(f);
+                if (i < nb && j < nb) big = max(big, !fit || g >= 0x1p-5f ? 2 : g >= 0x1p-34f ? 1 : 0);
                 R[i * kPs + j] = f;   // (every thread is done with Q)
             }
         const int any2 = __syncthreads_or(big == 2), any1 = __syncthreads_or(big >= 1);
         if (any2) {
             if (swept) break;   // nothing to correct: the status says why, or the block is beyond FP64
             load();
-            double(&ad)[4][4] = a;
-            if (!gauss_jordan(ad, sw, sw + 2 * kOzK, sw + 3 * kOzK, s_bad, nb, tid) && tid == 0)
-                atomicCAS(status, 0, DD_ERR_NOT_SPD);
+            spread();
+            if (!sweep64(Q, nb, tid) && tid == 0) atomicCAS(status, 0, DD_ERR_NOT_SPD);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) a[u][v] = Q[(ty + 16 * u) * kPs + tx + 16 * v];
+            __syncthreads();
             swept = true;
             continue;
+        }
+        float y[4][4] = {};   // (X R) in units of 2^(cx_i - 28) X's
+#pragma unroll 8
+        for (int k = 0; k < kOzK; ++k) {
+            float x[4], r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x[u] = (float)Xi[k * kPs + ty + 16 * u].x;
+                r[u] = R[k * kPs + tx + 16 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) y[u][v] = fmaf(x[u], r[v], y[u][v]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int v = 0; v <= u; ++v) {
                 const int i = ty + 16 * u, j = tx + 16 * v;
-                float s = 0.0f;
-                for (int k = 0; k < nb; ++k) s = fmaf((float)Xi[k * kPs + i].x, R[k * kPs + j], s);
-                if (i < nb && j <= i) a[u][v] += (double)s * pow2(cx[i] - (kBits - kLow));
+                if (i < nb && j <= i) a[u][v] += (double)y[u][v] * pow2(cx[i] - (kBits - kLow));
             }
         __syncthreads();
         if (!any1) break;
@@ -460,7 +521,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 }
 
 // The first pivot block, one CTA per matrix; the later ones are formed by k_oz_update.
-__global__ void __launch_bounds__(kOzPivThreads, 2) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
+__global__ void __launch_bounds__(kOzPivThreads, 1) k_oz_pivot(const MatDesc* __restrict__ mats, double* __restrict__ M,
                                                                uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
                                                                int32_t* __restrict__ status) {
     const MatDesc md = mats[blockIdx.x];
