@@ -210,19 +210,20 @@ __device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, 
 // ---- pivot block -------------------------------------------------------------
 // P^-1 of the pivot block, one CTA per matrix.
 //  * A first X by a Gauss-Jordan sweep in FP32 (SPD: no pivoting; the block scaled by powers of
-//    two to a diagonal in [1/4, 1)) over the lower triangle in registers: thread (ty, tx) of
-//    16 x 16 holds elements (ty + 16 u, tx + 16 v), v <= u.  Step k publishes the vector r (row
-//    k left of the diagonal, column k below it) and 1 / d; then P_ij -= (s_i r_i) (r_j / d).
-//  * Newton: R = I - P X from exact 57-bit fixed-point sums, X += X R in FP32, until |R| was
-//    below 2^-34 (twice as a rule: 2^-19, then 2^-38): X ends at its own FP64 rounding.
-//  * Where the FP32 sweep meets a pivot that is not positive or leaves |R| >= 2^-5, the sweep
-//    is done in FP64 (it decides whether the matrix is positive definite) and corrected once.
-// The FP64 sweep is 64 steps of ten FMAs per thread, FP64-ALU bound at 124 us per block; with
-// one correction 173 us, in FP32 with two corrections 147 us (40 matrices).  Its 64
-// roundings per element would be the largest error of the elimination (the products are
-// exact to 2^-54).  Measured, coupled operator against an extended-precision reference, seven
-// meshes (six bisected into 139 to 600 uneven subdomains): 2.3e-16 .. 3.8e-16; with the FP64
-// sweep alone 2.9e-16 .. 4.5e-16, with 32-wide pivot blocks in plain FP64 2.5e-16 .. 4.0e-16.
+//    two to a diagonal in [1/4, 1)).
+//  * Newton: R = I - P X from exact 57-bit fixed-point sums, X += X R in FP32, twice as a rule (|R| is 2^-20,
+//    then 2^-41): X ends at its own FP64 rounding.
+//  * A block that FP32 does not serve (a pivot that is not positive, |R| >= 2^-5, or >= 2^-36 at
+//    the second look: the contraction is 2^-24 of the condition number) is swept in FP64 and
+//    taken as swept, in full: its errors are those of a nearby block, which cancel in the
+//    panels, while with growing condition number a rounded symmetric X loses more and more of
+//    it (measured, coupled operator, condition number of A_rr 3e3: 3e-13 and 2e-12).
+// With the FP64 sweep for every block, and one correction, 173 us (its FMAs alone 124 us: the
+// FP64 pipe), with this 76 us (40 matrices).  The sweep's 64 roundings per element would be the
+// largest error of a well-conditioned elimination (the products are exact to 2^-54).  Measured,
+// coupled operator against an extended-precision reference, seven meshes (six bisected into
+// 139 to 600 uneven subdomains): 2.3e-16 .. 3.8e-16; with the FP64 sweep alone 2.9e-16 ..
+// 4.5e-16, with 32-wide pivot blocks in plain FP64 2.5e-16 .. 4.0e-16.
 // Writes P^-1 back into M[p, p] (the panel kernel does not read that block), and its slices
 // and exponents.
 constexpr int kOzPivThreads = 256;
@@ -421,8 +422,8 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 #pragma unroll
             for (int v = 0; v <= u; ++v) a[u][v] = 0.0;
     }
-    bool swept = false;   // in FP64
-    for (int pass = 0; pass < 4; ++pass) {
+    bool swept = false;   // in FP64, X in Q
+    for (int pass = 0; pass < 2; ++pass) {
         spread();
         {
             const int e = row_exp();   // X is symmetric: also its column exponent
@@ -445,7 +446,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 #pragma unroll
                 for (int v = 0; v < 4; ++v) mac(hh[u][v], xx[u][v], p[u].x, p[u].y, x[v].x, x[v].y);
         }
-        int big = 0;   // 2: |R| >= 2^-5 (or exponents out of range), 1: |R| >= 2^-34
+        int big = 0;   // 2: |R| >= 2^-5 (or exponents out of range), 1: |R| >= 2^-36
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -458,22 +459,16 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
                 const float lo = (float)((int)xx[u][v] & ((1 << kLow) - 1)) * (1.0f / (1 << kLow));
                 const float f = fit ? ((float)t - lo) * __int_as_float((127 + kLow - sh) << 23) : 0.0f;
                 const float g = fabsf(f);
-                if (i < nb && j < nb) big = max(big, !fit || g >= 0x1p-5f ? 2 : g >= 0x1p-34f ? 1 : 0);
+                if (i < nb && j < nb) big = max(big, !fit || g >= 0x1p-5f ? 2 : g >= 0x1p-36f ? 1 : 0);
                 R[i * kPs + j] = f;   // (every thread is done with Q)
             }
         const int any2 = __syncthreads_or(big == 2), any1 = __syncthreads_or(big >= 1);
-        if (any2) {
-            if (swept) break;   // nothing to correct: the status says why, or the block is beyond FP64
+        if (any2 || (any1 && pass == 1)) {
             load();
             spread();
             if (!sweep64(Q, nb, tid) && tid == 0) atomicCAS(status, 0, DD_ERR_NOT_SPD);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v <= u; ++v) a[u][v] = Q[(ty + 16 * u) * kPs + tx + 16 * v];
-            __syncthreads();
             swept = true;
-            continue;
+            break;
         }
         float y[4][4] = {};   // (X R) in units of 2^(cx_i - 28) X's
 #pragma unroll 8
@@ -499,8 +494,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
         __syncthreads();
         if (!any1) break;
     }
-    __syncthreads();
-    spread();
+    if (!swept) spread();
     for (int p = tid; p < kOzK * kOzK; p += kOzPivThreads) {
         const int i = p >> 6, j = p & 63;
         if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i * kPs + j];
