@@ -345,7 +345,8 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
         L.take(d.zu, (size_t)nu);
         L.take(d.zuf, (size_t)nu);
         L.take(d.gs, 1);
-        L.take(d.gpart, (size_t)(kMaxRestart + 1) * (size_t)h->gm_blocks);
+        L.take(d.gpart, std::max((size_t)(kMaxRestart + 1) * (size_t)h->gm_blocks,
+                                 2 * (size_t)(kMaxRestart + 2) * (size_t)kGmStepBlocks));
     }
     L.take(d.delta, nd);
     L.take(d.delta_k, nd);
@@ -627,7 +628,13 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
             Prof P(h, ST_SCHUR, st, 1);
             CK(h, launch_gemv(h, GEMV_COUPLED, prec, xs_z, go, false, st, skip), "coupled operator");
         }
-        Prof P(h, ST_VEC, st, 3);
+        {
+            Prof P(h, ST_VEC, st, 1);
+            bool whole = false;
+            CK(h, launch_gm_step(h, U, V.wf, zuf, cond_inner, &whole, st), "gmres step");
+            if (whole) return DD_OK;
+        }
+        Prof P(h, ST_VEC, st, 2);
         CK(h, launch_gm_pass(h, U, 0, V.wf, zuf, 0ull, st), "gmres pass 0");
         CK(h, launch_gm_pass(h, U, 1, V.wf, zuf, cond_inner, st), "gmres pass 1");
         CK(h, launch_gm_normalize(h, U, zuf, st), "gmres normalize");

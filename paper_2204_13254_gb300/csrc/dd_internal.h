@@ -233,6 +233,7 @@ constexpr int kTlW = 2;           // u32 words per tile-list entry (a << 16 | b 
 #endif
 constexpr int kGmElems = DD_GM_ELEMS;                // vector elements per thread in the GMRES kernels
 constexpr int kGmChunk = kGmElems * 256;             // elements per block
+constexpr int kGmStepBlocks = 256;                   // most CTAs of the one-kernel Arnoldi step
 
 // Device state of the restarted GMRES of the coupled system (one struct in the
 // workspace).  The control words come first: eager mode reads them back.
@@ -689,6 +690,8 @@ int launch_gm_init(const dd_handle* h, double tol, int max_it, int m, int adapti
 int launch_gm_start(const dd_handle* h, const UView& U, int have_q, const float* wf, unsigned long long cond_inner,
                     void* stream);
 int launch_gm_normalize(const dd_handle* h, const UView& U, float* zuf, void* stream);
+int launch_gm_step(const dd_handle* h, const UView& U, const float* wf, float* zuf, unsigned long long cond_inner,
+                   bool* ran, void* stream);
 int launch_gm_pass(const dd_handle* h, const UView& U, int phase, const float* wf, const float* zuf,
                    unsigned long long cond_inner, void* stream);
 int launch_gm_update(const dd_handle* h, const UView& U, unsigned long long cond_outer, void* stream);
