@@ -464,6 +464,19 @@ int apply_schur_w(dd_handle* h, int prec, int kind, const double* v, const doubl
                        check_done, s);
 }
 
+// The vectors of one CG iteration.
+int pcg_vectors(dd_handle* h, const Vecs& V, unsigned long long cond, cudaStream_t s) {
+    {
+        Prof P(h, ST_VEC, s, 1);
+        bool whole = false;
+        const int rc = launch_pcg_step(h, V.wf, V.pf, V.zf, V.lamf, cond, &whole, s);
+        if (rc || whole) return rc;
+    }
+    Prof P(h, ST_VEC, s, 1);
+    const int rc = launch_pcg_alpha(h, V.wf, V.pf, s);
+    return rc ? rc : launch_pcg_update(h, V.zf, V.lamf, cond, s);
+}
+
 // Adds n full-work CG iterations to the stage counters once the count is known.
 void count_cg_work(dd_handle* h, int prec, int n) {
     const bool c = !h->corner_dof.empty();
@@ -870,10 +883,7 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
             int brc = DD_OK;
             for (int k = 0; k < h->prm.chunk && brc == DD_OK; ++k) {
                 brc = apply_schur_w(h, prec, X_PCG, h->d.z, h->d.p, V.zf, V.pf, true, bs);
-                if (brc) break;
-                Prof P(h, ST_VEC, bs, 2);
-                brc = launch_pcg_alpha(h, V.wf, V.pf, bs);
-                if (!brc) brc = launch_pcg_update(h, V.zf, V.lamf, (unsigned long long)hc, bs);
+                if (!brc) brc = pcg_vectors(h, V, (unsigned long long)hc, bs);
             }
             cudaGraph_t out_body;
             const int erc = (int)cudaStreamEndCapture(bs, &out_body);
@@ -897,9 +907,7 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
             const int n = std::min(h->prm.chunk, h->prm.max_it - hs.it);
             for (int k = 0; k < n; ++k) {
                 CK(h, apply_schur_w(h, prec, X_PCG, h->d.z, h->d.p, V.zf, V.pf, true, s), "apply");
-                Prof P(h, ST_VEC, s, 2);
-                CK(h, launch_pcg_alpha(h, V.wf, V.pf, s), "pcg alpha");
-                CK(h, launch_pcg_update(h, V.zf, V.lamf, 0ull, s), "pcg update");
+                CK(h, pcg_vectors(h, V, 0ull, s), "pcg vectors");
             }
             CK(h, read_scalars(h, &hs, s), "pcg scalars");
         }

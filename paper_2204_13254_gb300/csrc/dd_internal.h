@@ -637,6 +637,8 @@ int launch_step_begin(const dd_handle* h, void* stream);
 int launch_extrapolate(const dd_handle* h, bool f32, void* stream);
 int launch_solve_end(const dd_handle* h, void* stream);
 int launch_refine_cond(const dd_handle* h, unsigned long long cond, void* stream);
+int launch_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, float* lamf, unsigned long long cond,
+                    bool* ran, void* stream);
 int launch_pcg_alpha(const dd_handle* h, const float* wf, float* pf, void* stream);
 int launch_pcg_update(const dd_handle* h, float* zf, float* lamf, unsigned long long cond, void* stream);
 int launch_writeback(const dd_handle* h, const double* e_n, const double* e_nm1, double* delta_k, double* delta_acc,

@@ -34,6 +34,7 @@
 #include <algorithm>
 
 #include "dd_internal.h"
+#include "gridbar.cuh"
 
 namespace {
 
@@ -556,28 +557,6 @@ __global__ void __launch_bounds__(kT) k_gm_pass(UView U, const double* __restric
 // cycle of 20): FP32 136,000 unknowns 25.8 -> 15.9 us, FP64 64 -> 35 us, FP64 40,000 unknowns
 // 35 -> 18 us.  256 threads with twice the elements: 19.0 us FP32, 43 us FP64; 1,024 with half
 // of them: 16.7 us FP32.
-constexpr unsigned kStepPolls = 1u << 19;   // of one barrier wait (about half a second)
-
-// Grid barrier at a counter that is zero at its first arrival; false, in every thread, when it
-// gave up (then *err is set).
-__device__ bool step_barrier(uint32_t* ctr, int32_t* err, int* failed) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(ctr, 1u);
-        unsigned k = 0;
-        uint32_t v;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-        } while (v < gridDim.x && ++k < kStepPolls);
-        *failed = v < gridDim.x;
-        if (*failed) atomicExch(err, 1);
-        __threadfence();
-    }
-    __syncthreads();
-    return *failed == 0;
-}
-
 // Sums over the warp of eight values a lane; sum q in the four lanes with lane / 4 == q.
 __device__ __forceinline__ float wsum8(float (&p)[kKB], int lane) {
     static_assert(kKB == 8, "three halving steps");
@@ -747,7 +726,7 @@ __global__ void __launch_bounds__(kSt, 1) k_gm_step(UView U, const double* w, co
                 if (k < nsum && tid % kSw == 0) part[(size_t)k * nb + blockIdx.x] = v;
             }
         }
-        if (!step_barrier(bar, &sc->wait_err, &s_failed)) return false;
+        if (!grid_meet(bar, &sc->wait_err, &s_failed)) return false;
         for (int k = warp; k < nsum; k += kSw) {
             double s = 0.0;
             for (int b0 = lane; b0 < nb; b0 += 256) {
