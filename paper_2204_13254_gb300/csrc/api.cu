@@ -606,12 +606,19 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
     const bool dp2 = U.n2 > 0;
     const bool use_warm = warm && (h->lam_valid || h->capturing);
     if (!use_warm) {
-        if (nm) CK(h, (int)cudaMemsetAsync(h->d.lam, 0, sizeof(double) * nm, s), "memset");
-        if (nc) CK(h, (int)cudaMemsetAsync(h->d.xC, 0, sizeof(double) * nc, s), "memset");
-        if (V.f32 && nm) CK(h, (int)cudaMemsetAsync(V.lamf, 0, sizeof(float) * nm, s), "memset");
-        if (V.f32 && nc) CK(h, (int)cudaMemsetAsync(V.xCf, 0, sizeof(float) * nc, s), "memset");
-        if (dp2) CK(h, (int)cudaMemsetAsync(h->d.lam2, 0, sizeof(double) * nm, s), "memset");
-        if (dp2 && V.f32) CK(h, (int)cudaMemsetAsync(h->d.lam2f, 0, sizeof(float) * nm, s), "memset");
+        CopyParts c;
+        c.add(h->d.lam, nullptr, sizeof(double) * nm);
+        c.add(h->d.xC, nullptr, sizeof(double) * nc);
+        if (V.f32) {
+            c.add(V.lamf, nullptr, sizeof(float) * nm);
+            c.add(V.xCf, nullptr, sizeof(float) * nc);
+        }
+        if (dp2) {
+            c.add(h->d.lam2, nullptr, sizeof(double) * nm);
+            if (V.f32) c.add(h->d.lam2f, nullptr, sizeof(float) * nm);
+        }
+        Prof P(h, ST_VEC, s, 1);
+        CK(h, launch_copy_parts(c, s), "cold start");
     }
     float* zuf = V.f32 ? h->d.zuf : nullptr;
     // DP1: x = [B_r^T u_l ; -u_c] over the [Gamma | c] columns of every local matrix;
@@ -834,8 +841,11 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
         // launching it when the multipliers are not valid (same values as a cold start)
         const bool use_warm = warm && (h->lam_valid || h->capturing);
         if (!use_warm) {
-            CK(h, (int)cudaMemsetAsync(h->d.lam, 0, nlb, s), "memset");
-            CK(h, (int)cudaMemsetAsync(h->d.lamf, 0, sizeof(float) * h->mult_dof.size(), s), "memset");
+            CopyParts c;
+            c.add(h->d.lam, nullptr, nlb);
+            c.add(h->d.lamf, nullptr, sizeof(float) * h->mult_dof.size());
+            Prof P(h, ST_VEC, s, 1);
+            CK(h, launch_copy_parts(c, s), "cold start");
         }
         // the whole CG in one kernel where every subdomain's operator finds room on chip
         bool resident = false;
@@ -1264,22 +1274,21 @@ int extrapolate_lambda(dd_handle* h, int prec, cudaStream_t s) {
 // corrections.  save: copy it aside after the first pass; !save: put it back.
 int keep_first_pass(dd_handle* h, bool save, cudaStream_t s) {
     const size_t nm = h->mult_dof.size(), nc = h->corner_dof.size();
-    auto cp = [&](void* a, void* b, size_t n) -> int {
-        if (!n) return DD_OK;
-        CK(h, (int)cudaMemcpyAsync(save ? b : a, save ? a : b, n, cudaMemcpyDeviceToDevice, s), "warm-start copy");
-        return DD_OK;
-    };
-    int rc = cp(h->d.lam, h->d.lam_scratch, sizeof(double) * nm);
-    if (!rc) rc = cp(h->d.lamf, h->d.lamf_scratch, sizeof(float) * nm);
-    if (!rc && h->prm.solver == DD_SOLVER_COUPLED_GMRES) {
-        rc = cp(h->d.xC, h->d.xC_scratch, sizeof(double) * nc);
-        if (!rc) rc = cp(h->d.xCf, h->d.xCf_scratch, sizeof(float) * nc);
+    CopyParts c;
+    auto cp = [&](void* a, void* b, size_t n) { c.add(save ? b : a, save ? a : b, n); };
+    cp(h->d.lam, h->d.lam_scratch, sizeof(double) * nm);
+    cp(h->d.lamf, h->d.lamf_scratch, sizeof(float) * nm);
+    if (h->prm.solver == DD_SOLVER_COUPLED_GMRES) {
+        cp(h->d.xC, h->d.xC_scratch, sizeof(double) * nc);
+        cp(h->d.xCf, h->d.xCf_scratch, sizeof(float) * nc);
     }
-    if (!rc && h->factored_scheme == DD_SCHEME_DP2) {
-        rc = cp(h->d.lam2, h->d.lam2_scratch, sizeof(double) * nm);
-        if (!rc) rc = cp(h->d.lam2f, h->d.lam2f_scratch, sizeof(float) * nm);
+    if (h->factored_scheme == DD_SCHEME_DP2) {
+        cp(h->d.lam2, h->d.lam2_scratch, sizeof(double) * nm);
+        cp(h->d.lam2f, h->d.lam2f_scratch, sizeof(float) * nm);
     }
-    return rc;
+    Prof P(h, ST_VEC, s, c.k > 0 ? 1 : 0);
+    CK(h, launch_copy_parts(c, s), "warm-start copy");
+    return DD_OK;
 }
 
 // One level of the Newmark recurrence from (u_n, u_nm1) into u_np1:

@@ -637,6 +637,20 @@ int launch_step_begin(const dd_handle* h, void* stream);
 int launch_extrapolate(const dd_handle* h, bool f32, void* stream);
 int launch_solve_end(const dd_handle* h, void* stream);
 int launch_refine_cond(const dd_handle* h, unsigned long long cond, void* stream);
+// Device copies (src null: zeroes) of up to six arrays of whole 4-byte words, as one kernel.
+struct CopyParts {
+    uint32_t* dst[6];
+    const uint32_t* src[6];
+    int64_t n[6];   // words
+    int k = 0;
+    void add(void* d, const void* s, size_t bytes) {
+        if (!bytes) return;
+        dst[k] = (uint32_t*)d;
+        src[k] = (const uint32_t*)s;
+        n[k++] = (int64_t)(bytes / 4);
+    }
+};
+int launch_copy_parts(const CopyParts& c, void* stream);
 int launch_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, float* lamf, unsigned long long cond,
                     bool* ran, void* stream);
 int launch_pcg_alpha(const dd_handle* h, const float* wf, float* pf, void* stream);
