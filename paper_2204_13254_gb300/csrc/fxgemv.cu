@@ -38,7 +38,7 @@
 // is copied any more.
 //
 // Measured (GB300), dense k_gemv<double> / here: coupled operator of 256 subdomains with
-// 400-480 interface rows, 42 M elements, 106 / 66 us (170 MB at 2.6 TB/s); the FP64 step of
+// 400-480 interface rows, 42 M elements, 106 / 64 us (170 MB at 2.7 TB/s); the FP64 step of
 // 512 subdomains of 1,854 unknowns 11.1 / 7.0 ms, its GEMVs 9.7 / 5.7 ms (3.6 TB/s).  What
 // bounds it now is instruction latency at two CTAs (16 warps) per SM: about 470 warp
 // instructions per strip, 96 of them multiply-adds, 36 % of the issue slots.
@@ -463,8 +463,13 @@ bool fx_active(const dd_handle* h, int mode) { return h->fx_ok && sym_active(h, 
 //    11.10 / 6.98 ms, 64 of them 2.16 / 1.92, 128 of 604 1.83 / 1.66, 64 of 604 1.15 /
 //    1.11; but 27 of 1,854 1.47 / 1.65, 8 of 1,512 0.99 / 1.13, 8 of 3,584 1.32 / 1.64,
 //    8 of 448 0.87 / 0.89.
-//  * CTAs per subdomain: one as soon as every SM has one (every CTA more stages x again),
-//    otherwise up to a cluster of 8.
+//  * CTAs per subdomain: every CTA more stages x again, but one CTA per subdomain leaves SMs
+//    with one CTA beside SMs with two where there are fewer subdomains than slots (two per
+//    SM).  So two up to 256 subdomains, and more (a cluster of 8 at most) only until every
+//    SM has a CTA.  Measured, FP64 GMRES step with 1 / 2 / 4 / 8 CTAs per subdomain, in us: 64
+//    subdomains of 1,854 unknowns 3,203 / 2,086 / 1,559 / 1,618, 100 of 741 1,323 / 1,047 /
+//    1,108 / 1,405, 128 of 2,196 3,947 / 3,110 / 3,330 / 4,164, 216 of 1,115 2,200 / 1,947 /
+//    2,207 / 3,091, 256 of 1,152 2,241 / 2,198 / 2,602 / 3,576, 343 of 604 1,511 / 1,624.
 //  * Subdomains kept in L2 between the launches of a Krylov solve: 64 MB worth, about half
 //    of L2, as the FP32 tuner settled on.
 void build_fx(dd_handle* h) {
@@ -511,7 +516,7 @@ void build_fx(dd_handle* h) {
             h->fx_tl[m].clear();
             continue;
         }
-        int cl = 1;
+        int cl = h->n_sub <= 256 ? 2 : 1;
         while (cl < kSymCLMax && h->n_sub * cl < 152) cl *= 2;
         h->fx_cl[m] = cl;
         int32_t longest = 0;
