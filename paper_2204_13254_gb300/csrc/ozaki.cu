@@ -565,12 +565,23 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     double* A = M + md.moff;
     double v[32];
     int mx = 0;
+    // below the block a thread's values are contiguous: 16-byte accesses
+    double2* const col = reinterpret_cast<double2*>(A + (int64_t)j * md.ld + k0 + kb);
+    if (on && !row) {
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const bool in = on && kb + k < nb;
-        v[k] = in ? (row ? A[(int64_t)(k0 + kb + k) * md.ld + j] : A[(int64_t)j * md.ld + k0 + kb + k]) : 0.0;
-        mx = max(mx, __double2hiint(v[k]) & 0x7fffffff);
+        for (int k = 0; k < 32; k += 2) {
+            double2 t = make_double2(0.0, 0.0);
+            if (kb + k + 1 < nb) t = col[k / 2];
+            else if (kb + k < nb) t.x = col[k / 2].x;
+            v[k] = t.x;
+            v[k + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = on && kb + k < nb ? A[(int64_t)(k0 + kb + k) * md.ld + j] : 0.0;
     }
+#pragma unroll
+    for (int k = 0; k < 32; ++k) mx = max(mx, __double2hiint(v[k]) & 0x7fffffff);
     xmax[half][r] = mx;
     tc::fence_before_sync();
     __syncthreads();
@@ -618,12 +629,15 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
                 mx = max(mx, __double2hiint(y) & 0x7fffffff);
             }
         }
-        if (on) {
+        if (on && row) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                if (kb + k >= nb) continue;
-                if (row) A[(int64_t)(k0 + kb + k) * md.ld + j] = v[k];
-                else A[(int64_t)j * md.ld + k0 + kb + k] = -v[k];
+            for (int k = 0; k < 32; ++k)
+                if (kb + k < nb) A[(int64_t)(k0 + kb + k) * md.ld + j] = v[k];
+        } else if (on) {
+#pragma unroll
+            for (int k = 0; k < 32; k += 2) {
+                if (kb + k + 1 < nb) col[k / 2] = make_double2(-v[k], -v[k + 1]);
+                else if (kb + k < nb) col[k / 2].x = -v[k];
             }
         }
     }
