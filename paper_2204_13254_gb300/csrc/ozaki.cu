@@ -62,19 +62,36 @@ __device__ __forceinline__ uint32_t small_float(int d) {
     return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
 }
 
+// rint(v 2^(56-e)) of |v| < 2^e (halves away from zero) in integer arithmetic: the multiply and
+// the conversion would take 32 clocks of the SM's FP64 pipe for a warp, these about 8 of the
+// integer pipe.  Subnormals count as zero.
+__device__ __forceinline__ long long to_digits(double v, int e) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
+    const unsigned long long m =
+        ((unsigned long long)(uint32_t)((hi & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(v);
+    const int r = min(1022 + e - ex, 63);   // >= 0; the value is (m 2^4 >> r) / 2
+    const unsigned long long t = ex ? (((m << 4) >> r) + 1) >> 1 : 0ull;
+    return hi < 0 ? -(long long)t : (long long)t;
+}
+
+// v 2^x, by the exponent field where the result is a normal number.
+__device__ __forceinline__ double scale_exp(double v, int x) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
+    if (ex && (unsigned)(ex + x - 1) < 2046u) return __hiloint2double(hi + (x << 20), __double2loint(v));
+    return v * pow2(x);
+}
+
 // Slices of eight consecutive elements v[0..7] (K direction) of a vector with
 // exponent e: one 16-byte chunk per slice, handed to put(slice, chunk).
 template <typename Put>
 __device__ __forceinline__ void cut8(const double* v, int e, Put put) {
-    const int x = 56 - e;
-    const double sc = pow2(x > 1023 ? 1023 : x);   // e < -967: v below 2^-967, digits from a smaller scale
     uint32_t w[kOzS][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         uint32_t f[2][kOzS];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const long long t = __double2ll_rn(v[2 * q + u] * sc);
+            const long long t = to_digits(v[2 * q + u], e);
             const unsigned long long b = (unsigned long long)t + 0x0000808080808080ull;   // balanced digits
             const uint32_t lo = (uint32_t)b, hi = (uint32_t)(b >> 32);
             f[u][6] = small_float((int)(lo & 255u) - 128);
@@ -624,7 +641,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int i = kb + 8 * g + c;
-                const double y = -join_classes(D, c) * pow2(e + ep[(int64_t)m * kOzK + i] - 56);
+                const double y = -scale_exp(join_classes(D, c), e + ep[(int64_t)m * kOzK + i] - 56);
                 v[8 * g + c] = y;
                 mx = max(mx, __double2hiint(y) & 0x7fffffff);
             }
