@@ -20,17 +20,19 @@
 // kept (k_oz_mirror fills the rest at the end), and the column panel of a pivot
 // block p is its row panel B = M[p, :] transposed up to the sign s_i = -1 for
 // swept rows, +1 otherwise.  One pivot block is three kernels:
-//   k_oz_pivot   P^-1 in FP64 (64 x 64, one CTA per matrix), its slices;
 //   k_oz_panel   slices of B; B' = -P^-1 B as a slice product; slices of B'; the
 //                row and column panels of M;
-//   k_oz_update  M_ij += s_i B_i . B'_j over the lower triangle outside p.
-// What bounds it: the update's two FP64 operations per element and pivot block
-// (GB300: two FP64 lanes per clock and SM) against 16 bytes of HBM traffic; the
-// wide pivot block and the triangle each halve both against 32-wide blocks over
-// the full square.  Measured, 40 matrices of up to 2,454 rows with their 1,229-row
-// coarse matrix: pivot 0.15, panel 0.07, update 0.26 ms per 64-wide block (mean over
-// both), against 0.51 + 0.09 (panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide
-// block over the full square; the whole factorisation 33 against 170 ms.
+//   k_oz_update  M_ij += s_i B_i . B'_j over the lower triangle outside p, and,
+//                in its first CTAs (one per matrix), P^-1 and its slices of the next
+//                block; k_oz_pivot forms the first block's.
+// What bounds it: instruction latency and the path to L2 in the update (two FP64
+// operations per element and pivot block at two lanes per clock and SM, 16 bytes of
+// HBM traffic); the wide pivot block and the triangle each halve both against 32-wide
+// blocks over the full square; with a single matrix the pivots one after another.
+// Measured, 40 matrices of up to 2,454 rows with their 1,229-row coarse matrix, per
+// 64-wide block (mean over both): panel 0.06, update with the next pivot 0.28 ms, against
+// 0.51 + 0.09 (pivot, panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide block over
+// the full square; the whole factorisation 25 against 170 ms.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
