@@ -39,7 +39,7 @@
 //
 // Measured (GB300), dense k_gemv<double> / here: coupled operator of 256 subdomains with
 // 400-480 interface rows, 42 M elements, 106 / 64 us (170 MB at 2.7 TB/s); the FP64 step of
-// 512 subdomains of 1,854 unknowns 11.1 / 7.0 ms, its GEMVs 9.7 / 5.7 ms (3.6 TB/s).  What
+// 512 subdomains of 1,854 unknowns 11.1 / 6.5 ms, its GEMVs 9.7 / 5.7 ms (3.8 TB/s).  What
 // bounds it now is instruction latency at two CTAs (16 warps) per SM: about 470 warp
 // instructions per strip, 96 of them multiply-adds, 36 % of the issue slots.
 #include <cooperative_groups.h>
