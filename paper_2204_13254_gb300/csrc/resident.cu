@@ -38,6 +38,7 @@
 
 #include <algorithm>
 
+#include "cg_rows.h"
 #include "dd_internal.h"
 #include "symtile.cuh"
 
@@ -595,7 +596,7 @@ struct CgArgs {
     void* v;
     PcgScalars* sc;
     uint32_t* bar;
-    double* partials;         // [3][gridDim.x]
+    double* partials;         // [kCgRows][gridDim.x]
     double tol, refine_tol;
     int64_t nl;
     int nc, ldc, ld, span, floats, have_q, adaptive, max_it, clustered;
@@ -750,9 +751,11 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
         if (gam) q = (double)__ldcg(w + 2 * mi) - (double)__ldcg(w + 2 * mi + 1);
         return true;
     };
-    // n sums over the multipliers (each counted by its first side), in CTA order, left in red[k][0]
+    // the sums R over the multipliers (each counted by its first side), in CTA order, left in
+    // red[k][0]; through the rows of the exchange buffer that cg_rows.h gives them
     const int nw = (nGam + 31) >> 5;   // warps with interface entries
-    auto sums = [&](int n, double a0, double a1, double a2) -> bool {
+    auto sums = [&](CgSums R, double a0, double a1, double a2) -> bool {
+        const int n = R.n;
         double v[3] = {own ? a0 : 0.0, own ? a1 : 0.0, own ? a2 : 0.0};
         if (warp < nw)
 #pragma unroll
@@ -765,12 +768,12 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
         if (tid < n) {
             double s = 0.0;
             for (int k = 0; k < nw; ++k) s += red[tid][k];
-            P.partials[(size_t)tid * nb + b] = s;
+            P.partials[(size_t)(R.row + tid) * nb + b] = s;
         }
         if (!grid_barrier<0>(meet)) return false;
         if (warp < n) {
             double s = 0.0;
-            for (int k = lane; k < nb; k += 32) s += __ldcg(P.partials + (size_t)warp * nb + k);
+            for (int k = lane; k < nb; k += 32) s += __ldcg(P.partials + (size_t)(R.row + warp) * nb + k);
             s = warp_sum(s);
             if (lane == 0) red[warp][0] = s;
         }
@@ -786,7 +789,7 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
         r = rhs - q;
         z = r * dinv;
     }
-    if (!sums(3, r * z, rhs * rhs, r * r)) return;
+    if (!sums(kCgStart, r * z, rhs * rhs, r * r)) return;
     if (tid == 0) {
         const double a = red[0][0], gg = red[1][0], rr = red[2][0];
         const bool finite = isfinite(a) && isfinite(gg) && isfinite(rr);
@@ -810,7 +813,7 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
             else x = (T)(sgn * pn);
         }
         if (!apply(x, q)) return;
-        if (!sums(1, warp < nw ? pn * q : 0.0, 0.0, 0.0)) return;
+        if (!sums(kCgPq, warp < nw ? pn * q : 0.0, 0.0, 0.0)) return;
         if (tid == 0) s_alpha = s_rz / red[0][0];
         __syncthreads();
         if (warp < nw) {
@@ -821,7 +824,7 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
             p = pn;
         }
         ++it;
-        if (!sums(2, warp < nw ? r * r : 0.0, warp < nw ? r * z : 0.0, 0.0)) return;
+        if (!sums(kCgRes, warp < nw ? r * r : 0.0, warp < nw ? r * z : 0.0, 0.0)) return;
         if (tid == 0) {
             const double rr = red[0][0], rz = red[1][0];
             const bool finite = isfinite(rr) && isfinite(rz) && isfinite(s_alpha);
