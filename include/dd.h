@@ -562,9 +562,11 @@ int dd_get_sym_config(const dd_handle* h, int32_t* cl, int32_t* st, int32_t* kee
 int dd_set_sym_config(dd_handle* h, int32_t kind, int32_t cl, int32_t st, int32_t keep, int32_t ws, void* stream);
 
 /* Failure-path testing aid for the bounded device waits.  With
- * first_wait_polls > 0, the first wait of every CTA of the packed-tile GEMVs
- * (DD_MIXED with sym_fp32) polls an mbarrier that nothing completes that many
- * times and gives up, as a wait on a lost copy would: the CTA records the
+ * first_wait_polls > 0, the first wait of every CTA of the packed GEMVs (FP32
+ * tiles of DD_MIXED, fixed-point tiles of DD_FP64), of the one-kernel interface
+ * solves and of the one-kernel Krylov steps is for something that never comes:
+ * it polls that many times and gives up, as a wait on a lost copy or on a CTA
+ * that never arrives would: the CTA records the
  * failure in the device status word, waits (bounded) for the copies it has in
  * flight and exits.  The step then returns DD_ERR_TIMEOUT -- in eager mode at
  * once, in graph mode from the first call that reads stats -- and is not

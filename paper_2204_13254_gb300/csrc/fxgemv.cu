@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     int32_t* yhi = reinterpret_cast<int32_t*>(full + st * kWarps);                // [span_max] high 32 bits
     __shared__ int wmax[kWarps];
     __shared__ int abort_flag;
+    __shared__ uint64_t never;   // completed by nothing (first_wait_test)
 
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -154,12 +155,19 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     const uint64_t pol = l2_policy(stored < keep);
     int32_t* wring = ring + warp * st * kStripInts;   // this warp's slots and barriers
     uint64_t* wfull = full + warp * st;
-    if (tid == 0) abort_flag = 0;
+    const int first_polls = tid == 0 ? xs.sc->wait_first : 0;   // (asked for ahead of its use)
+    if (tid == 0) {
+        abort_flag = 0;
+        mbar_init(&never, 1);
+    }
+    uint32_t flight = 0;   // lane 0: slots whose copy has not been waited for
     if (lane == 0) {
         for (int s = 0; s < st; ++s) mbar_init(&wfull[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         for (int s = 0; s < st && s < nt_cta; ++s) {
-            issue_strip(fx_entry(__ldg(lst + s), warp), tiles, wring + s * kStripInts, &wfull[s], pol);
+            const Strip t = fx_entry(__ldg(lst + s), warp);
+            issue_strip(t, tiles, wring + s * kStripInts, &wfull[s], pol);
+            flight |= (t.r0 < t.R ? 1u : 0u) << s;
         }
     }
     // x 2^d in FP64 (into the words its integers will take), its largest exponent, then the integers
@@ -207,6 +215,7 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     const bool finite = mx < 0x7ff00000;   // NaN or Inf in x: every row of this CTA becomes NaN
     const int X = exp_of_hi(mx);
     for (int p = p_lo + tid; p < p_end; p += kT) xq[p - p_lo] = finite ? split57(xd[p - p_lo], kBits - X) : make_int2(0, 0);
+    if (tid == 0 && !first_wait_test(first_polls, &never)) abort_flag = 1;
     __syncthreads();
 
     const int ri = lane >> 1, c8 = 8 * warp + 4 * (lane & 1);   // row in a block, first column in a tile
@@ -281,11 +290,15 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
             flush_d(cur);
         }
         if (t.r0 < t.R) {   // (uniform over the warp)
-            if (!bad && !wait_or_abort(&wfull[slot], (phases >> slot) & 1u, &abort_flag)) {
-                bad = true;
-                *(volatile int*)&abort_flag = 1;
+            if (!bad) {
+                if (wait_or_abort(&wfull[slot], (phases >> slot) & 1u, &abort_flag)) {
+                    phases ^= 1u << slot;
+                    flight &= ~(1u << slot);
+                } else {
+                    bad = true;
+                    *(volatile int*)&abort_flag = 1;
+                }
             }
-            phases ^= 1u << slot;
             int32_t* strip = wring + slot * kStripInts;
             const int32_t* base = strip - t.r0 * kBlkInts + 4 * lane;
             long long ch[4] = {}, cx[4] = {};
@@ -344,8 +357,11 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
             }
         }
         __syncwarp();   // every lane is done with the slot
-        if (lane == 0 && k + st < nt_cta && !*(volatile int*)&abort_flag)
-            issue_strip(fx_entry(fill, warp), tiles, wring + slot * kStripInts, &wfull[slot], pol);
+        if (lane == 0 && k + st < nt_cta && !*(volatile int*)&abort_flag) {
+            const Strip f = fx_entry(fill, warp);
+            issue_strip(f, tiles, wring + slot * kStripInts, &wfull[slot], pol);
+            flight |= (f.r0 < f.R ? 1u : 0u) << slot;
+        }
         if (k + st + 1 < nt_cta) fill = __ldg(lst + k + st + 1);
         ++cnt;
         if (++slot == st) slot = 0;
@@ -356,7 +372,7 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     if (bad) {   // let the copies still in flight land (bounded), then report
         if (lane == 0)
             for (int s = 0; s < st; ++s)
-                for (int par = 0; par < 2; ++par) mbar_wait(&wfull[s], (uint32_t)par, 1u << 16);
+                if ((flight >> s) & 1u) mbar_wait(&wfull[s], (phases >> s) & 1u);
         if (tid == 0) atomicExch(err, 1);
         __syncthreads();
     }

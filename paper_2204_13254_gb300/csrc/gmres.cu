@@ -613,6 +613,7 @@ __global__ void __launch_bounds__(kSt, 1) k_gm_step(UView U, const double* w, co
     const bool ctl = (int)blockIdx.x == nb - 1;
     const int64_t ib = (int64_t)blockIdx.x * (kSt * E), i0 = ib + tid;
     const bool work = ib < nu;
+    if (tid == 0) s_failed = sc->wait_first;
     uint32_t* const bar_a = &gs->counter[1];
     uint32_t* const bar_b = &gs->counter[2];
     if (ctl) {

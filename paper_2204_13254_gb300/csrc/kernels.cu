@@ -776,6 +776,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_pcg_step(int64_t n_lambda, cons
     const int nb = (int)gridDim.x, tid = threadIdx.x;
     const int64_t m0 = blockIdx.x * (int64_t)kThreads + tid, stride = (int64_t)nb * kThreads;
     const double beta = sc->beta, rz = sc->rz;
+    if (tid == 0) s_failed = sc->wait_first;
     double pn[E], qq[E], rr[E], lm[E], di[E];
     double v[1] = {0.0};
 #pragma unroll

@@ -75,6 +75,7 @@ struct Meet {
     uint32_t target;
     int32_t* err;
     int* failed;   // shared memory
+    int first;     // thread 0: PcgScalars::wait_first (> 0: wait, this many polls long, for an arrival nobody makes)
 };
 
 // Grid barrier: writes of the product warps (W > 0: only these are waited for before the
@@ -92,12 +93,14 @@ __device__ bool grid_barrier(Meet& m) {
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(m.bar, 1u);
+        const uint32_t target = m.target + (m.first > 0 ? 1u : 0u);
+        const unsigned limit = m.first > 0 ? (unsigned)m.first : kBarLimit;
         unsigned k = 0;
         uint32_t v;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(m.bar) : "memory");
-        } while (v < m.target && ++k < kBarLimit);
-        if (v < m.target) {
+        } while (v < target && ++k < limit);
+        if (v < target) {
             *m.failed = 1;
             atomicExch(m.err, 1);
         }
@@ -105,6 +108,20 @@ __device__ bool grid_barrier(Meet& m) {
     }
     __syncthreads();
     return *m.failed == 0;
+}
+
+// The wait for the copy of the tiles, by every thread of the CTA (first: thread 0's
+// PcgScalars::wait_first).  False, in every thread, when it gave up; the copy has then been
+// given a second wait, so that it does not land in a CTA that has ended.
+__device__ bool tiles_landed(uint64_t* bar, uint64_t* never, int first, int32_t* err, int* failed) {
+    const bool ok = first_wait_test(first, never) && mbar_wait(bar, 0u);
+    if (!ok) {
+        *failed = 1;
+        atomicExch(err, 1);
+        mbar_wait(bar, 0u);
+    }
+    __syncthreads();
+    return *failed == 0;
 }
 
 // Sum of nb FP32 partial sums (a warp; lanes take q = lane, lane + 32, ...) as an integer in
@@ -250,7 +267,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     __shared__ double shnext, sresid, s_beta, s_bnorm, s_thr;
     __shared__ float sinv;
     __shared__ int s_end, s_final, s_k, s_conv, s_status, s_it, s_fail;
-    __shared__ uint64_t bar_tiles;
+    __shared__ uint64_t bar_tiles, never;
     __shared__ int tile_ab[64], tile_off[64];
 
     const UView& U = P.U;
@@ -261,7 +278,8 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     GmresScalars* gs = P.gs;
     const int m = gs->m, max_it = gs->max_it;
     const double tol = gs->tol;
-    Meet meet{P.clustered ? nullptr : &gs->bar, 0u, &P.sc->wait_err, &s_fail};
+    const int first_polls = tid == 0 ? P.sc->wait_first : 0;
+    Meet meet{P.clustered ? nullptr : &gs->bar, 0u, &P.sc->wait_err, &s_fail, first_polls};
 
     // the tiles of the [Gamma | c] block: the subdomain's first run
     if (tid == 0) {
@@ -270,6 +288,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
         s_status = DD_OK;
         const int off = tile_table(sd, tile_ab, tile_off);
         mbar_init(&bar_tiles, 1);
+        mbar_init(&never, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         load_tile(tiles, P.Msym + sd.toff, 4u * (uint32_t)off, &bar_tiles, l2_policy(true));
     }
@@ -321,12 +340,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     const float dinvf = (float)dinv;
     const int nw = (g + 31) >> 5;   // warps with entries
     __syncthreads();
-    if (!mbar_wait(&bar_tiles, 0u)) {   // (every thread waits itself)
-        s_fail = 1;
-        atomicExch(&P.sc->wait_err, 1);
-    }
-    __syncthreads();
-    if (s_fail) return;
+    if (!tiles_landed(&bar_tiles, &never, first_polls, &P.sc->wait_err, &s_fail)) return;
 
     auto product = [&]() { tile_product<kW>(sd, tiles, tile_ab, tile_off, 0, nT, xg, yw, P.span); };
     // this entry's row of M_s x, published (the corner rows of M = J S change sign)
@@ -618,7 +632,7 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
     __shared__ double s_rz, s_gg, s_rr, s_tol2, s_alpha, s_beta;
     __shared__ int s_done, s_finite;
     __shared__ int s_fail, tile_ab[64], tile_off[64];
-    __shared__ uint64_t bar_tiles;
+    __shared__ uint64_t bar_tiles, never;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, b = blockIdx.x;
     const SymDesc sd = P.descs[b];
     const MatDesc md = P.mats[b];
@@ -632,12 +646,14 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
     T* w = reinterpret_cast<T*>(P.w);
     T* vC = reinterpret_cast<T*>(P.v);
     const T* K = reinterpret_cast<const T*>(P.K);
-    Meet meet{P.clustered ? nullptr : P.bar, 0u, &P.sc->wait_err, &s_fail};
+    const int first_polls = tid == 0 ? P.sc->wait_first : 0;
+    Meet meet{P.clustered ? nullptr : P.bar, 0u, &P.sc->wait_err, &s_fail, first_polls};
     if (tid == 0) s_fail = 0;
     if constexpr (kF32) {
         if (tid == 0) {
             const int off = tile_table(sd, tile_ab, tile_off);
             mbar_init(&bar_tiles, 1);
+            mbar_init(&never, 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             load_tile(tiles, P.Msym + sd.toff, 4u * (uint32_t)off, &bar_tiles, l2_policy(true));
         }
@@ -676,12 +692,7 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 2) k_cg_resident(CgArgs 
     }
     __syncthreads();
     if constexpr (kF32) {
-        if (!mbar_wait(&bar_tiles, 0u)) {
-            s_fail = 1;
-            atomicExch(&P.sc->wait_err, 1);
-        }
-        __syncthreads();
-        if (s_fail) return;
+        if (!tiles_landed(&bar_tiles, &never, first_polls, &P.sc->wait_err, &s_fail)) return;
     }
     // rows [i0, g) of M_s x; the result of entry e in y(e)
     auto product = [&](int i0) {

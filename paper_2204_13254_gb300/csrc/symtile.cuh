@@ -62,9 +62,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // Failure-path test (PcgScalars::wait_first > 0): the CTA's first wait polls
 // `never`, an mbarrier no thread or copy ever completes, wait_first times and
 // gives up, exercising the give-up / drain / report path with every copy issued.
-__device__ __forceinline__ bool first_wait_test(const XSrc& xs, uint64_t* never) {
-    const int n = xs.sc ? xs.sc->wait_first : 0;
+__device__ __forceinline__ bool first_wait_test(int n, uint64_t* never) {
     return n > 0 ? mbar_wait(never, 0u, (unsigned)n) : true;
+}
+__device__ __forceinline__ bool first_wait_test(const XSrc& xs, uint64_t* never) {
+    return first_wait_test(xs.sc ? xs.sc->wait_first : 0, never);
 }
 
 // Shape of a listed tile: rows, padded width (floats per row of a rectangle),

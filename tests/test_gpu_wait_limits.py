@@ -1,0 +1,73 @@
+"""Every bounded device wait of a step, made to run out by dd_set_wait_limit: the step is
+reported as DD_ERR_TIMEOUT and not taken, the context stays usable, and the march goes on
+as if nothing had happened.  One problem per kernel that waits: the fixed-point FP64 GEMV
+(64 subdomains), the one-kernel Arnoldi and CG steps (8 large subdomains, dense FP64
+GEMVs, which wait for nothing), the one-kernel interface solves of small tearings (216
+subdomains) in FP64 and mixed precision.  No GPU fault is involved.
+
+Tolerances: the solves after the interrupted step start cold, so the fields agree with
+those of an undisturbed march to the tolerance of the solves (FP64 1e-13, mixed 1e-11)
+times a margin for the steps between."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2204_13254_gb300 import dd as D
+from paper_2204_13254_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+GMRES, CG = D.DD_SOLVER_COUPLED_GMRES, D.DD_SOLVER_SCHUR_CG
+PROBLEMS = {
+    "fixed_gmres": (16, 4, D.DD_FP64, GMRES), "fixed_cg": (16, 4, D.DD_FP64, CG),
+    "step_gmres": (12, 2, D.DD_FP64, GMRES), "step_cg": (12, 2, D.DD_FP64, CG),
+    "resident_cg64": (12, 6, D.DD_FP64, CG), "resident_cg32": (12, 6, D.DD_MIXED, CG),
+    "resident_gmres32": (12, 6, D.DD_MIXED, GMRES),
+}
+
+
+def solver(kind, graph):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n, k, prec, solver_ = PROBLEMS[kind]
+    w = W.box(n, n, n, k, k, k)
+    mixed = prec == D.DD_MIXED
+    prm = D.make_params(precision=prec, tol=1e-5 if mixed else 1e-13, refine_tol=1e-11, max_refine=8, max_it=2000,
+                        solver=solver_, use_graph=graph)
+    fs = D.FieldSolver(w.xyz, w.tets, w.part, w.n_sub, w.eps, w.mu, params=prm).bind()
+    fs.factor(0.46 / n)
+    return fs
+
+
+def march(fs, interrupt):
+    src = torch.tensor(np.random.default_rng(2).standard_normal(fs.n_dof), device="cuda")
+    out = torch.empty_like(src)
+    fields = []
+    for k in range(4):
+        if interrupt and k == 2:
+            e0, e1, step = fs.get_state()
+            D.dd_set_wait_limit(fs.h, 4)
+            st = D.dd_step_scaled(fs.h, src, 1.0 / (1 + k), out, stats=True, raise_on_error=False)
+            D.dd_set_wait_limit(fs.h, 0)
+            assert st["rc"] == D.DD_ERR_TIMEOUT, st
+            assert "wait" in D.lib().dd_last_error(fs.h).decode()
+            f0, f1, step2 = fs.get_state()
+            assert step2 == step and torch.equal(f0, e0) and torch.equal(f1, e1)
+        D.dd_step_scaled(fs.h, src, 1.0 / (1 + k), out)
+        fields.append(out.clone())
+    return fields
+
+
+@pytest.mark.parametrize("graph", [1])
+@pytest.mark.parametrize("kind", list(PROBLEMS))
+def test_wait_that_runs_out_is_reported(kind, graph):
+    runs = []
+    for interrupt in (False, True):
+        fs = solver(kind, graph)
+        try:
+            runs.append(march(fs, interrupt))
+        finally:
+            fs.close()
+    for a, b in zip(*runs):
+        assert torch.linalg.norm(a - b) <= 1e-9 * torch.linalg.norm(b)
