@@ -862,6 +862,10 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
             } else {
                 PcgScalars hs;
                 CK(h, read_scalars(h, &hs, s), "pcg scalars");
+                if (hs.wait_err) {   // the kernel ended early: the other words are an earlier solve's
+                    h->err = "a bounded device wait of the interface CG gave up";
+                    return DD_ERR_TIMEOUT;
+                }
                 iters = hs.it;
                 h->work[ST_SCHUR] += hs.it;
                 res = hs.gg > 0 ? std::sqrt(hs.rr / hs.gg) : 0.0;
@@ -1303,7 +1307,7 @@ int report_timeout(dd_handle* h, cudaStream_t s) {
     CK(h, (int)cudaMemsetAsync(&h->d.sc->wait_err, 0, sizeof(int32_t), s), "clear wait error");
     CK(h, (int)cudaStreamSynchronize(s), "sync");
     h->lam_valid = false;
-    h->err = "a bounded device wait of the packed-tile GEMV gave up; the step was not taken";
+    h->err = "a bounded device wait gave up; the step was not taken";
     return DD_ERR_TIMEOUT;
 }
 
@@ -1322,12 +1326,17 @@ int advance(dd_handle* h, const double* u_n, const double* u_nm1, double* u_np1,
     }
     if (h->prm.precision == DD_FP64) {
         status = dd_solve(h, DD_FP64, h->prm.tol, h->prm.warm_start != 0, &iters, &resid, s);
-        if (status != DD_OK && status != DD_ERR_NO_CONVERGENCE) {   // a wait that gave up leaves NaN behind
+        if (status != DD_OK && status != DD_ERR_NO_CONVERGENCE) {   // a wait that gave up voids the solve
             if (status != DD_ERR_CUDA && wait_err_set(h, s)) return report_timeout(h, s);
             return status;
         }
-        Prof P(h, ST_VEC, s, 1);
-        CK(h, launch_writeback(h, u_n, u_nm1, nullptr, nullptr, 1, u_np1, s), "writeback");
+        {
+            Prof P(h, ST_VEC, s, 1);
+            CK(h, launch_writeback(h, u_n, u_nm1, nullptr, nullptr, 1, u_np1, s), "writeback");
+        }
+        // the GEMVs behind the interface solve wait too in their fixed-point form: nothing later
+        // in the step would notice (the time level moves in the caller, on DD_OK)
+        if ((fx_active(h, GEMV_RECOVER) || fx_active(h, GEMV_SCHUR_C)) && wait_err_set(h, s)) return report_timeout(h, s);
     } else {
         // FP64 iterative refinement of the step system with FP32 DD correction solves
         {

@@ -753,6 +753,7 @@ __global__ void __launch_bounds__(kSt, 1) k_gm_step(UView U, const double* w, co
         if (tid == 0) {
             gs->k = 0;
             gs->converged = 0;
+            gs->status = DD_ERR_TIMEOUT;
             gs->final = gs->cycle_end = gs->skip = 1;
             if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 0u);
         }

@@ -59,7 +59,7 @@ def march(fs, interrupt):
     return fields
 
 
-@pytest.mark.parametrize("graph", [1])
+@pytest.mark.parametrize("graph", [0, 1])
 @pytest.mark.parametrize("kind", list(PROBLEMS))
 def test_wait_that_runs_out_is_reported(kind, graph):
     runs = []
@@ -71,3 +71,27 @@ def test_wait_that_runs_out_is_reported(kind, graph):
             fs.close()
     for a, b in zip(*runs):
         assert torch.linalg.norm(a - b) <= 1e-9 * torch.linalg.norm(b)
+
+
+@pytest.mark.parametrize("kind", ["fixed_gmres", "fixed_cg"])
+def test_wait_behind_the_interface_solve(kind):
+    """Only the last GEMVs of an eager FP64 step give up: the solve has converged by then, and
+    the error word alone tells.  The word is set by hand before the step (it is sticky): 24
+    bytes in front of the limit that dd_set_wait_limit writes."""
+    fs = solver(kind, 0)
+    try:
+        src = torch.tensor(np.random.default_rng(2).standard_normal(fs.n_dof), device="cuda")
+        out = torch.empty_like(src)
+        D.dd_step(fs.h, src, out)
+        words = fs.ws_view.view(torch.int32)
+        D.dd_set_wait_limit(fs.h, 1987654321)
+        at = torch.nonzero(words == 1987654321).flatten()
+        D.dd_set_wait_limit(fs.h, 0)
+        assert at.numel() == 1 and words[at].item() == 0
+        words[at - 6] = 1
+        st = D.dd_step(fs.h, src, out, stats=True, raise_on_error=False)
+        assert st["rc"] == D.DD_ERR_TIMEOUT and fs.get_state()[2] == 1
+        assert words[at - 6].item() == 0
+        assert D.dd_step(fs.h, src, out, stats=True)["rc"] == D.DD_OK
+    finally:
+        fs.close()
