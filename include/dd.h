@@ -406,7 +406,10 @@ int dd_pic_state(const dd_handle* h, double* x, int32_t* status, double* G, doub
 
 /* Apply the Schur-complement interface operator of Eq. f1schur,
  * out = (F_rr + F_rc K~cc^-1 F_rc^T) lam, in FP64 with the factors of the last
- * dd_factor.  lam, out: device [n_lambda]. */
+ * dd_factor.  lam, out: device [n_lambda].  This call, dd_coupled_apply,
+ * dd_dp2_apply and dd_schur_apply_static only launch on `stream`: a bounded
+ * device wait that gives up in one of them leaves NaN in out, and no error for
+ * a later call to report. */
 int dd_schur_apply(dd_handle* h, const double* lam, double* out, void* stream);
 
 /* Apply the coupled operator of Eqs. F1lr + F1uc in FP64 with the factors of

@@ -429,8 +429,10 @@ GemvOut gout_coupled(const dd_handle* h, double* out, float* out32) {
 // Inside the CG loop (check_done) launches after convergence exit early; their
 // full-work count is added by dd_solve once the iteration count is known.
 int apply_schur_w(dd_handle* h, int prec, int kind, const double* v, const double* v2, const float* vf,
-                  const float* v2f, bool check_done, cudaStream_t s) {
+                  const float* v2f, bool check_done, cudaStream_t s, bool apply = false) {
     const Vecs V = vecs(h, prec);
+    GemvOut go_w = V.f32 ? gout(nullptr, nullptr, V.wf, nullptr, 1.0) : gout(h->d.w, nullptr, nullptr, nullptr, 1.0);
+    go_w.apply = apply ? 1 : 0;
     const double full = check_done ? 0.0 : 1.0;   // CG-loop launches are counted by count_cg_work
     int rc;
     const int kind_cv = kind == X_PCG ? X_PCG_CV : X_LAMBDA_CV;
@@ -438,9 +440,7 @@ int apply_schur_w(dd_handle* h, int prec, int kind, const double* v, const doubl
         // u_s = A_cr A_rr^-1 B_r^T z (corner rows), K~cc^-1 sum_s B_c^T u_s
         {
             Prof P(h, ST_CORNER, s, 1, full * mb(h, GEMV_SCHUR_C, prec));
-            rc = launch_gemv(h, GEMV_SCHUR_C, prec, xsrc(kind, v, v2, vf, v2f),
-                             V.f32 ? gout(nullptr, nullptr, V.wf, nullptr, 1.0) : gout(h->d.w, nullptr, nullptr, nullptr, 1.0),
-                             check_done, s);
+            rc = launch_gemv(h, GEMV_SCHUR_C, prec, xsrc(kind, v, v2, vf, v2f), go_w, check_done, s);
         }
         if (rc) return rc;
         {
@@ -459,9 +459,7 @@ int apply_schur_w(dd_handle* h, int prec, int kind, const double* v, const doubl
     // interface rows over [Gamma | c] columns with x = [B_r^T z ; -v]:
     // A_rr^-1 B_r^T z + A_rr^-1 A_rc B_c K~cc^-1 (...) in one pass (M[Gamma, c] = -A_rr^-1 A_rc)
     Prof P(h, ST_SCHUR, s, 1, full * mb(h, GEMV_SCHUR_G, prec));
-    return launch_gemv(h, GEMV_SCHUR_G, prec, xsrc(kind_cv, v, v2, vf, v2f, h->d.vC, V.vCf),
-                       V.f32 ? gout(nullptr, nullptr, V.wf, nullptr, 1.0) : gout(h->d.w, nullptr, nullptr, nullptr, 1.0),
-                       check_done, s);
+    return launch_gemv(h, GEMV_SCHUR_G, prec, xsrc(kind_cv, v, v2, vf, v2f, h->d.vC, V.vCf), go_w, check_done, s);
 }
 
 // The vectors of one CG iteration.
@@ -1777,7 +1775,7 @@ int dd_schur_apply(dd_handle* h, const double* lam, double* out, void* stream) {
     if (h->factored_scheme != DD_SCHEME_DP1) return h->fail(DD_ERR_STATE, "dd_schur_apply needs the DP1 factorisation");
     if (h->mult_dof.empty()) return DD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    CK(h, apply_schur_w(h, DD_FP64, X_LAMBDA, lam, nullptr, nullptr, nullptr, false, s), "apply");
+    CK(h, apply_schur_w(h, DD_FP64, X_LAMBDA, lam, nullptr, nullptr, nullptr, false, s, true), "apply");
     Prof P(h, ST_VEC, s, 1);
     CK(h, launch_jump(h, h->d.w, nullptr, nullptr, 1.0, out, s), "jump");
     return DD_OK;
@@ -1790,10 +1788,12 @@ int dd_coupled_apply(dd_handle* h, const double* u, double* out, void* stream) {
     const size_t nm = h->mult_dof.size(), nc = h->corner_dof.size();
     if (nm + nc == 0) return DD_OK;
     cudaStream_t s = (cudaStream_t)stream;
+    GemvOut go = gout_coupled(h, h->d.w, nullptr);
+    go.apply = 1;
     {
         Prof P(h, ST_SCHUR, s, 1, mb(h, GEMV_COUPLED, DD_FP64));
         CK(h, launch_gemv(h, GEMV_COUPLED, DD_FP64, xsrc(X_LAMBDA_CV, u, nullptr, nullptr, nullptr, u + nm, nullptr),
-                          gout_coupled(h, h->d.w, nullptr), false, s), "coupled operator");
+                          go, false, s), "coupled operator");
     }
     Prof P(h, ST_VEC, s, 1);
     CK(h, launch_gm_combine(h, uview(h, DD_FP64), u, out, s), "combine");
@@ -1807,11 +1807,13 @@ int dd_dp2_apply(dd_handle* h, const double* u, double* out, void* stream) {
     const size_t nm = h->mult_dof.size(), nc = h->corner_dof.size();
     if (nm + nc == 0) return DD_OK;
     cudaStream_t s = (cudaStream_t)stream;
+    GemvOut go = gout_coupled(h, h->d.w, nullptr);
+    go.apply = 1;
     {
         Prof P(h, ST_SCHUR, s, 1, mb(h, GEMV_COUPLED, DD_FP64));
         CK(h, launch_gemv(h, GEMV_COUPLED, DD_FP64,
                           xsrc(X_SIDE_CP, u, u + nm, nullptr, nullptr, u + 2 * nm, nullptr),
-                          gout_coupled(h, h->d.w, nullptr), false, s), "DP2 operator");
+                          go, false, s), "DP2 operator");
     }
     Prof P(h, ST_VEC, s, 1);
     CK(h, launch_gm_combine(h, uview(h, DD_FP64), u, out, s), "combine");

@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
         if (lane == 0)
             for (int s = 0; s < st; ++s)
                 if ((flight >> s) & 1u) mbar_wait(&wfull[s], (phases >> s) & 1u);
-        if (tid == 0) atomicExch(err, 1);
+        if (tid == 0 && err) atomicExch(err, 1);
         __syncthreads();
     }
     // this CTA's partial sums in units of 2^d_i (NaN when x was not finite or a wait gave up)
@@ -590,5 +590,6 @@ int launch_fxgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32
     return (int)cudaLaunchKernelEx(&cfg, k_fxgemv, (const SymDesc*)h->d.symd, (const int32_t*)h->d.fx_rng[mode],
                                    (const uint32_t*)h->d.fx_tl[mode], (const int32_t*)h->d.Mfx,
                                    (const int64_t*)h->d.fx_moff, (const int32_t*)h->d.fx_exps, span, cl, st, rmask, cmask, h->fx_keep[mode],
-                                   std::max(1, h->n_sub_real), xs, go, skip, &h->d.sc->wait_err);
+                                   std::max(1, h->n_sub_real), xs, go, skip,
+                                   go.apply ? (int32_t*)nullptr : &h->d.sc->wait_err);
 }

@@ -89,7 +89,7 @@ extern "C" int dd_schur_apply_static(dd_handle* h, const double* lam, double* ou
         xs = XSrc{};
         xs.kind = X_LAMBDA;
         xs.v = lam;
-        go = GemvOut{w, nullptr, nullptr, nullptr, 1.0};
+        go = GemvOut{w, nullptr, nullptr, nullptr, 1.0, nullptr, 1};
         e = launch_gemv(h, GEMV_SCHUR_C, DD_FP64, xs, go, false, stream);
         if (!e) e = launch_corner_gather(h, w, nullptr, nullptr, uC, nullptr, false, stream);
         if (!e) {
@@ -105,7 +105,7 @@ extern "C" int dd_schur_apply_static(dd_handle* h, const double* lam, double* ou
         xs.kind = X_LAMBDA_CV;
         xs.v = lam;
         xs.v3 = vC;
-        go = GemvOut{w, nullptr, nullptr, nullptr, 1.0};
+        go = GemvOut{w, nullptr, nullptr, nullptr, 1.0, nullptr, 1};
         e = launch_gemv(h, GEMV_SCHUR_G, DD_FP64, xs, go, false, stream);
     }
     if (!e) e = launch_jump(h, w, nullptr, nullptr, 1.0, out, stream);

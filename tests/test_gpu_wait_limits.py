@@ -95,3 +95,35 @@ def test_wait_behind_the_interface_solve(kind):
         assert D.dd_step(fs.h, src, out, stats=True)["rc"] == D.DD_OK
     finally:
         fs.close()
+
+
+@pytest.mark.parametrize("scheme", [D.DD_SCHEME_DP1, D.DD_SCHEME_DP2])
+def test_operator_calls(scheme):
+    """An operator call that gives up leaves NaN in its own result and nothing behind."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w = W.box(16, 16, 16, 4, 4, 4)
+    fs = D.FieldSolver(w.xyz, w.tets, w.part, w.n_sub, params=D.make_params(solver=GMRES, scheme=scheme, tol=1e-12)).bind()
+    try:
+        fs.factor(0.03)
+        nc, gen = fs.sizes.n_corner, torch.Generator().manual_seed(1)
+        calls = [lambda u, v: D.dd_dp2_apply(fs.h, u, v)]
+        sizes = [2 * fs.n_lambda + nc]
+        if scheme == D.DD_SCHEME_DP1:
+            calls = [lambda u, v: D.dd_coupled_apply(fs.h, u, v), lambda u, v: D.dd_schur_apply(fs.h, u, v),
+                     lambda u, v: D.dd_schur_apply_static(fs.h, u, v)]
+            sizes = [fs.n_lambda + nc, fs.n_lambda, fs.n_lambda]
+        src = torch.randn(fs.n_dof, dtype=torch.float64, generator=gen).cuda()
+        for call, n in zip(calls, sizes):
+            u = torch.randn(n, dtype=torch.float64, generator=gen).cuda()
+            a, b, c = (torch.zeros_like(u) for _ in range(3))
+            call(u, a)
+            D.dd_set_wait_limit(fs.h, 4)
+            call(u, b)
+            D.dd_set_wait_limit(fs.h, 0)
+            assert torch.isfinite(a).all() and torch.isnan(b).any()
+            assert D.dd_step(fs.h, src, None, stats=True)["rc"] == D.DD_OK
+            call(u, c)
+            assert torch.equal(a, c)
+    finally:
+        fs.close()
