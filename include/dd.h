@@ -567,13 +567,13 @@ int dd_set_sym_config(dd_handle* h, int32_t kind, int32_t cl, int32_t st, int32_
 /* Failure-path testing aid for the bounded device waits.  With
  * first_wait_polls > 0, the first wait of every CTA of the packed GEMVs (FP32
  * tiles of DD_MIXED, fixed-point tiles of DD_FP64), of the one-kernel interface
- * solves and of the one-kernel Krylov steps is for something that never comes:
- * it polls that many times and gives up, as a wait on a lost copy or on a CTA
- * that never arrives would: the CTA records the
+ * solves, of the one-kernel Krylov steps and of the tensor-core elimination is
+ * for something that never comes: it polls that many times and gives up, as a
+ * wait on a lost copy or on a CTA that never arrives would: the CTA records the
  * failure in the device status word, waits (bounded) for the copies it has in
- * flight and exits.  The step then returns DD_ERR_TIMEOUT -- in eager mode at
- * once, in graph mode from the first call that reads stats -- and is not
- * taken: e^n, e^{n-1} and the step counter stay where they were and the next
+ * flight and exits.  dd_factor then returns DD_ERR_TIMEOUT, and so does a step
+ * -- in eager mode at once, in graph mode from the first call that reads stats
+ * -- which is not taken: e^n, e^{n-1} and the step counter stay where they were and the next
  * solve starts cold.  0 restores the normal waits (2^20 polls).  Synchronises
  * `stream`.  Errors: DD_ERR_ARG (negative), DD_ERR_STATE (no workspace). */
 int dd_set_wait_limit(dd_handle* h, int32_t first_wait_polls, void* stream);

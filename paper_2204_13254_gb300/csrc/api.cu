@@ -1215,12 +1215,13 @@ int dd_factor(dd_handle* h, double dt, void* stream) {
     int32_t st = 0;
     CK(h, (int)cudaMemcpyAsync(&st, h->d.status, 4, cudaMemcpyDeviceToHost, s), "status");
     CK(h, (int)cudaStreamSynchronize(s), "sync");
-    if (st != 0) return h->fail(DD_ERR_NOT_SPD, "non-positive pivot in the local or coarse elimination");
-    if (wait_err_set(h, s)) {   // a bounded wait of the tensor-core update gave up: the factors are void
+    if (wait_err_set(h, s)) {   // a bounded wait of the tensor-core elimination gave up: the factors are void, and so
+                               // is what their pivots say
         CK(h, (int)cudaMemsetAsync(&h->d.sc->wait_err, 0, sizeof(int32_t), s), "clear wait error");
         CK(h, (int)cudaStreamSynchronize(s), "sync");
         return h->fail(DD_ERR_TIMEOUT, "a bounded device wait of the tensor-core elimination gave up");
     }
+    if (st != 0) return h->fail(DD_ERR_NOT_SPD, "non-positive pivot in the local or coarse elimination");
     const size_t nd = (size_t)h->n_dof;
     for (int k = 0; k < 3; ++k) CK(h, (int)cudaMemsetAsync(h->d.e[k], 0, sizeof(double) * nd, s), "memset");
     CK(h, (int)cudaStreamSynchronize(s), "sync");

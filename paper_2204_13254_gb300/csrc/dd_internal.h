@@ -688,7 +688,7 @@ bool sym_active(const dd_handle* h, int mode);
 // ozaki.cu
 size_t oz_bytes(int nm, int nmax);
 int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, unsigned char* ws, int32_t* status,
-                    int32_t* err, void* stream);
+                    PcgScalars* sc, void* stream);
 int launch_oz_mirror(const MatDesc* mats, double* M, int nm, int nmax, void* stream);
 // tensor.cu
 void build_tc(dd_handle* h);

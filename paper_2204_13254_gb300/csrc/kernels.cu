@@ -1240,7 +1240,7 @@ int launch_sweep(const dd_handle* h, bool coarse, int k0, void* stream) {
     const int nm = coarse ? 1 : h->n_sub_real;
     const int nmax = coarse ? (int)h->corner_dof.size() : h->max_ns;
     if (h->prm.factor_mode == DD_FACTOR_TENSOR)
-        return launch_oz_sweep(mats, M, nm, nmax, k0, h->d.oz, h->d.status, &h->d.sc->wait_err, stream);
+        return launch_oz_sweep(mats, M, nm, nmax, k0, h->d.oz, h->d.status, h->d.sc, stream);
     double* Pinv = coarse ? h->d.Pinv + (size_t)h->n_sub * kNB * kNB : h->d.Pinv;
     // chunks of rows (column panel), and of columns (row panel) for the coarse matrix, whose
     // thousands of rows one CTA per pivot block would serialise; the many local matrices keep one CTA

@@ -160,8 +160,8 @@ __device__ __forceinline__ double join_classes(const uint32_t (&r)[kOzS][8], int
     return (double)((H << 24) + ((L + 128) >> 8));
 }
 
-__device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity) {
-    for (unsigned k = 0; k < kOzPolls; ++k) {
+__device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity, unsigned polls = kOzPolls) {
+    for (unsigned k = 0; k < polls; ++k) {
         uint32_t ok;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -185,6 +185,12 @@ __device__ __forceinline__ bool oz_wait_or_abort(uint64_t* bar, uint32_t parity,
         if ((k & 255u) == 255u && *abort) return false;
     }
     return false;
+}
+
+// Failure-path test (PcgScalars::wait_first = n > 0): the CTA's first wait is for `never`, which
+// nothing completes at that point, n polls long.
+__device__ __forceinline__ bool oz_first_wait(int n, uint64_t* never) {
+    return n > 0 ? oz_wait(never, 0u, (unsigned)n) : true;
 }
 
 __device__ __forceinline__ void oz_init(uint64_t* bar, uint32_t count) {
@@ -557,7 +563,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
                                                                const int32_t* __restrict__ ep, uint16_t* __restrict__ Bs,
                                                                int32_t* __restrict__ eb, uint16_t* __restrict__ Cs,
                                                                int32_t* __restrict__ ec, int nmax,
-                                                               int32_t* __restrict__ err) {
+                                                               PcgScalars* __restrict__ sc) {
     const int m = blockIdx.y, rb = blockIdx.x;
     const MatDesc md = mats[m];
     if (k0 >= md.nr || rb * kOzRows >= md.ns) return;
@@ -624,7 +630,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     __syncthreads();
     bool ok = true;
     if (tid == 0) {
-        ok = oz_wait(&bars[0], 0u);
+        ok = oz_first_wait(sc->wait_first, &bars[1]) && oz_wait(&bars[0], 0u);
         if (ok) {
             tc::fence_after_sync();
             oz_products(tmem, kOzK, tc::smem_addr(sB), tc::smem_addr(sP));
@@ -672,7 +678,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
             cut8(v + 8 * g, f, [&](int p, uint4 w) { *reinterpret_cast<uint4*>(gC + p * kOzPiece + o) = w; });
         }
     } else if (tid == 0) {
-        atomicExch(err, 1);
+        atomicExch(&sc->wait_err, 1);
         oz_wait(&bars[0], 0u);   // the copy lands before the CTA ends (bounded)
     }
     tc::fence_before_sync();
@@ -709,7 +715,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
                                                              const int32_t* __restrict__ ec, int nmax,
                                                              uint16_t* __restrict__ Ps, int32_t* __restrict__ ep,
                                                              int nm, int runs, int32_t* __restrict__ status,
-                                                             int32_t* __restrict__ err) {
+                                                             PcgScalars* __restrict__ pcg) {
     const bool ahead = (int)blockIdx.x < nm;
     const int m = ahead ? (int)blockIdx.x : ((int)blockIdx.x - nm) / runs;
     const MatDesc md = mats[m];
@@ -809,7 +815,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
     };
     if (warp == 8) {
         if (lane == 0) {
-            if (!oz_wait(abar, 0u)) abort_flag = 1;
+            if (!oz_first_wait(pcg->wait_first, &tempty[0]) || !oz_wait(abar, 0u)) abort_flag = 1;
             for (int n = 0; n < nu && !abort_flag; ++n) issue(n);
         }
     } else {
@@ -906,7 +912,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
         oz_wait(abar, 0u);
         for (int n = issued > kOzStages ? issued - kOzStages : 0; n < issued; ++n)
             oz_wait(&full[n % kOzStages], (uint32_t)(n / kOzStages) & 1u);
-        atomicExch(err, 1);
+        atomicExch(&pcg->wait_err, 1);
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -964,7 +970,7 @@ size_t oz_bytes(int nm, int nmax) { return oz_layout(nm, std::max(nmax, 1)).tota
 // One pivot block [k0, k0 + 64) of the sweep of nm matrices (of at most nmax rows), and the
 // inverse of the next one; called for k0 = 0, 64, ... in turn.
 int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, unsigned char* ws, int32_t* status,
-                    int32_t* err, void* stream) {
+                    PcgScalars* sc, void* stream) {
     const int nrb = (nmax + kOzRows - 1) / kOzRows;
     const OzLayout L = oz_layout(nm, nmax);
     uint16_t* Ps = reinterpret_cast<uint16_t*>(ws + L.ps);
@@ -979,11 +985,11 @@ int launch_oz_sweep(const MatDesc* mats, double* M, int nm, int nmax, int k0, un
     if (e != cudaSuccess) return (int)e;
     if (k0 == 0) k_oz_pivot<<<(unsigned)nm, kOzPivThreads, kOzPivSmem, S(stream)>>>(mats, M, Ps, ep, status);
     k_oz_panel<<<dim3((unsigned)nrb, (unsigned)nm), kOzPanThreads, kOzPanSmem, S(stream)>>>(mats, M, k0, nrb, Ps, ep, Bs,
-                                                                                            eb, Cs, ec, nmax, err);
+                                                                                            eb, Cs, ec, nmax, sc);
     unsigned runs = 0;
     for (int rb = 0; rb < nrb; ++rb) runs += (unsigned)((4 * (rb + 1) + kOzRun - 1) / kOzRun);
     k_oz_update<<<(unsigned)nm * (1 + runs), kOzThreads, kOzSmem, S(stream)>>>(mats, M, k0, nrb, Bs, Cs, eb, ec, nmax, Ps,
-                                                                              ep, nm, (int)runs, status, err);
+                                                                              ep, nm, (int)runs, status, sc);
     return (int)cudaGetLastError();
 }
 

@@ -127,3 +127,31 @@ def test_operator_calls(scheme):
             assert torch.equal(a, c)
     finally:
         fs.close()
+
+
+def test_factorisation():
+    """The tensor-core elimination: reported as what it is (its pivots say nothing then), nothing
+    factored, nothing left behind, and the next factorisation is as good as the first."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    w = W.cavity(8, 2)
+    fs = D.FieldSolver(w.xyz, w.tets, w.part, w.n_sub,
+                       params=D.make_params(solver=GMRES, factor_mode=D.DD_FACTOR_TENSOR)).bind()
+    try:
+        u = torch.randn(fs.n_lambda + fs.sizes.n_corner, dtype=torch.float64,
+                        generator=torch.Generator().manual_seed(1)).cuda()
+        fs.factor(0.05)
+        a = fs.coupled_apply(u)
+        for _ in range(2):
+            D.dd_set_wait_limit(fs.h, 4)
+            with pytest.raises(D.DDError) as e:
+                fs.factor(0.05)
+            assert e.value.code == D.DD_ERR_TIMEOUT
+            D.dd_set_wait_limit(fs.h, 0)
+            with pytest.raises(D.DDError) as e:
+                fs.coupled_apply(u)
+            assert e.value.code == D.DD_ERR_STATE
+        fs.factor(0.05)
+        assert torch.equal(fs.coupled_apply(u), a)
+    finally:
+        fs.close()
