@@ -265,8 +265,12 @@ typedef struct {
 int dd_setup(const dd_mesh* mesh, const int32_t* part, int32_t n_sub, const dd_params* params,
              dd_handle** out);
 
-/* Change solver parameters of an existing handle (precision needs a
- * workspace large enough for it: the workspace is always sized for both). */
+/* Change solver parameters of an existing handle.  The workspace serves either
+ * precision; the packed operators of DD_MIXED and the fixed-point ones of
+ * DD_FP64 share a part of it, so the first step, adjoint step or autotuning in
+ * another precision than the last forms them again from the factors (a pass
+ * over them on its stream).  A graph of operator calls (dd_*_apply) that a
+ * caller has captured belongs to the precision that it was captured in. */
 int dd_set_params(dd_handle* h, const dd_params* params);
 
 int dd_get_sizes(const dd_handle* h, dd_sizes* out);
@@ -286,7 +290,7 @@ int dd_bind_workspace(dd_handle* h, void* dev_ptr, size_t bytes, void* stream);
  * memory): assemble the dense local A^(s) = T^(s) + dt^2/4 S^(s), eliminate
  * its r block in FP64 to obtain A_rr^-1, A_rr^-1 A_rc and the local corner
  * Schur complements, assemble and invert K~cc, build the Jacobi diagonal, and
- * (always) FP32 copies for DD_MIXED.  Resets the time level to n = 0 with
+ * the packed operators of the handle's precision.  Resets the time level to n = 0 with
  * e^0 = e^{-1} = 0.  Synchronises `stream`.  Errors: DD_ERR_STATE (no
  * workspace), DD_ERR_NOT_SPD, DD_ERR_CUDA. */
 int dd_factor(dd_handle* h, double dt, void* stream);

@@ -227,14 +227,25 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.probe_dof, 6 * kMaxProbes);
     L.take(d.probe_w, 18 * kMaxProbes);
     L.take(d.M64, (size_t)h->dense_elems);
-    L.take(d.M32, (size_t)h->dense_elems);
-    L.take(d.Msym, (size_t)h->sym_elems);
-    L.take(d.Mfx, 256 * (size_t)h->fx_blocks);
+    {   // One region for the packed operators of DD_MIXED or those of DD_FP64 (h->packed) and, until the
+        // factors are complete, the slices and exponents of the pivot block of the tensor-core
+        // elimination (local or coarse)
+        const size_t at = L.off;
+        L.take(d.M32, (size_t)h->dense_elems);
+        L.take(d.Msym, (size_t)h->sym_elems);
+        size_t end = L.off;
+        L.off = at;
+        L.take(d.Mfx, 256 * (size_t)h->fx_blocks);
+        end = std::max(end, L.off);
+        L.off = at;
+        L.take(d.oz, std::max(oz_bytes(std::max(1, h->n_sub_real), h->max_ns), oz_bytes(1, (int)nc)));
+        L.off = std::max(end, L.off);
+    }
     L.take(d.fx_dir, h->fx_dir.size());
     L.take(d.fx_moff, h->fx_moff.size());
     L.take(d.fx_exps, (size_t)h->sub_ptr[h->n_sub_real]);
     for (int m = 0; m < GEMV_NMODES; ++m)
-        if (fx_active(h, m)) {
+        if (fx_built(h, m)) {
             L.take(d.fx_rng[m], h->fx_rng[m].size());
             L.take(d.fx_tl[m], h->fx_tl[m].size());
         }
@@ -254,8 +265,6 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.K64, nc * (size_t)h->ldc);
     L.take(d.K32, nc * (size_t)h->ldc);
     L.take(d.Pinv, (size_t)(h->n_sub + 1) * kNB * kNB);
-    // slices and exponents of one pivot block of the tensor-core elimination (local or coarse)
-    L.take(d.oz, std::max(oz_bytes(std::max(1, h->n_sub_real), h->max_ns), oz_bytes(1, (int)nc)));
     L.take(d.dinv, nm);
     L.take(d.rpart, (size_t)(kMaxRestart + 4) * (size_t)h->n_sub);
     for (int k = 0; k < 3; ++k) L.take(d.e[k], nd);
@@ -366,6 +375,23 @@ bool wait_err_set(dd_handle* h, cudaStream_t s) {
     if (cudaMemcpyAsync(&v, &h->d.sc->wait_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return false;
     if (cudaStreamSynchronize(s) != cudaSuccess) return false;
     return v != 0;
+}
+
+// Forms the packed operators of one precision from the factors.  Where FP64 has packed ones of
+// its own (fixed point) the two share their storage.
+int pack_operators(dd_handle* h, int prec, cudaStream_t s) {
+    const bool fx = h->fx_ok && prec == DD_FP64;
+    Prof P(h, ST_FACTOR, s, 2);
+    if (fx) CK(h, launch_fx_pack(h, s), "fixed-point tiles");
+    else CK(h, launch_fp32_copy(h, s), "FP32 operators");
+    if (!fx) CK(h, launch_sym_pack(h, s), "packed symmetric tiles");
+    h->packed = prec;
+    return DD_OK;
+}
+
+// The packed operators of the precision that a solve runs in: they change when dd_set_params does.
+int use_precision(dd_handle* h, int prec, cudaStream_t s) {
+    return !h->fx_ok || h->packed == prec ? DD_OK : pack_operators(h, prec, s);
 }
 
 // Read the CG scalars back (synchronises the stream).
@@ -1207,9 +1233,9 @@ int dd_factor(dd_handle* h, double dt, void* stream) {
         CK(h, launch_corner_diag(h, s), "coarse diagonal");
     }
     {
-        Prof P(h, ST_FACTOR, s, 3);
-        CK(h, launch_sym_pack(h, s), "packed symmetric tiles");
-        CK(h, launch_fx_pack(h, s), "fixed-point tiles");
+        const int prc = pack_operators(h, h->prm.precision, s);
+        if (prc) return prc;
+        Prof P(h, ST_FACTOR, s, 1);
         CK(h, launch_tc_pack(h, s), "tensor-core panels");
     }
     int32_t st = 0;
@@ -1316,6 +1342,10 @@ int advance(dd_handle* h, const double* u_n, const double* u_nm1, double* u_np1,
     int status = DD_OK, iters = 0, refinements = 0;
     double resid = 0.0;
     {
+        const int prc = use_precision(h, h->prm.precision, s);
+        if (prc) return prc;
+    }
+    {
         Prof P(h, ST_RHS, s, 1, h->bytes_per_launch[ST_RHS]);
         CK(h, launch_rhs(h, u_n, src, src_sign, h->dt, s), "rhs");
     }
@@ -1335,7 +1365,7 @@ int advance(dd_handle* h, const double* u_n, const double* u_nm1, double* u_np1,
         }
         // the GEMVs behind the interface solve wait too in their fixed-point form: nothing later
         // in the step would notice (the time level moves in the caller, on DD_OK)
-        if ((fx_active(h, GEMV_RECOVER) || fx_active(h, GEMV_SCHUR_C)) && wait_err_set(h, s)) return report_timeout(h, s);
+        if (fx_active(h, GEMV_RECOVER) && wait_err_set(h, s)) return report_timeout(h, s);
     } else {
         // FP64 iterative refinement of the step system with FP32 DD correction solves
         {
@@ -1559,6 +1589,10 @@ int capture_step(dd_handle* h, int phase) {
 
 int dd_step_graph(dd_handle* h, const double* d2g, double scale, double* e_out, dd_stats* stats, cudaStream_t s) {
     const int phase = h->cur;
+    {
+        const int prc = use_precision(h, h->prm.precision, s);
+        if (prc) return prc;
+    }
     if (!h->gexec[phase]) {
         int rc = capture_step(h, phase);
         if (rc) return rc;
@@ -1999,6 +2033,10 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
         }
     }
     const bool cached = found.size() == (size_t)(2 * GEMV_NMODES) && found_cl.size() == (size_t)n_sym;
+    if (!cached) {   // the FP32 kinds are timed on their own operators, FP64 ones in their dense form
+        const int prc = use_precision(h, DD_MIXED, s);
+        if (prc) return prc;
+    }
     cudaEvent_t e0, e1;
     CK(h, (int)cudaEventCreate(&e0), "event");
     CK(h, (int)cudaEventCreate(&e1), "event");
@@ -2098,7 +2136,7 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
                     }
                 }
                 h->prm.sym_fp32 = 0;   // the dense tiles below time the dense kernel
-                if (h->tasks[p][m].empty() || (p == 0 && fx_active(h, m))) {   // (fixed point: nothing to choose)
+                if (h->tasks[p][m].empty() || (p == 0 && fx_built(h, m) && h->prm.precision == DD_FP64)) {   // (fixed point: nothing to choose)
                     found[{p, m}] = h->tile[p][m];
                     h->prm.sym_fp32 = sym_saved ? 1 : 0;
                     continue;
@@ -2167,6 +2205,10 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
         h->sym_ws[kv.first] = kv.second.ws;
         sym_ranges(h, kv.first, kv.second.cl);
         CK(h, upload(h->d.sym_rng[kv.first], h->sym_rng[kv.first], s), "upload ranges");
+    }
+    {
+        const int prc = use_precision(h, h->prm.precision, s);
+        if (prc) return prc;
     }
     CK(h, (int)cudaStreamSynchronize(s), "sync");
     drop_graphs(h);

@@ -331,7 +331,7 @@ struct DevPtrs {
     int32_t* sym_rng[GEMV_NMODES] = {};   // [n_sub * kSymCLMax * kSymRng] (list offset, tile count, end tile row,
                                           // subdomain, ensemble members served) per CTA
     uint32_t* sym_tl[GEMV_NMODES] = {};   // tiles of each packed mode, every subdomain in row order
-    int32_t* Mfx = nullptr;          // packed tiles in fixed point, blocks of 16 x 8 elements of two words
+    int32_t* Mfx = nullptr;          // (in the place of M32, Msym) packed tiles in fixed point, blocks of 16 x 8 elements of two words
     int32_t* fx_dir = nullptr;       // [tiles * 4], first block of every stored subdomain, tile lists
     int64_t* fx_moff = nullptr;
     uint32_t* fx_tl[GEMV_NMODES] = {};
@@ -516,6 +516,7 @@ struct dd_handle {
     bool sym_ok = false;                           // the packed GEMV's shared memory fits one CTA
     ResSizes res{0, 0, 0};                         // sizes of the resident solves (resident.cu)
     bool fx_ok = false;                            // the same for the fixed-point FP64 form (fxgemv.cu)
+    int packed = 0;                                // fx_ok: precision of the packed operators in the workspace
     std::vector<int32_t> fx_dir;                   // its directory (as sym_dir, offsets in blocks), the first block of
     std::vector<int64_t> fx_moff;                  // every stored subdomain, blocks in all, tile lists (order of sym_tl) and
     int64_t fx_blocks = 0;                         // the bytes one launch streams
@@ -614,6 +615,7 @@ int launch_sweep(const dd_handle* h, bool coarse, int k0, void* stream);
 int launch_mirror(const dd_handle* h, bool coarse, void* stream);
 int launch_coarse_assemble(const dd_handle* h, void* stream);
 int launch_factor_finish(const dd_handle* h, void* stream);
+int launch_fp32_copy(const dd_handle* h, void* stream);
 int launch_rhs(const dd_handle* h, const double* e_n, const double* src, double src_sign, double dt, void* stream);
 int launch_grad_eps(const dd_handle* h, const double* mu, const double* e_k, const double* e_km1, const double* e_km2,
                     double* grad_eps, void* stream);
@@ -677,6 +679,7 @@ int launch_gm_resident(const dd_handle* h, const UView& U, int have_q, int m, bo
 int launch_cg_resident(const dd_handle* h, int prec, double tol, int have_q, int adaptive, bool* ran, void* stream);
 // fxgemv.cu
 void build_fx(dd_handle* h);
+bool fx_built(const dd_handle* h, int mode);
 bool fx_active(const dd_handle* h, int mode);
 int launch_fx_pack(const dd_handle* h, void* stream);
 int launch_fxgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);

@@ -467,8 +467,10 @@ __global__ void __launch_bounds__(256) k_fx_pack(const SymDesc* __restrict__ des
 
 }  // namespace
 
-// True when the fixed-point form serves FP64 GEMVs of `mode`.
-bool fx_active(const dd_handle* h, int mode) { return h->fx_ok && sym_active(h, mode) && h->fx_bytes[mode] > 0.0; }
+// True when the fixed-point form can serve FP64 GEMVs of `mode`, and when it does (its tiles are
+// the packed operators in the workspace).
+bool fx_built(const dd_handle* h, int mode) { return h->fx_ok && sym_active(h, mode) && h->fx_bytes[mode] > 0.0; }
+bool fx_active(const dd_handle* h, int mode) { return fx_built(h, mode) && h->packed == DD_FP64; }
 
 // Host side: the directory and the tile lists with block offsets, CTAs per subdomain, the
 // ranges of every mode.
@@ -490,6 +492,7 @@ bool fx_active(const dd_handle* h, int mode) { return h->fx_ok && sym_active(h, 
 //    of L2, as the FP32 tuner settled on.
 void build_fx(dd_handle* h) {
     h->fx_ok = h->sym_elems > 0 && fx_depth(h->sym_np_max) > 0;
+    h->packed = h->prm.precision;
     h->fx_dir.clear();
     h->fx_moff.clear();
     h->fx_blocks = 0;

@@ -1273,9 +1273,13 @@ int launch_factor_finish(const dd_handle* h, void* stream) {
     if (nl)
         k_jacobi<<<reduce_blocks(nl), kThreads, 0, S(stream)>>>(nl, h->d.mult_slot, h->d.slot_sub, h->d.mats, h->d.M64,
                                                                 h->d.dinv);
-    k_to_fp32<<<4 * 152, kThreads, 0, S(stream)>>>(h->dense_elems, h->d.M64, h->d.M32);
     const int64_t kc = (int64_t)h->corner_dof.size() * h->ldc;
     if (kc) k_to_fp32<<<reduce_blocks(kc), kThreads, 0, S(stream)>>>(kc, h->d.K64, h->d.K32);
+    return (int)cudaGetLastError();
+}
+
+int launch_fp32_copy(const dd_handle* h, void* stream) {
+    k_to_fp32<<<4 * 152, kThreads, 0, S(stream)>>>(h->dense_elems, h->d.M64, h->d.M32);
     return (int)cudaGetLastError();
 }
 
