@@ -130,6 +130,9 @@ typedef struct {
  *            CTAs on the device at once, each solve is one cooperative kernel
  *            (the packed launch of the coupled kind, dd_set_sym_config, is then
  *            not used by it, nor is chunk).
+ *            The GEMVs of DD_FP64 steps run in fixed point from 48 subdomains
+ *            and 8 MB of operators upward: 57 bits below the largest entry of a
+ *            subdomain, so accurate in the norm like FP64 sums, not row by row.
  * restart    GMRES restart length m, 1..DD_MAX_RESTART (the paper: 20).
  * scheme     DD_SCHEME_DP1 (default) or DD_SCHEME_DP2.  DP2 (Sec. III-B, read for
  *            the edge-only step system A = T + dt^2/4 S): every local matrix
@@ -411,9 +414,9 @@ int dd_pic_state(const dd_handle* h, double* x, int32_t* status, double* G, doub
 /* Apply the Schur-complement interface operator of Eq. f1schur,
  * out = (F_rr + F_rc K~cc^-1 F_rc^T) lam, in FP64 with the factors of the last
  * dd_factor.  lam, out: device [n_lambda].  This call, dd_coupled_apply,
- * dd_dp2_apply and dd_schur_apply_static only launch on `stream`: a bounded
- * device wait that gives up in one of them leaves NaN in out, and no error for
- * a later call to report. */
+ * dd_dp2_apply and dd_schur_apply_static only launch on `stream` and wait for
+ * nothing on the device.  They sum FP64 products of FP64 numbers, row by row,
+ * whatever form the steps of the handle use. */
 int dd_schur_apply(dd_handle* h, const double* lam, double* out, void* stream);
 
 /* Apply the coupled operator of Eqs. F1lr + F1uc in FP64 with the factors of

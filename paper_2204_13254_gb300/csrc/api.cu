@@ -484,7 +484,7 @@ int apply_schur_w(dd_handle* h, int prec, int kind, const double* v, const doubl
     }
     // interface rows over [Gamma | c] columns with x = [B_r^T z ; -v]:
     // A_rr^-1 B_r^T z + A_rr^-1 A_rc B_c K~cc^-1 (...) in one pass (M[Gamma, c] = -A_rr^-1 A_rc)
-    Prof P(h, ST_SCHUR, s, 1, full * mb(h, GEMV_SCHUR_G, prec));
+    Prof P(h, ST_SCHUR, s, 1, full * (apply ? h->mode_bytes[GEMV_SCHUR_G] : mb(h, GEMV_SCHUR_G, prec)));
     return launch_gemv(h, GEMV_SCHUR_G, prec, xsrc(kind_cv, v, v2, vf, v2f, h->d.vC, V.vCf), go_w, check_done, s);
 }
 
@@ -1826,7 +1826,7 @@ int dd_coupled_apply(dd_handle* h, const double* u, double* out, void* stream) {
     GemvOut go = gout_coupled(h, h->d.w, nullptr);
     go.apply = 1;
     {
-        Prof P(h, ST_SCHUR, s, 1, mb(h, GEMV_COUPLED, DD_FP64));
+        Prof P(h, ST_SCHUR, s, 1, h->mode_bytes[GEMV_COUPLED]);
         CK(h, launch_gemv(h, GEMV_COUPLED, DD_FP64, xsrc(X_LAMBDA_CV, u, nullptr, nullptr, nullptr, u + nm, nullptr),
                           go, false, s), "coupled operator");
     }
@@ -1845,7 +1845,7 @@ int dd_dp2_apply(dd_handle* h, const double* u, double* out, void* stream) {
     GemvOut go = gout_coupled(h, h->d.w, nullptr);
     go.apply = 1;
     {
-        Prof P(h, ST_SCHUR, s, 1, mb(h, GEMV_COUPLED, DD_FP64));
+        Prof P(h, ST_SCHUR, s, 1, h->mode_bytes[GEMV_COUPLED]);
         CK(h, launch_gemv(h, GEMV_COUPLED, DD_FP64,
                           xsrc(X_SIDE_CP, u, u + nm, nullptr, nullptr, u + 2 * nm, nullptr),
                           go, false, s), "DP2 operator");
@@ -2055,6 +2055,8 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
             const int prec = p == 0 ? DD_FP64 : DD_MIXED;
             for (int m = 0; m < GEMV_NMODES && !rc; ++m) {
                 const bool sym_saved = h->prm.sym_fp32 != 0;
+                // FP64 kinds of an FP64 handle in fixed point; the operator calls' ones are applied dense too
+                const bool fixed_only = fx_built(h, m) && h->prm.precision == DD_FP64 && m != GEMV_COUPLED && m != GEMV_SCHUR_G;
                 if (p == 1 && h->sym_ok && sym_active(h, m)) {
                     // packed symmetric tiles: time both kernel forms with 1, 2, 4 and 8 CTAs per subdomain and
                     // rings of 2, 3 and 4 tiles
@@ -2136,7 +2138,7 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
                     }
                 }
                 h->prm.sym_fp32 = 0;   // the dense tiles below time the dense kernel
-                if (h->tasks[p][m].empty() || (p == 0 && fx_built(h, m) && h->prm.precision == DD_FP64)) {   // (fixed point: nothing to choose)
+                if (h->tasks[p][m].empty() || (p == 0 && fixed_only)) {   // (fixed point: nothing to choose)
                     found[{p, m}] = h->tile[p][m];
                     h->prm.sym_fp32 = sym_saved ? 1 : 0;
                     continue;

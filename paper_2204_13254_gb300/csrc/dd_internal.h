@@ -190,7 +190,7 @@ struct GemvOut {
     const float* base32;
     double alpha;
     const int32_t* pos = nullptr;
-    int32_t apply = 0;   // an operator call (dd_*_apply): its caller sees `out`, and nobody reads wait_err after it
+    int32_t apply = 0;   // an operator call (dd_*_apply): FP64 in its dense form (see fxgemv.cu)
 };
 
 // Tile shape of a batched GEMV launch: lanes cooperating on one row and rows

@@ -1,10 +1,8 @@
 """One handle stepped in FP64, in mixed precision and in FP64 again, on a tearing whose FP64
 operators are packed in fixed point (they share their storage with the FP32 ones): every
 result equals, bit for bit, that of a handle that has only ever had that precision;
-autotuning in between leaves the packed operators as they are; and the operator calls, in FP64 whatever
-the handle's precision, agree between the fixed-point and the dense form.
-
-Tolerance of the last: both are within a few 1e-16 of the operator in the norm."""
+autotuning in between leaves the packed operators as they are; and the operator calls, in FP64
+whatever the handle's precision, are the same."""
 import numpy as np
 import pytest
 
@@ -49,17 +47,16 @@ def test_switch(solver, graph):
 
     want = {p: step(one[p]) for p in prms}
     assert torch.linalg.norm(want[D.DD_MIXED] - want[D.DD_FP64]) <= 1e-8 * torch.linalg.norm(want[D.DD_FP64])
-    fixed, dense = one[D.DD_FP64].coupled_apply(u), one[D.DD_MIXED].coupled_apply(u)
-    assert not torch.equal(fixed, dense)          # two forms
-    assert torch.linalg.norm(fixed - dense) <= 2e-15 * torch.linalg.norm(dense)
+    applied = one[D.DD_FP64].coupled_apply(u)
+    assert torch.equal(applied, one[D.DD_MIXED].coupled_apply(u))
     try:
         for prec in (D.DD_FP64, D.DD_MIXED, D.DD_FP64, D.DD_MIXED):
             both.set_params(prms[prec])
             assert torch.equal(step(both), want[prec])
-            assert torch.equal(both.coupled_apply(u), fixed if prec == D.DD_FP64 else dense)
+            assert torch.equal(both.coupled_apply(u), applied)
         both.set_params(prms[D.DD_FP64])
         D.dd_autotune(both.h)
-        assert torch.equal(both.coupled_apply(u), fixed)
+        assert close(both.coupled_apply(u), applied)   # (its dense form is tuned)
         same = torch.equal if solver == D.DD_SOLVER_COUPLED_GMRES else close   # (the CG's dense kinds are tuned)
         assert same(step(both), want[D.DD_FP64])
         both.factor(0.02)                         # and a new factorisation packs for the precision in force

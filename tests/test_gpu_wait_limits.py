@@ -99,7 +99,8 @@ def test_wait_behind_the_interface_solve(kind):
 
 @pytest.mark.parametrize("scheme", [D.DD_SCHEME_DP1, D.DD_SCHEME_DP2])
 def test_operator_calls(scheme):
-    """An operator call that gives up leaves NaN in its own result and nothing behind."""
+    """The operator calls only launch, and nobody reads the error word after them: they wait for
+    nothing, and leave nothing behind that a later step would report."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     w = W.box(16, 16, 16, 4, 4, 4)
@@ -121,7 +122,7 @@ def test_operator_calls(scheme):
             D.dd_set_wait_limit(fs.h, 4)
             call(u, b)
             D.dd_set_wait_limit(fs.h, 0)
-            assert torch.isfinite(a).all() and torch.isnan(b).any()
+            assert torch.isfinite(a).all() and torch.equal(a, b)
             assert D.dd_step(fs.h, src, None, stats=True)["rc"] == D.DD_OK
             call(u, c)
             assert torch.equal(a, c)
