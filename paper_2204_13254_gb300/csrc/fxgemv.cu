@@ -18,7 +18,7 @@
 // and the sums of hi hi' and of hi lo' + lo hi' run in two 64-bit accumulators: a product
 // adds at most 2^56 to the first and less than 2^57 to the second, so 64 products fit
 // (a tile's transposed sums; the direct sums of two lanes over kFlush = 8 tiles).  From
-// there the sums go on as 96-bit integers in shared memory and become FP64 numbers once
+// there the sums go on as 96-bit integers (fx96.h) in shared memory and become FP64 numbers once
 // per CTA and row (conversions run on the FP64 pipe, at two per clock and SM).  lo lo' is
 // dropped.
 //
@@ -63,6 +63,7 @@
 
 #include "dd_internal.h"
 #include "fixpoint.cuh"
+#include "fx96.h"
 #include "symtile.cuh"
 #include "xsrc.cuh"
 
@@ -78,6 +79,8 @@ constexpr int kBlkInts = 256;          // one 16 x 8 block: 128 hi words, 128 lo
 constexpr int kStripInts = 4 * kBlkInts;   // ring slot of one warp: 64 rows x 8 columns, 4 KB
 constexpr int kPad = 17;               // column stride of the transposed sums in a slot (16 row lanes, no bank conflicts)
 constexpr int kFxW = 4;                // words per tile list entry: tile_entry(), first block, block rows | strips << 8, 0
+
+static_assert(kFx96Low == kLow, "the split of the integers");
 
 inline cudaStream_t S(void* s) { return (cudaStream_t)s; }
 
@@ -174,14 +177,11 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
         abort_flag = 0;
         mbar_init(&never, 1);
     }
-    uint32_t flight = 0;   // lane 0: slots whose copy has not been waited for
     if (lane == 0) {
         for (int s = 0; s < st; ++s) mbar_init(&wfull[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         for (int s = 0; s < st && s < nt_cta; ++s) {
-            const Strip t = fx_entry(__ldg(lst + s), warp);
-            issue_strip(t, tiles, wring + s * kStripInts, &wfull[s], pol);
-            flight |= (t.r0 < t.R ? 1u : 0u) << s;
+            issue_strip(fx_entry(__ldg(lst + s), warp), tiles, wring + s * kStripInts, &wfull[s], pol);
         }
     }
     // x 2^d in FP64 (into the words its integers will take), its largest exponent, then the integers
@@ -237,12 +237,8 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     int xh[4], xl[4];         // x of those rows
     int cur = -1, cnt = 0;
     bool bad = false;
-    // entry p of y += h 2^kLow + x (a 96-bit integer; the entry belongs to this warp)
-    auto add_y = [&](int p, __int128 v) {
-        v += ((__int128)yhi[p] << 64) + ylo[p];
-        ylo[p] = (uint64_t)v;
-        yhi[p] = (int32_t)(v >> 64);
-    };
+    // entry p of y += v (a 96-bit integer; the entry belongs to this warp)
+    auto add_y = [&](int p, __int128 v) { fx96_add(ylo[p], yhi[p], v); };
     // direct sums of tile row `row` -> y: the two column quads of the lane pair (each lane keeps
     // two rows), then over the eight warps; warp w adds rows 8 w .. 8 w + 7
     auto flush_d = [&](int row) {
@@ -264,7 +260,7 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const longlong2 t = red[(2 * q + u) * 64 + i];
-            v += ((__int128)t.x << kLow) + t.y;
+            v += fx96_part(t.x, t.y);
         }
 #pragma unroll
         for (int o = 8; o <= 16; o <<= 1) {
@@ -307,7 +303,6 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
             if (!bad) {
                 if (wait_or_abort(&wfull[slot], (phases >> slot) & 1u, &abort_flag)) {
                     phases ^= 1u << slot;
-                    flight &= ~(1u << slot);
                 } else {
                     bad = true;
                     *(volatile int*)&abort_flag = 1;
@@ -366,16 +361,13 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
                 long long v = ((sr[0] + sr[1]) + (sr[2] + sr[3])) + ((sr[4] + sr[5]) + (sr[6] + sr[7]));
                 v += __shfl_xor_sync(0xffffffffu, v, 16);
                 const long long x = __shfl_xor_sync(0xffffffffu, v, 8);   // lanes 0..7: hi sums here, cross sums there
-                if (lane < 8) add_y(cb * kSymT + 8 * warp + lane - p_lo, ((__int128)v << kLow) + x);
+                if (lane < 8) add_y(cb * kSymT + 8 * warp + lane - p_lo, fx96_part(v, x));
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the slot's next copy
             }
         }
         __syncwarp();   // every lane is done with the slot
-        if (lane == 0 && k + st < nt_cta && !*(volatile int*)&abort_flag) {
-            const Strip f = fx_entry(fill, warp);
-            issue_strip(f, tiles, wring + slot * kStripInts, &wfull[slot], pol);
-            flight |= (f.r0 < f.R ? 1u : 0u) << slot;
-        }
+        if (lane == 0 && k + st < nt_cta && !*(volatile int*)&abort_flag)
+            issue_strip(fx_entry(fill, warp), tiles, wring + slot * kStripInts, &wfull[slot], pol);
         if (k + st + 1 < nt_cta) fill = __ldg(lst + k + st + 1);
         ++cnt;
         if (++slot == st) slot = 0;
@@ -383,18 +375,18 @@ __global__ void __launch_bounds__(kT, 2) k_fxgemv(const SymDesc* __restrict__ de
     if (cur >= 0) flush_d(cur);
     __syncthreads();
     bad = abort_flag != 0;
-    if (bad) {   // let the copies still in flight land (bounded), then report
+    if (bad) {   // let the copies still in flight land (bounded; a slot may have none), then report
         if (lane == 0)
             for (int s = 0; s < st; ++s)
-                if ((flight >> s) & 1u) mbar_wait(&wfull[s], (phases >> s) & 1u);
+                for (unsigned k = 0; k < (1u << 16) && !mbar_done(&wfull[s], (phases >> s) & 1u); ++k) {}
         if (tid == 0) atomicExch(err, 1);
         __syncthreads();
     }
     // this CTA's partial sums in units of 2^d_i (NaN when x was not finite or a wait gave up)
-    const double unit = (bad || !finite) ? __longlong_as_double(0x7ff8000000000000ll) : pow2(X - 2 * kBits + kLow);
+    const double unit = (bad || !finite) ? __longlong_as_double(0x7ff8000000000000ll) : pow2(X - 2 * kBits + kFx96Unit);
     double* y = reinterpret_cast<double*>(ylo);
     for (int p = tid; p < np - p_lo; p += kT)   // 96 bits: the high 64 and the low 32
-        y[p] = fma((double)(long long)(((uint64_t)(uint32_t)yhi[p] << 32) | (ylo[p] >> 32)), 0x1p32, (double)(uint32_t)ylo[p]) * unit;
+        y[p] = fma((double)fx96_high(ylo[p], yhi[p]), 0x1p32, (double)fx96_low(ylo[p])) * unit;
     cluster.sync();
     const int rank = (int)cluster.block_rank();
     for (int p = r_lo + rank * kT + tid; p < np; p += cl * kT) {
