@@ -266,7 +266,7 @@ size_t dd_workspace_layout(dd_handle* h, bool assign) {
     L.take(d.K32, nc * (size_t)h->ldc);
     L.take(d.Pinv, (size_t)(h->n_sub + 1) * kNB * kNB);
     L.take(d.dinv, nm);
-    L.take(d.rpart, (size_t)(kMaxRestart + 4) * (size_t)h->n_sub);
+    L.take(d.rpart, (size_t)(2 * (kMaxRestart + 2) + 2) * (size_t)h->n_sub);
     for (int k = 0; k < 3; ++k) L.take(d.e[k], nd);
     for (int k = 0; k < 3; ++k) L.take(d.mu[k], nd);
     L.take(d.lam_adj, nm);

@@ -19,8 +19,9 @@
 // other sixteen already multiply by the new vector (the last product of a cycle is
 // dropped).  Every CTA adds the partial sums in the same fixed order, so all of them
 // take the same decisions and the result does not depend on scheduling.  Algorithm,
-// precisions and stopping rules are those of gmres.cu: FP32 vectors, FP64 dot totals,
-// least-squares problem and iterate.
+// precisions and stopping rules are those of gmres.cu: FP32 vectors, dot products in FP32 up
+// to 128 entries and beyond as in FP64 (sum2.h, partial_sum), FP64 least-squares problem and
+// iterate.
 //
 // Measured (GB300, FP32 solve of a step): 9.3 us per Arnoldi step on 128 subdomains with up
 // to 288 interface entries, 26 us as separate kernels in a graph (GEMV 10, Gram-Schmidt 6.7
@@ -40,6 +41,7 @@
 
 #include "cg_rows.h"
 #include "dd_internal.h"
+#include "sum2.h"
 #include "symtile.cuh"
 
 namespace {
@@ -60,7 +62,7 @@ struct ResArgs {
     float* zuf;           // published z (DP2)
     GmresScalars* gs;
     PcgScalars* sc;
-    double* partials;     // [2][kM1 + 1][gridDim.x]
+    double* partials;     // [2][kM1 + 1][gridDim.x] of two FP32 words, then [2][gridDim.x] in FP64
     int span, tile_floats, have_q, clustered;
 };
 
@@ -124,23 +126,28 @@ __device__ bool tiles_landed(uint64_t* bar, uint64_t* never, int first, int32_t*
     return *failed == 0;
 }
 
-// Sum of nb FP32 partial sums (a warp; lanes take q = lane, lane + 32, ...) as an integer in
-// units of 2^(*e - shift): exact down to 2^-53 (up to 512 CTAs; 2^-50 beyond) of the
-// largest, like an FP64 sum but off the two-lane FP64 pipe.  *e = 255 when one is not finite.
-__device__ __forceinline__ long long partial_sum(const float* part, int nb, int lane, int shift, int* e) {
+// Sum of nb partial sums of two FP32 words each (a warp; lanes take q = lane, lane + 32, ...)
+// as an integer in units of 2^(*e - shift): exact down to 2^-53 (up to 512 CTAs; 2^-50
+// beyond) of the largest, like an FP64 sum but off the two-lane FP64 pipe.  *e = 255 when
+// one is not finite.
+__device__ __forceinline__ long long partial_sum(const float2* part, int nb, int lane, int shift, int* e) {
     uint32_t mx = 0;
-    for (int q = lane; q < nb; q += 32) mx = max(mx, __float_as_uint(__ldcg(part + q)) & 0x7fffffffu);
+    for (int q = lane; q < nb; q += 32) mx = max(mx, __float_as_uint(__ldcg(part + q).x) & 0x7fffffffu);
     mx = __reduce_max_sync(0xffffffffu, mx);
     const int em = (int)(mx >> 23);
     *e = em;
-    long long v = 0;
-    for (int q = lane; q < nb; q += 32) {
-        const uint32_t w = __float_as_uint(__ldcg(part + q));
+    auto units = [&](float f) -> long long {
+        const uint32_t w = __float_as_uint(f);
         const int x = (int)((w >> 23) & 255u);
         const long long t = x ? (long long)((w & 0x7fffffu) | 0x800000u) : 0ll;   // subnormals count as zero
         const int sh = shift - (em - x);
         const long long u = sh >= 0 ? t << sh : (sh > -24 ? t >> -sh : 0ll);
-        v += (int32_t)w < 0 ? -u : u;
+        return (int32_t)w < 0 ? -u : u;
+    };
+    long long v = 0;
+    for (int q = lane; q < nb; q += 32) {
+        const float2 f = __ldcg(part + q);
+        v += units(f.x) + units(f.y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -380,13 +387,21 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
     const int shift = nb <= 512 ? 29 : 26;
     auto dots = [&](int s, int nv, bool norm, double* tot, float* totf) -> bool {
         const int nsum = nv + (norm ? 1 : 0);
-        float* part = reinterpret_cast<float*>(P.partials) + (size_t)s * (kM1 + 1) * nb;
+        float2* part = reinterpret_cast<float2*>(P.partials) + (size_t)s * (kM1 + 1) * nb;
         for (int k = warp; k < nsum; k += kW + 1) {
             const float* v = k < nv ? V + k * P.span : tm;
-            float p = 0.0f;
-            for (int q = lane; q < g; q += 32) p = fmaf(tm[q], v[q], p);
-            p = warp_sum(p);
-            if (lane == 0) part[(size_t)k * nb + b] = p;
+            Sum2 p{0.0f, 0.0f};
+            for (int q0 = 0; q0 < g; q0 += 128) {   // (no more than 128 products in FP32)
+                float f = 0.0f;
+#pragma unroll
+                for (int q = q0 + lane; q < q0 + 128; q += 32)
+                    if (q < g) f = fmaf(tm[q], v[q], f);
+                p = sum2_add(p, Sum2{f, 0.0f});
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                p = sum2_add(p, Sum2{__shfl_xor_sync(0xffffffffu, p.hi, o), __shfl_xor_sync(0xffffffffu, p.lo, o)});
+            if (lane == 0) part[(size_t)k * nb + b] = make_float2(p.hi, p.lo);
         }
         if (!grid_barrier<0>(meet)) return false;
         for (int k = warp; k < nsum; k += kW + 1) {
@@ -436,7 +451,7 @@ __global__ void __launch_bounds__(32 * W + 32, 16 / W) k_gm_resident(ResArgs P) 
                 }
             }
             __syncthreads();
-            double* part = P.partials + (size_t)(kM1 + 1) * nb;   // past the FP32 sets
+            double* part = P.partials + (size_t)2 * (kM1 + 1) * nb;   // past the FP32 sets
             if (tid < 2) {
                 double v = 0.0;
                 for (int w = 0; w < nw; ++w) v += red[tid][w];
