@@ -180,8 +180,11 @@ typedef struct {
  *            the row panel is scaled by a power of two and cut into seven 8-bit
  *            BF16 slices, the slice products of each weight class are summed
  *            exactly in FP32 tensor memory (tcgen05 MMAs) and the classes are
- *            combined in FP64 (an Ozaki splitting).  Results agree with the FP64
- *            path to FP64 rounding.  Read by dd_factor. */
+ *            combined in FP64 (an Ozaki splitting); so are the panels, from
+ *            eight slices.  Results agree with the FP64 path to FP64 rounding of
+ *            the scales of their rows and columns; single operator entries many
+ *            orders of magnitude below those scales keep fewer digits than the
+ *            FP64 path gives them.  Read by dd_factor. */
 typedef struct {
     int precision;
     double tol;

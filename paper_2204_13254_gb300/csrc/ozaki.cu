@@ -9,18 +9,24 @@
 // in BF16).  For two such vectors and every weight class d = p + q <= 6 the
 // products a_p b_q are summed over K = 64 and over the class's d + 1 pairs in one
 // FP32 accumulator in tensor memory: every partial sum is an integer below
-// 64 (2 2^15 + 5 2^14) < 2^24, so the accumulation is exact.  The classes are
+// 64 (2 2^15 + 6 2^14) < 2^24, so the accumulation is exact.  The classes are
 // joined in 64-bit integers (T, exact but for a rounding below 2^-62 of the
 // largest product) and scaled back with one conversion and one FP64 FMA.
 // Dropping the classes d >= 7 leaves an error below 2^-54 of |A_i||B_j| per term:
-// FP64 accuracy.
+// FP64 accuracy in the norm, not of every small element (an element far below the largest of
+// its row and column has correspondingly fewer digits; DD_FACTOR_FP64 keeps those).
+// The pivot rows k are scaled by powers of two before they are cut, D = diag(2^-s_k) with
+// D P D of diagonal 1/4 .. 1, and B' by the inverse: with materials of eight decades contrast
+// inside a pivot block the rows of the operator agree with an FP64 elimination to 2e-15 (nine
+// in ten), without D to 1.7e-14.  The panel's own product takes eight slices of each operand,
+// as B' becomes part of the operator: 1.5 % of a factorisation.
 //
 // Symmetry.  While a set K of indices has been swept, M_ij = M_ji when both or
 // none of i, j are in K and M_ij = -M_ji otherwise, so only the lower triangle is
 // kept (k_oz_mirror fills the rest at the end), and the column panel of a pivot
 // block p is its row panel B = M[p, :] transposed up to the sign s_i = -1 for
 // swept rows, +1 otherwise.  One pivot block is three kernels:
-//   k_oz_panel   slices of B; B' = -P^-1 B as a slice product; slices of B'; the
+//   k_oz_panel   slices of D B; B' = -P^-1 B as a slice product; slices of D^-1 B'; the
 //                row and column panels of M;
 //   k_oz_update  M_ij += s_i B_i . B'_j over the lower triangle outside p, and,
 //                in its first CTAs (one per matrix), P^-1 and its slices of the next
@@ -37,6 +43,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "dd_internal.h"
 #include "fixpoint.cuh"
@@ -44,14 +51,16 @@
 
 namespace {
 
-constexpr int kOzS = 7;                      // slices per operand (8 bits each)
+constexpr int kOzS = 7;                      // slices per operand (8 bits each) of the update
+constexpr int kOzPanS = 8;                   // of the panel's product
 constexpr int kOzRows = 128;                 // rows of a tile (MMA M)
 constexpr int kOzCols = 32;                  // columns of one unit of the update (MMA N)
 constexpr int kOzK = kOzNB;                  // pivot block width (MMA K = 4 x 16)
 constexpr uint32_t kOzPiece = kOzRows * kOzK * 2;    // 16 KB: one slice of a 128-row block
 constexpr uint32_t kOzBlock = kOzS * kOzPiece;       // 112 KB: the slices of a 128-row block
+constexpr uint32_t kOzPanBlock = kOzPanS * kOzPiece; // 128 KB: the same in the panel's shared memory
 constexpr uint32_t kOzPPiece = kOzK * kOzK * 2;      // 8 KB: one slice of P^-1
-constexpr uint32_t kOzPBlock = kOzS * kOzPPiece;     // 56 KB
+constexpr uint32_t kOzPBlock = kOzPanS * kOzPPiece;  // 64 KB
 constexpr uint32_t kOzUPiece = kOzCols * kOzK * 2;   // 4 KB: one slice of a 32-column unit
 constexpr uint32_t kOzUnit = kOzS * kOzUPiece;       // 28 KB
 constexpr unsigned kOzPolls = 1u << 22;
@@ -71,8 +80,22 @@ __device__ __forceinline__ long long to_digits(double v, int e) {
     const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
     const unsigned long long m =
         ((unsigned long long)(uint32_t)((hi & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(v);
-    const int r = min(1022 + e - ex, 63);   // >= 0; the value is (m 2^4 >> r) / 2
+    const unsigned r = min((unsigned)(1022 + e - ex), 63u);   // the value is (m 2^4 >> r) / 2
     const unsigned long long t = ex ? (((m << 4) >> r) + 1) >> 1 : 0ull;
+    return hi < 0 ? -(long long)t : (long long)t;
+}
+
+// The same with eight bits more: the integer t of to_digits and, in `low` (|low| <= 128), the
+// multiples of 2^-8 that it leaves.  Bits below those are dropped.
+__device__ __forceinline__ long long to_digits(double v, int e, int& low) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
+    const unsigned long long m =
+        ((unsigned long long)(uint32_t)((hi & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(v);
+    const unsigned r = (unsigned)(1022 + e - ex);   // the value is m 2^11 >> r in units of 2^-8
+    const unsigned long long t8 = ex && r < 64u ? (m << 11) >> r : 0ull;
+    const unsigned long long t = (t8 + 128) >> 8;   // (m 2^11 ends in eleven zeros: no carry out)
+    const int l = (int)(t8 - (t << 8));
+    low = hi < 0 ? -l : l;
     return hi < 0 ? -(long long)t : (long long)t;
 }
 
@@ -84,16 +107,23 @@ __device__ __forceinline__ double scale_exp(double v, int x) {
 }
 
 // Slices of eight consecutive elements v[0..7] (K direction) of a vector with
-// exponent e: one 16-byte chunk per slice, handed to put(slice, chunk).
-template <typename Put>
-__device__ __forceinline__ void cut8(const double* v, int e, Put put) {
-    uint32_t w[kOzS][4];
+// exponent e, scaled by 2^-x[0..7]: one 16-byte chunk per slice, handed to put(slice, chunk).
+template <int kS, typename Put>
+__device__ __forceinline__ void cut8(const double* v, int e, const int (&x)[8], Put put) {
+    uint32_t w[kS][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        uint32_t f[2][kOzS];
+        uint32_t f[2][kS];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const long long t = to_digits(v[2 * q + u], e);
+            long long t;
+            if constexpr (kS == 8) {
+                int low;
+                t = to_digits(v[2 * q + u], e + x[2 * q + u], low);
+                f[u][7] = small_float(low);
+            } else {
+                t = to_digits(v[2 * q + u], e + x[2 * q + u]);
+            }
             const unsigned long long b = (unsigned long long)t + 0x0000808080808080ull;   // balanced digits
             const uint32_t lo = (uint32_t)b, hi = (uint32_t)(b >> 32);
             f[u][6] = small_float((int)(lo & 255u) - 128);
@@ -105,27 +135,50 @@ __device__ __forceinline__ void cut8(const double* v, int e, Put put) {
             f[u][0] = small_float((int)hi >> 16);
         }
 #pragma unroll
-        for (int p = 0; p < kOzS; ++p) w[p][q] = __byte_perm(f[0][p], f[1][p], 0x7632);
+        for (int p = 0; p < kS; ++p) w[p][q] = __byte_perm(f[0][p], f[1][p], 0x7632);
     }
 #pragma unroll
-    for (int p = 0; p < kOzS; ++p) put(p, make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]));
+    for (int p = 0; p < kS; ++p) put(p, make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]));
 }
 
-// Eight columns of the seven class accumulators (stride `cls` tensor-memory columns
+// The high word of |v| 2^-x, for the largest of several: exponents compare as such (zero and
+// subnormal numbers below every other), and the exponent of the largest (0 where all are zero).
+constexpr int kOzNone = INT_MIN;
+__device__ __forceinline__ int scaled_hi(double v, int x) {
+    const int hi = __double2hiint(v) & 0x7fffffff;
+    return hi >> 20 ? hi - (x << 20) : kOzNone;
+}
+__device__ __forceinline__ int scaled_exp(int hi) { return hi == kOzNone ? 0 : (hi >> 20) - 1022; }
+// Eight scales of the pivot block's rows (a multiple of four integers).
+__device__ __forceinline__ void load_scales(const int32_t* p, int (&x)[8]) {
+    const int4 a = __ldg(reinterpret_cast<const int4*>(p)), b = __ldg(reinterpret_cast<const int4*>(p) + 1);
+    x[0] = a.x;
+    x[1] = a.y;
+    x[2] = a.z;
+    x[3] = a.w;
+    x[4] = b.x;
+    x[5] = b.y;
+    x[6] = b.z;
+    x[7] = b.w;
+}
+
+// Eight columns of the panel's eight class accumulators (stride `cls` tensor-memory columns
 // apart) of the warp's 32 lanes, all loads in flight together.
-__device__ __forceinline__ void ld_classes(uint32_t t, uint32_t cls, uint32_t (&r)[kOzS][8]) {
+__device__ __forceinline__ void ld_classes(uint32_t t, uint32_t cls, uint32_t (&r)[kOzPanS][8]) {
 #define OZ_O(d) "=r"(r[d][0]), "=r"(r[d][1]), "=r"(r[d][2]), "=r"(r[d][3]), "=r"(r[d][4]), "=r"(r[d][5]), "=r"(r[d][6]), "=r"(r[d][7])
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%56];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%57];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%58];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%59];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%60];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%61];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%48,%49,%50,%51,%52,%53,%54,%55}, [%62];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%64];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%65];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%66];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%67];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%68];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%69];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%48,%49,%50,%51,%52,%53,%54,%55}, [%70];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%56,%57,%58,%59,%60,%61,%62,%63}, [%71];\n"
         "tcgen05.wait::ld.sync.aligned;\n"
-        : OZ_O(0), OZ_O(1), OZ_O(2), OZ_O(3), OZ_O(4), OZ_O(5), OZ_O(6)
-        : "r"(t), "r"(t + cls), "r"(t + 2 * cls), "r"(t + 3 * cls), "r"(t + 4 * cls), "r"(t + 5 * cls), "r"(t + 6 * cls)
+        : OZ_O(0), OZ_O(1), OZ_O(2), OZ_O(3), OZ_O(4), OZ_O(5), OZ_O(6), OZ_O(7)
+        : "r"(t), "r"(t + cls), "r"(t + 2 * cls), "r"(t + 3 * cls), "r"(t + 4 * cls), "r"(t + 5 * cls), "r"(t + 6 * cls),
+          "r"(t + 7 * cls)
         : "memory");
 #undef OZ_O
 }
@@ -152,11 +205,13 @@ __device__ __forceinline__ void ld_classes_pairs(uint32_t t, uint32_t cls, uint3
 }
 
 // T of one element: sum_d D_d 2^(8 (5-d)) ... in units of 2^-40 of class 0, i.e. the
-// product is T 2^(e + f - 56) (|T| < 2^63; class 6 rounded in, see the file comment).
-__device__ __forceinline__ double join_classes(const uint32_t (&r)[kOzS][8], int c) {
+// product is T 2^(e + f - 56) (|T| < 2^63; classes 6 and 7 rounded in, see the file comment).
+template <int kS>
+__device__ __forceinline__ double join_classes(const uint32_t (&r)[kS][8], int c) {
     auto I = [&](int d) { return (long long)__float2int_rn(__uint_as_float(r[d][c])); };
     const long long H = (I(0) << 16) + (I(1) << 8) + I(2);
-    const long long L = (I(3) << 24) + (I(4) << 16) + (I(5) << 8) + I(6);
+    long long L = (I(3) << 24) + (I(4) << 16) + (I(5) << 8) + I(6);
+    if constexpr (kS == 8) L += (I(7) + 128) >> 8;
     return (double)((H << 24) + ((L + 128) >> 8));
 }
 
@@ -211,18 +266,19 @@ __device__ __forceinline__ void oz_bulk(void* dst, const void* src, uint32_t byt
         : "memory");
 }
 
-// The 28 slice products of A rows (slices at a0, kOzPiece bytes apart) and `cls` B rows (slices
+// The kS (kS + 1) / 2 slice products of A rows (slices at a0, kOzPiece bytes apart) and `cls` B rows (slices
 // at b0, one after the other) into the class accumulators at `acc`, `cls` columns apart.
 // For one slice p of A the classes p + q lie side by side, and so do the slices q of B: one
 // MMA takes as many q as N = 256 columns allow.  An MMA reads its 128 x 16 A operand from
 // shared memory whatever N is, which at N = 32 takes four times the product itself (measured,
 // per-block means: update 384 -> 367 us, panel 77 -> 72 us against 112 MMAs of N = 32 per unit).
+template <int kS>
 __device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, uint32_t b0) {
     const int qmax = 256 / cls;
     const uint32_t sb = (uint32_t)cls * kOzK * 2;
-    for (int p = 0; p < kOzS; ++p)
-        for (int q = 0; q < kOzS - p; q += qmax) {
-            const int nq = min(qmax, kOzS - p - q);
+    for (int p = 0; p < kS; ++p)
+        for (int q = 0; q < kS - p; q += qmax) {
+            const int nq = min(qmax, kS - p - q);
             const uint32_t idesc = tc::idesc_bf16_f32(kOzRows, nq * cls);
             for (int ks = 0; ks < kOzK / 16; ++ks) {
                 const uint64_t ad = tc::smem_desc(a0 + p * kOzPiece + ks * 256, 128, (kOzK / 8) * 128);
@@ -234,23 +290,26 @@ __device__ __forceinline__ void oz_products(uint32_t acc, int cls, uint32_t a0, 
 
 // ---- pivot block -------------------------------------------------------------
 // P^-1 of the pivot block, one CTA per matrix.
-//  * A first X by a Gauss-Jordan sweep in FP32 (SPD: no pivoting; the block scaled by powers of
-//    two to a diagonal in [1/4, 1)).
+//  * All on D P D, whose inverse D^-1 P^-1 D^-1 is called X here.
+//  * A first X by a Gauss-Jordan sweep in FP32 (SPD: no pivoting).
 //  * Newton: R = I - P X from exact 57-bit fixed-point sums, X += X R in FP32, twice as a rule (|R| is 2^-20,
 //    then 2^-41): X ends at its own FP64 rounding.
 //  * A block that FP32 does not serve (a pivot that is not positive, |R| >= 2^-5, or >= 2^-36 at
 //    the second look: the contraction is 2^-24 of the condition number) is swept in FP64 and
 //    taken as swept, in full: its errors are those of a nearby block, which cancel in the
 //    panels, while with growing condition number a rounded symmetric X loses more and more of
-//    it (measured, coupled operator, condition number of A_rr 3e3: 3e-13 and 2e-12).
+//    it (measured, coupled operator, condition number of A_rr 3e3: 3e-13 and 2e-12).  Eight
+//    meshes of 5 to 9 cells a side against an extended-precision reference, geometric mean,
+//    with time steps that make the condition number 1e3 .. 3e5: 1.8e-13, 2.9e-12, 1.7e-11,
+//    6.2e-11; FP64 elimination 1.6e-13, 3.0e-12, 1.6e-11, 5.5e-11.
 // With the FP64 sweep for every block, and one correction, 173 us (its FMAs alone 124 us: the
 // FP64 pipe), with this 76 us (40 matrices).  The sweep's 64 roundings per element would be the
 // largest error of a well-conditioned elimination (the products are exact to 2^-54).  Measured,
 // coupled operator against an extended-precision reference, seven meshes (six bisected into
-// 139 to 600 uneven subdomains): 2.3e-16 .. 3.8e-16; with the FP64 sweep alone 2.9e-16 ..
+// 139 to 600 uneven subdomains): 1.9e-16 .. 3.5e-16; with the FP64 sweep alone 2.9e-16 ..
 // 4.5e-16, with 32-wide pivot blocks in plain FP64 2.5e-16 .. 4.0e-16.
-// Writes P^-1 back into M[p, p] (the panel kernel does not read that block), and its slices
-// and exponents.
+// Writes P^-1 back into M[p, p] (the panel kernel does not read that block), and the slices of
+// P^-1 D^-1, their exponents and the exponents of D.
 constexpr int kOzPivThreads = 256;
 constexpr int kPs = kOzK + 1;   // row stride in shared memory
 
@@ -373,6 +432,12 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
                 a[u][v] = (i < nb && j <= i) ? A[(int64_t)i * md.ld + j] : 0.0;
             }
     };
+    auto scale = [&]() {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v) a[u][v] *= pow2n(-sd[ty + 16 * u] - sd[tx + 16 * v]);
+    };
     // the lower triangle in registers -> the full symmetric block in Q (zero outside nb)
     auto spread = [&]() {
 #pragma unroll
@@ -406,17 +471,22 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
             for (int k = 0; k < 16; ++k) put(qc(k), split57(Q[ri * kPs + qc(k)], x));
         }
     };
+    // P from here on is D P D with D = diag(2^-sd), its diagonal in [1/4, 1) (D = 1 where an exponent
+    // is far out), and X its inverse
     load();
+    const int dx = tid < nb ? (exp_of_hi(__double2hiint(A[(int64_t)tid * md.ld + tid]) & 0x7fffffff) + 1) >> 1 : 0;
+    const int far = __syncthreads_or(abs(dx) > 200);
+    if (tid < kOzK) sd[tid] = far ? 0 : dx;
+    __syncthreads();
+    scale();
     spread();
     {
         const int e = row_exp();
         rp[ri] = e;
         split_row(e, [&](int c, int2 w) { Pi[ri * kPs + c] = w; });
-        sd[ri] = ri < nb ? (exp_of_hi(__double2hiint(Q[ri * kPs + ri]) & 0x7fffffff) + 1) >> 1 : 0;
     }
-    // X = D (D P D)^-1 D with D = diag(2^-sd); zero, so that the FP64 sweep follows, where an
-    // exponent is far out or a pivot was not positive
-    const int far = __syncthreads_or(abs(sd[ri]) > 500);
+    __syncthreads();
+    // X = 0, so that the FP64 sweep follows, where an exponent is far out or a pivot was not positive
     float* F = reinterpret_cast<float*>(Xi);   // [kOzK][kPs]
     if (!far) {
         float f[4][4];
@@ -425,7 +495,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 const int i = ty + 16 * u, j = 4 * tx + v;
-                f[u][v] = (float)(Q[i * kPs + j] * pow2n(-sd[i] - sd[j]));
+                f[u][v] = (float)Q[i * kPs + j];
                 if (i == j && i >= nb) f[u][v] = 1.0f;
             }
         const bool ok = sweep32(f, sw, nb, tid);
@@ -439,7 +509,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
 #pragma unroll
             for (int v = 0; v <= u; ++v) {
                 const int i = ty + 16 * u, j = tx + 16 * v;
-                a[u][v] = (double)F[i * kPs + j] * pow2n(-sd[i] - sd[j]);
+                a[u][v] = (double)F[i * kPs + j];
             }
     } else {
 #pragma unroll
@@ -490,6 +560,7 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
         const int any2 = __syncthreads_or(big == 2), any1 = __syncthreads_or(big >= 1);
         if (any2 || (any1 && pass == 1)) {
             load();
+            scale();
             spread();
             if (!sweep64(Q, nb, tid) && tid == 0) atomicCAS(status, 0, DD_ERR_NOT_SPD);
             swept = true;
@@ -522,18 +593,22 @@ __device__ __forceinline__ void pivot_block(const MatDesc& md, double* __restric
     if (!swept) spread();
     for (int p = tid; p < kOzK * kOzK; p += kOzPivThreads) {
         const int i = p >> 6, j = p & 63;
-        if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i * kPs + j];
+        if (i < nb && j <= i) A[(int64_t)i * md.ld + j] = Q[i * kPs + j] * pow2n(-sd[i] - sd[j]);
     }
     // slices
     const int e = row_exp();
-    if (rq == 0) ep[(int64_t)m * kOzK + ri] = e;
+    if (rq == 0) {
+        ep[(int64_t)m * 2 * kOzK + ri] = e - sd[ri];
+        ep[(int64_t)m * 2 * kOzK + kOzK + ri] = sd[ri];
+    }
     unsigned char* out = reinterpret_cast<unsigned char*>(Ps) + (int64_t)m * kOzPBlock;
     for (int g = 0; g < 2; ++g) {
         const int k = 16 * rq + 8 * g;
         double v[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] = Q[ri * kPs + k + c];
-        cut8(v, e, [&](int p, uint4 w) {
+        const int none[8] = {};
+        cut8<kOzPanS>(v, e, none, [&](int p, uint4 w) {
             *reinterpret_cast<uint4*>(out + p * kOzPPiece + tc::kmajor_off(ri, k, kOzK)) = w;
         });
     }
@@ -555,9 +630,9 @@ __global__ void __launch_bounds__(kOzPivThreads, 1) k_oz_pivot(const MatDesc* __
 // in shared memory (the MMA's A operand) and in global memory (the update's rows); the
 // slice product with P^-1 gives B' = -P^-1 B, which is written back to the row panel
 // (j < k0) or, negated, to the column panel (j >= k0 + nb), and cut into slices again
-// (the update's columns).  168 KB of shared memory, 448 tensor-memory columns.
+// (the update's columns).  192 KB of shared memory, 512 tensor-memory columns.
 constexpr int kOzPanThreads = 256;
-constexpr size_t kOzPanSmem = kOzBlock + kOzPBlock + 64;
+constexpr size_t kOzPanSmem = kOzPanBlock + kOzPBlock + 64;
 __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __restrict__ mats, double* __restrict__ M,
                                                                int k0, int nrb, const uint16_t* __restrict__ Ps,
                                                                const int32_t* __restrict__ ep, uint16_t* __restrict__ Bs,
@@ -570,7 +645,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     const int nb = min(kOzK, md.nr - k0);
     extern __shared__ __align__(128) unsigned char sm[];
     unsigned char* sB = sm;
-    unsigned char* sP = sm + kOzBlock;
+    unsigned char* sP = sm + kOzPanBlock;
     uint64_t* bars = reinterpret_cast<uint64_t*>(sP + kOzPBlock);   // [0] P^-1 slices, [1] products
     uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
     __shared__ int xmax[2][kOzRows];
@@ -589,7 +664,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     const bool row = j < k0;   // stored in the row panel
     double* A = M + md.moff;
     double v[32];
-    int mx = 0;
+    int mx = kOzNone;
     // below the block a thread's values are contiguous: 16-byte accesses
     double2* const col = reinterpret_cast<double2*>(A + (int64_t)j * md.ld + k0 + kb);
     if (on && !row) {
@@ -605,23 +680,32 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = on && kb + k < nb ? A[(int64_t)(k0 + kb + k) * md.ld + j] : 0.0;
     }
+    const int32_t* const epm = ep + (int64_t)m * 2 * kOzK;   // exponents of the rows of P^-1 D^-1, then sd
+    const int32_t* const sdm = epm + kOzK + kb;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) mx = max(mx, __double2hiint(v[k]) & 0x7fffffff);
+    for (int g = 0; g < 4; ++g) {
+        int x[8];
+        load_scales(sdm + 8 * g, x);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) mx = max(mx, scaled_hi(v[8 * g + c], x[c]));
+    }
     xmax[half][r] = mx;
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
     const int64_t blk = ((int64_t)m * nrb + rb) * kOzBlock;
-    const int e = exp_of_hi(max(xmax[0][r], xmax[1][r]));
-    {
+    const int e = scaled_exp(max(xmax[0][r], xmax[1][r]));
+    {   // D B
         unsigned char* gB = reinterpret_cast<unsigned char*>(Bs) + blk;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const uint32_t o = tc::kmajor_off(r, kb + 8 * g, kOzK);
-            cut8(v + 8 * g, e, [&](int p, uint4 w) {
+            int x[8];
+            load_scales(sdm + 8 * g, x);
+            cut8<kOzPanS>(v + 8 * g, e, x, [&](int p, uint4 w) {
                 *reinterpret_cast<uint4*>(sB + p * kOzPiece + o) = w;
-                *reinterpret_cast<uint4*>(gB + p * kOzPiece + o) = w;
+                if (p < kOzS) *reinterpret_cast<uint4*>(gB + p * kOzPiece + o) = w;
             });
         }
     }
@@ -633,7 +717,7 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
         ok = oz_first_wait(sc->wait_first, &bars[1]) && oz_wait(&bars[0], 0u);
         if (ok) {
             tc::fence_after_sync();
-            oz_products(tmem, kOzK, tc::smem_addr(sB), tc::smem_addr(sP));
+            oz_products<kOzPanS>(tmem, kOzK, tc::smem_addr(sB), tc::smem_addr(sP));
         }
         tc::mma_commit(&bars[1]);
     }
@@ -641,17 +725,19 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     tc::fence_after_sync();
     const bool good = __syncthreads_and(done && ok) != 0;
     if (good) {
-        mx = 0;
+        mx = kOzNone;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            uint32_t D[kOzS][8];
+            int x[8];
+            load_scales(sdm + 8 * g, x);
+            uint32_t D[kOzPanS][8];
             ld_classes(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + kb + 8 * g, kOzK, D);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int i = kb + 8 * g + c;
-                const double y = -scale_exp(join_classes(D, c), e + ep[(int64_t)m * kOzK + i] - 56);
+                const double y = -scale_exp(join_classes(D, c), e + epm[i] - 56);
                 v[8 * g + c] = y;
-                mx = max(mx, __double2hiint(y) & 0x7fffffff);
+                mx = max(mx, scaled_hi(y, -x[c]));
             }
         }
         if (on && row) {
@@ -669,13 +755,17 @@ __global__ void __launch_bounds__(kOzPanThreads, 1) k_oz_panel(const MatDesc* __
     xmax[half][r] = mx;   // the first exchange was read before the previous barriers
     __syncthreads();
     if (good) {
-        const int f = exp_of_hi(max(xmax[0][r], xmax[1][r]));
+        const int f = scaled_exp(max(xmax[0][r], xmax[1][r]));   // of D^-1 B'
         if (half == 0 && j < md.ns) ec[(int64_t)m * nmax + j] = f;
         unsigned char* gC = reinterpret_cast<unsigned char*>(Cs) + blk;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const uint32_t o = tc::kmajor_off(r, kb + 8 * g, kOzK);
-            cut8(v + 8 * g, f, [&](int p, uint4 w) { *reinterpret_cast<uint4*>(gC + p * kOzPiece + o) = w; });
+            int x[8];
+            load_scales(sdm + 8 * g, x);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) x[c] = -x[c];
+            cut8<kOzS>(v + 8 * g, f, x, [&](int p, uint4 w) { *reinterpret_cast<uint4*>(gC + p * kOzPiece + o) = w; });
         }
     } else if (tid == 0) {
         atomicExch(&sc->wait_err, 1);
@@ -809,7 +899,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_update(const MatDesc* __re
             return;
         }
         tc::fence_after_sync();
-        oz_products(tmem + 256u * hh, kOzCols, tc::smem_addr(sA), tc::smem_addr(sC + s * kOzUnit));
+        oz_products<kOzS>(tmem + 256u * hh, kOzCols, tc::smem_addr(sA), tc::smem_addr(sC + s * kOzUnit));
         tc::mma_commit(&tfull[hh]);
         tc::mma_commit(&empty[s]);
     };
@@ -958,7 +1048,7 @@ OzLayout oz_layout(int nm, int nmax) {
     L.bs = L.ps + up((size_t)nm * kOzPBlock);
     L.cs = L.bs + up((size_t)nm * nrb * kOzBlock);
     L.ep = L.cs + up((size_t)nm * nrb * kOzBlock);
-    L.eb = L.ep + up((size_t)nm * kOzK * sizeof(int32_t));
+    L.eb = L.ep + up((size_t)nm * 2 * kOzK * sizeof(int32_t));
     L.ec = L.eb + up((size_t)nm * nmax * sizeof(int32_t));
     L.total = L.ec + up((size_t)nm * nmax * sizeof(int32_t));
     return L;
