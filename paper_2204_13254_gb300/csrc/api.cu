@@ -117,6 +117,11 @@ struct Prof {
             if (a) cudaEventRecord(a, s);
         }
     }
+    // n of the announced launches did not happen
+    void none(int n) {
+        h->launches[stage] -= n;
+        h->total_launches -= n;
+    }
     ~Prof() {
         if (on && i0 + 1 < h->ev_used) {
             cudaEventRecord((cudaEvent_t)h->ev_pool[i0 + 1], s);
@@ -495,8 +500,9 @@ int pcg_vectors(dd_handle* h, const Vecs& V, unsigned long long cond, cudaStream
         bool whole = false;
         const int rc = launch_pcg_step(h, V.wf, V.pf, V.zf, V.lamf, cond, &whole, s);
         if (rc || whole) return rc;
+        P.none(1);
     }
-    Prof P(h, ST_VEC, s, 1);
+    Prof P(h, ST_VEC, s, 2);
     const int rc = launch_pcg_alpha(h, V.wf, V.pf, s);
     return rc ? rc : launch_pcg_update(h, V.zf, V.lamf, cond, s);
 }
@@ -677,8 +683,9 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
             bool whole = false;
             CK(h, launch_gm_step(h, U, V.wf, zuf, cond_inner, &whole, st), "gmres step");
             if (whole) return DD_OK;
+            P.none(1);
         }
-        Prof P(h, ST_VEC, st, 2);
+        Prof P(h, ST_VEC, st, 3);
         CK(h, launch_gm_pass(h, U, 0, V.wf, zuf, 0ull, st), "gmres pass 0");
         CK(h, launch_gm_pass(h, U, 1, V.wf, zuf, cond_inner, st), "gmres pass 1");
         CK(h, launch_gm_normalize(h, U, zuf, st), "gmres normalize");
@@ -689,11 +696,12 @@ int gmres_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, doub
     if (prec == DD_MIXED && h->prm.sym_fp32)
         CK(h, launch_gm_resident(h, U, 0, h->prm.restart, true, &resident, s), "resident gmres");
     if (resident) {
-        {
-            Prof P(h, ST_VEC, s, 2);
-            CK(h, launch_gm_init(h, tol, h->prm.max_it, h->prm.restart, h->capturing ? adaptive : 0, 0ull, s), "gmres init");
-            CK(h, launch_gm_resident(h, U, use_warm ? 1 : 0, h->prm.restart, false, &resident, s), "resident gmres");
-        }
+        Prof P(h, ST_VEC, s, 2);
+        CK(h, launch_gm_init(h, tol, h->prm.max_it, h->prm.restart, h->capturing ? adaptive : 0, 0ull, s), "gmres init");
+        CK(h, launch_gm_resident(h, U, use_warm ? 1 : 0, h->prm.restart, false, &resident, s), "resident gmres");
+        if (!resident) P.none(1);
+    }
+    if (resident) {
         h->lam_valid = true;
         if (h->capturing) {
             Prof P(h, ST_VEC, s, 1);
@@ -876,6 +884,7 @@ int dd_solve(dd_handle* h, int prec, double tol, bool warm, int* it_out, double*
         {
             Prof P(h, ST_VEC, s, 1);
             CK(h, launch_cg_resident(h, prec, tol, use_warm ? 1 : 0, h->capturing ? adaptive : 0, &resident, s), "resident cg");
+            if (!resident) P.none(1);
         }
         if (resident) {
             h->lam_valid = true;

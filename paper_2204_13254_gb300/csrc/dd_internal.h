@@ -653,6 +653,11 @@ struct CopyParts {
         n[k++] = (int64_t)(bytes / 4);
     }
 };
+// Outcome of a launch that needs all its CTAs on the device at once (cooperative, or one
+// cluster): *ran = false, and no error left behind, where the stream does not offer that (a
+// stream of a green context, say, has a part of the multiprocessors); the kernels that need no
+// such launch serve then.
+int launch_or_decline(int e, bool* ran);
 int launch_copy_parts(const CopyParts& c, void* stream);
 int launch_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, float* lamf, unsigned long long cond,
                     bool* ran, void* stream);

@@ -1018,15 +1018,16 @@ int run_step(const dd_handle* h, const UView& U, const float* wf, float* zuf, un
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     const UIn in{d.zu, U.n2 ? d.zu + U.n1 : d.zu, zuf, (zuf && U.n2) ? zuf + U.n1 : zuf};
-    *ran = true;
-    return (int)cudaLaunchKernelEx(&cfg, k_gm_step<kSt, E, VT>, U, (const double*)d.w, wf, in, reinterpret_cast<VT*>(d.Vk),
-                                   h->gm_ldv, wf ? nullptr : d.zu, zuf, d.gs, d.sc, d.gpart, cond);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gm_step<kSt, E, VT>, U, (const double*)d.w, wf, in,
+                                             reinterpret_cast<VT*>(d.Vk), h->gm_ldv, wf ? nullptr : d.zu, zuf, d.gs, d.sc,
+                                             d.gpart, cond);
+    return launch_or_decline((int)e, ran);
 }
 }  // namespace
 
-// The vector part of an Arnoldi step as one kernel where the vectors fit one CTA of 256
-// threads and eight elements a thread on every SM (311,000 unknowns on 152); *ran = false, and
-// nothing launched, beyond.
+// The vector part of an Arnoldi step as one kernel where the vectors fit one CTA of 512
+// threads and four elements a thread on every SM (311,000 unknowns on 152) and the launch is to
+// be had; *ran = false, and nothing launched, otherwise.
 int launch_gm_step(const dd_handle* h, const UView& U, const float* wf, float* zuf, unsigned long long cond_inner,
                    bool* ran, void* stream) {
     *ran = false;

@@ -1422,6 +1422,13 @@ int launch_refine_cond(const dd_handle* h, unsigned long long cond, void* stream
     return (int)cudaGetLastError();
 }
 
+int launch_or_decline(int e, bool* ran) {
+    *ran = e == (int)cudaSuccess;
+    if (e != (int)cudaErrorCooperativeLaunchTooLarge && e != (int)cudaErrorLaunchOutOfResources) return e;
+    cudaGetLastError();
+    return 0;
+}
+
 int launch_copy_parts(const CopyParts& c, void* stream) {
     int64_t most = 0;
     for (int q = 0; q < c.k; ++q) most = std::max(most, (c.n[q] + 3) / 4);
@@ -1433,7 +1440,7 @@ int launch_copy_parts(const CopyParts& c, void* stream) {
 namespace {
 template <int E>
 int run_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, float* lamf, unsigned long long cond,
-                 cudaStream_t st) {
+                 bool* ran, cudaStream_t st) {
     const DevPtrs& d = h->d;
     const int64_t nl = (int64_t)h->mult_dof.size();
     cudaLaunchConfig_t cfg = {};
@@ -1445,24 +1452,25 @@ int run_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, floa
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return (int)cudaLaunchKernelEx(&cfg, k_pcg_step<E>, nl, (const int64_t*)d.mult_slot, (const double*)d.w, wf,
-                                   h->prm.precond ? (const double*)d.dinv : (const double*)nullptr, d.p, pf, d.lam, d.r,
-                                   d.z, zf, lamf, d.sc, d.partials, cond, h->prm.max_it);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_pcg_step<E>, nl, (const int64_t*)d.mult_slot, (const double*)d.w, wf,
+                                             h->prm.precond ? (const double*)d.dinv : (const double*)nullptr, d.p, pf,
+                                             d.lam, d.r, d.z, zf, lamf, d.sc, d.partials, cond, h->prm.max_it);
+    return launch_or_decline((int)e, ran);
 }
 }  // namespace
 
 // The vector part of a CG iteration as one kernel where two CTAs of 256 threads and four
-// elements a thread on every SM hold the vectors (311,000 multipliers on 152); *ran = false,
-// and nothing launched, beyond.
+// elements a thread on every SM hold the vectors (311,000 multipliers on 152) and the launch is
+// to be had; *ran = false, and nothing launched, otherwise.
 int launch_pcg_step(const dd_handle* h, const float* wf, float* pf, float* zf, float* lamf, unsigned long long cond,
                     bool* ran, void* stream) {
     const int64_t nl = (int64_t)h->mult_dof.size();
     const int64_t cap = kThreads * (int64_t)std::min(2 * h->n_sm, kMaxPartials / 4);
-    *ran = nl <= 4 * cap;
-    if (!*ran) return 0;
-    if (nl <= cap) return run_pcg_step<1>(h, wf, pf, zf, lamf, cond, S(stream));
-    if (nl <= 2 * cap) return run_pcg_step<2>(h, wf, pf, zf, lamf, cond, S(stream));
-    return run_pcg_step<4>(h, wf, pf, zf, lamf, cond, S(stream));
+    *ran = false;
+    if (nl > 4 * cap) return 0;
+    if (nl <= cap) return run_pcg_step<1>(h, wf, pf, zf, lamf, cond, ran, S(stream));
+    if (nl <= 2 * cap) return run_pcg_step<2>(h, wf, pf, zf, lamf, cond, ran, S(stream));
+    return run_pcg_step<4>(h, wf, pf, zf, lamf, cond, ran, S(stream));
 }
 
 int launch_pcg_alpha(const dd_handle* h, const float* wf, float* pf, void* stream) {

@@ -907,8 +907,11 @@ struct Launch {
     bool plan(const dd_handle* h, Kern kern, int threads, size_t smem) {
         cudaFuncAttributes fa;
         if (smem > 227 * 1024) return false;
-        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || smem + fa.sharedSizeBytes > 227 * 1024) return false;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || smem + fa.sharedSizeBytes > 227 * 1024 ||
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
         cfg.gridDim = dim3((unsigned)h->n_sub);
         cfg.blockDim = dim3((unsigned)threads);
         cfg.dynamicSmemBytes = smem;
@@ -926,7 +929,10 @@ struct Launch {
         at[0].id = cudaLaunchAttributeCooperative;
         at[0].val.cooperative = 1;
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess) return false;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
         return (int64_t)per_sm * h->n_sm >= h->n_sub;
     }
 };
@@ -938,7 +944,7 @@ bool res_candidate(const dd_handle* h) {
 }  // namespace
 
 // Runs the coupled GMRES (after k_gm_init) in its resident form; *ran = false, and nothing
-// launched, where it does not apply.  Sixteen product warps first (one CTA per SM), then
+// launched, where it does not apply or the launch is not to be had.  Sixteen product warps first (one CTA per SM), then
 // eight, then four, for the first with which every subdomain finds a CTA of its own.
 int launch_gm_resident(const dd_handle* h, const UView& U, int have_q, int m, bool probe, bool* ran, void* stream) {
     *ran = false;
@@ -968,7 +974,7 @@ int launch_gm_resident(const dd_handle* h, const UView& U, int have_q, int m, bo
         if (probe) return 0;
         P.clustered = L.clustered ? 1 : 0;
         L.cfg.stream = S(stream);
-        return (int)cudaLaunchKernelEx(&L.cfg, kern, P);
+        return launch_or_decline((int)cudaLaunchKernelEx(&L.cfg, kern, P), ran);
     }
     return 0;
 }
@@ -1022,8 +1028,7 @@ int launch_cg_resident(const dd_handle* h, int prec, double tol, int have_q, int
             if (e != cudaSuccess) return (int)e;
         }
         L.cfg.stream = S(stream);
-        *ran = true;
-        return (int)cudaLaunchKernelEx(&L.cfg, kern, P);
+        return launch_or_decline((int)cudaLaunchKernelEx(&L.cfg, kern, P), ran);
     }
     return 0;
 }
