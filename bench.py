@@ -41,6 +41,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "DD field-solve steps/s, mixed vs FP64 at rel err 1e-8; % of HBM/tensor roofline"
 FALLBACK_HBM_GBS = 6800.0
+FP64_NOMINAL_TFLOPS = 1.25   # nominal GB300 FP64 rate (CUDA-core FMA)
 
 
 def parse():
@@ -827,15 +828,25 @@ def stage_table(prof, K):
     return out
 
 
-def _fp64_roofline(st64, peak_gbs, peak_kind):
-    """FP64 path: the dominant GEMV reads packed symmetric tiles in 64-bit fixed point
-    (integer multiply-adds in place of GB300's two FP64 FMAs per clock and SM)."""
+def _fp64_roofline(st64, gemv_bytes, kind_of_stage, peak_gbs, peak_kind, fp64_tflops):
+    """FP64 path, by the form of its dominant GEMV: packed symmetric tiles in 64-bit fixed point
+    (k_fxgemv: integer multiply-adds, held against the HBM copy rate although instruction latency
+    bounds it), or dense rows (k_gemv<double>: GB300's two FP64 FMAs per clock and SM, 2 flops per
+    8-byte element, against the FMA rate measured in the same run)."""
     cand = {k: v for k, v in st64.items() if k not in ("vector", "factor") and v.get("achieved_GBs")}
     if not cand:
         return None
     dom = max(cand, key=lambda k: cand[k]["ms_per_step"])
     gbs = cand[dom]["achieved_GBs"]
-    return {"bound": "hbm", "kernel": f"k_fxgemv ({dom})", "achieved": gbs, "peak": peak_gbs, "unit": "GB/s",
+    alg, streamed = gemv_bytes.get(kind_of_stage.get(dom), (0.0, 0.0))
+    if alg == streamed:   # the dense form streams what it has to
+        gflops = gbs / 8.0 * 2.0
+        peak = (fp64_tflops or FP64_NOMINAL_TFLOPS) * 1e3
+        return {"bound": "alu", "kernel": f"k_gemv<double> ({dom})", "achieved": gflops, "peak": peak, "unit": "GFLOP/s",
+                "frac": gflops / peak,
+                "peak_source": ("measured in this run: dd_measure_fp64_rate (FMA chains on every SM, CUDA events)"
+                                if fp64_tflops else "nominal GB300 FP64 rate (1.25 TFLOP/s)")}
+    return {"bound": "instruction latency", "kernel": f"k_fxgemv ({dom})", "achieved": gbs, "peak": peak_gbs, "unit": "GB/s",
             "frac": gbs / peak_gbs, "peak_source": f"{peak_kind} hbm_gbs"}
 
 
@@ -976,7 +987,7 @@ def main():
         "rel_err_mixed_vs_fp64": r["rel"],
         "setup_s": r["t_setup"], "factor_s": r["t_factor"], "autotune_s": r["t_tune"],
         "gemv_tiles": r["tiles"],
-        "fp64_roofline": _fp64_roofline(st64, peak, peak_kind),
+        "fp64_roofline": _fp64_roofline(st64, r["gemv_bytes"]["fp64"], kind_of_stage, peak, peak_kind, r["fp64_tflops"]),
         "fp64_fma_tflops_measured": r["fp64_tflops"],
         "roofline": {"bound": "hbm", "kernel": (f"{packed_kernel(r['tiles'], dom, args.solver)} (packed FP32 tiles, {dom})"
                                                 if head == "mixed" and not args.no_sym and dom in ("local_solve", "iface_apply")

@@ -132,7 +132,7 @@ struct Prof {
 
 // algorithmic bytes of one full GEMV launch of `mode` at precision `prec`
 double mb(const dd_handle* h, int mode, int prec) {
-    if (prec != DD_MIXED) return fx_active(h, mode) ? 2.0 * h->mode_bytes_sym[mode] : h->mode_bytes[mode];
+    if (prec != DD_MIXED) return fx_built(h, mode) ? 2.0 * h->mode_bytes_sym[mode] : h->mode_bytes[mode];
     if (h->prm.sym_fp32 && h->sym_ok && sym_active(h, mode) && h->mode_bytes_sym[mode] > 0.0) return h->mode_bytes_sym[mode];
     return h->mode_bytes32[mode];
 }
@@ -2235,7 +2235,7 @@ int dd_get_gemv_bytes(const dd_handle* h, int32_t kind, int32_t precision, doubl
     double str = alg;
     if (precision == DD_MIXED && h->prm.sym_fp32 && h->sym_ok && sym_active(h, kind) && h->mode_tile_bytes_sym[kind] > 0.0)
         str = h->mode_tile_bytes_sym[kind];
-    if (precision == DD_FP64 && fx_active(h, kind)) str = h->fx_bytes[kind];
+    if (precision == DD_FP64 && fx_built(h, kind)) str = h->fx_bytes[kind];
     if (algorithmic) *algorithmic = alg;
     if (streamed) *streamed = str;
     return DD_OK;
