@@ -2064,8 +2064,8 @@ int dd_autotune(dd_handle* h, const char* cache_path, double* seconds, void* str
             const int prec = p == 0 ? DD_FP64 : DD_MIXED;
             for (int m = 0; m < GEMV_NMODES && !rc; ++m) {
                 const bool sym_saved = h->prm.sym_fp32 != 0;
-                // FP64 kinds of an FP64 handle in fixed point; the operator calls' ones are applied dense too
-                const bool fixed_only = fx_built(h, m) && h->prm.precision == DD_FP64 && m != GEMV_COUPLED && m != GEMV_SCHUR_G;
+                // FP64 steps run in fixed point where it is built; the operator calls' kinds are applied dense too
+                const bool fixed_only = fx_built(h, m) && m != GEMV_COUPLED && m != GEMV_SCHUR_G;
                 if (p == 1 && h->sym_ok && sym_active(h, m)) {
                     // packed symmetric tiles: time both kernel forms with 1, 2, 4 and 8 CTAs per subdomain and
                     // rings of 2, 3 and 4 tiles
