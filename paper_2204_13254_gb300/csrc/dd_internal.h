@@ -89,7 +89,7 @@ DD_HD inline int sym_tile_floats(int h, int w, bool diag) { return diag ? sym_tr
 DD_HD inline bool sym_masks(int mode, int* rmask, int* cmask) {
     switch (mode) {
         case 0: *rmask = 7; *cmask = 3; return true;   // GEMV_LOCAL:   rows all, cols r
-        case 3: *rmask = 3; *cmask = 6; return true;   // GEMV_RECOVER: rows r, cols Gamma c (ensembles only)
+        case 3: *rmask = 3; *cmask = 6; return true;   // GEMV_RECOVER: rows r, cols Gamma c
         case 5: *rmask = 2; *cmask = 6; return true;   // GEMV_SCHUR_G: rows Gamma, cols Gamma c
         case 6: *rmask = 6; *cmask = 6; return true;   // GEMV_COUPLED: rows Gamma c, cols Gamma c
         default: return false;
@@ -212,12 +212,12 @@ struct PcgScalars {
     int32_t it;       // iterations done
     int32_t done;     // 1 when converged (kernels become no-ops)
     int32_t status;   // DD_OK / DD_ERR_NONFINITE
-    int32_t wait_err; // nonzero once a bounded TMA wait of the packed-tile GEMV gave up
+    int32_t wait_err; // nonzero once a bounded device wait gave up
     double norm_b2;   // mixed mode: ||b||^2 of the step system
     double norm_r2;   // mixed mode: ||r||^2 of the current FP64 residual
     int32_t lam_levels;   // warm_start 2: multiplier history levels available (0, 1, 2)
-    int32_t wait_first;   // > 0: the first mbarrier wait of every packed-GEMV CTA polls an mbarrier
-                          // nothing completes, this many times, and gives up (failure-path test; 0 = off)
+    int32_t wait_first;   // > 0: the first wait of every CTA that waits polls for something that never comes,
+                          // this many times, and gives up (failure-path test; 0 = off)
     int32_t it_total;     // graph mode: CG iterations of the whole step
     int32_t refinements;  // graph mode: solves of the whole step
     int32_t step_status;  // graph mode: DD status of the whole step
@@ -690,8 +690,7 @@ int launch_fx_pack(const dd_handle* h, void* stream);
 int launch_fxgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);
 int launch_symgemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int32_t* skip, void* stream);
 size_t sym_smem_bytes(const dd_handle* h);
-// Packed kinds in use: the recovery reads the packed tiles only for an ensemble (its I x [Gamma|c]
-// rectangle has no symmetric twin, so one problem gains almost nothing; an ensemble shares the reads).
+// Kinds with a packed form: local, recovery, interface rows, coupled.
 bool sym_active(const dd_handle* h, int mode);
 // ozaki.cu
 size_t oz_bytes(int nm, int nmax);

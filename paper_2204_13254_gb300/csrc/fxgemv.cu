@@ -78,6 +78,7 @@ constexpr int kFlush = 8;              // tiles of one tile row between two flus
 constexpr int kBlkInts = 256;          // one 16 x 8 block: 128 hi words, 128 lo words
 constexpr int kStripInts = 4 * kBlkInts;   // ring slot of one warp: 64 rows x 8 columns, 4 KB
 constexpr int kPad = 17;               // column stride of the transposed sums in a slot (16 row lanes, no bank conflicts)
+constexpr int kSms = 152;              // multiprocessors of a GB300 (the ranges are cut before a device is bound)
 constexpr int kFxW = 4;                // words per tile list entry: tile_entry(), first block, block rows | strips << 8, 0
 
 static_assert(kFx96Low == kLow, "the split of the integers");
@@ -489,8 +490,9 @@ bool fx_active(const dd_handle* h, int mode) { return fx_built(h, mode) && h->pa
 //    8 of 448 0.87 / 0.89.
 //  * CTAs per subdomain: every CTA more stages x again, but one CTA per subdomain leaves SMs
 //    with one CTA beside SMs with two where there are fewer subdomains than slots (two per
-//    SM).  So two up to 256 subdomains, and more (a cluster of 8 at most) only until every
-//    SM has a CTA.  Measured, FP64 GMRES step with 1 / 2 / 4 / 8 CTAs per subdomain, in us: 64
+//    SM, 304).  So two up to 256 subdomains, the largest number below that line at which two
+//    were measured to be better (by 2 %; at 343 one is), and more (a cluster of 8 at most)
+//    only until every SM has a CTA.  Measured, FP64 GMRES step with 1 / 2 / 4 / 8 CTAs per subdomain, in us: 64
 //    subdomains of 1,854 unknowns 3,203 / 2,086 / 1,559 / 1,618, 100 of 741 1,323 / 1,047 /
 //    1,108 / 1,405, 128 of 2,196 3,947 / 3,110 / 3,330 / 4,164, 216 of 1,115 2,200 / 1,947 /
 //    2,207 / 3,091, 256 of 1,152 2,241 / 2,198 / 2,602 / 3,576, 343 of 604 1,511 / 1,624.
@@ -542,7 +544,7 @@ void build_fx(dd_handle* h) {
             continue;
         }
         int cl = h->n_sub <= 256 ? 2 : 1;
-        while (cl < kSymCLMax && h->n_sub * cl < 152) cl *= 2;
+        while (cl < kSymCLMax && h->n_sub * cl < kSms) cl *= 2;
         h->fx_cl[m] = cl;
         int32_t longest = 0;
         sym_split(h, m, cl, 1, h->fx_rng[m], &longest);

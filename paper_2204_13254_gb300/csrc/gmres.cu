@@ -546,17 +546,6 @@ __global__ void __launch_bounds__(kT) k_gm_pass(UView U, const double* __restric
     if (s_end && tid < s_k) gs->y[tid] = sy[tid];
 }
 
-// A whole Arnoldi step after the GEMV in one cooperative launch: both Gram-Schmidt passes, the
-// normalisation and the least-squares update, with one grid barrier behind each pass.  A thread
-// keeps its E elements of t in registers throughout and its basis entries in L1 from pass to
-// pass; every CTA adds the block partials itself (fixed order), so no result travels back
-// through a last block; the last CTA, which has elements only where the grid is full, does the
-// Givens rotations while the others normalise.
-// What bounds it: the two barriers with the reductions around them, in DD_FP64 the FP64 pipe
-// (two lanes a clock and SM).  Measured against the three kernels (mean over the columns of a
-// cycle of 20): FP32 136,000 unknowns 25.8 -> 15.9 us, FP64 64 -> 35 us, FP64 40,000 unknowns
-// 35 -> 18 us.  256 threads with twice the elements: 19.0 us FP32, 43 us FP64; 1,024 with half
-// of them: 16.7 us FP32.
 // Sums over the warp of eight values a lane; sum q in the four lanes with lane / 4 == q.
 __device__ __forceinline__ float wsum8(float (&p)[kKB], int lane) {
     static_assert(kKB == 8, "three halving steps");
@@ -592,6 +581,17 @@ __device__ __forceinline__ void rotate_column(double* col, double hsub, int j, d
     g[j] = c * g[j];
 }
 
+// A whole Arnoldi step after the GEMV in one cooperative launch: both Gram-Schmidt passes, the
+// normalisation and the least-squares update, with one grid barrier behind each pass.  A thread
+// keeps its E elements of t in registers throughout and its basis entries in L1 from pass to
+// pass; every CTA adds the block partials itself (fixed order), so no result travels back
+// through a last block; the last CTA, which has elements only where the grid is full, does the
+// Givens rotations while the others normalise.
+// What bounds it: the two barriers with the reductions around them, in DD_FP64 the FP64 pipe
+// (two lanes a clock and SM).  Measured against the three kernels (mean over the columns of a
+// cycle of 20): FP32 136,000 unknowns 25.8 -> 15.9 us, FP64 64 -> 35 us, FP64 40,000 unknowns
+// 35 -> 18 us.  256 threads with twice the elements: 19.0 us FP32, 43 us FP64; 1,024 with half
+// of them: 16.7 us FP32.
 template <int kSt, int E, typename VT>
 __global__ void __launch_bounds__(kSt, 1) k_gm_step(UView U, const double* w, const float* wf, UIn in, VT* V,
                                                     int64_t ldv, double* zu, float* zuf, GmresScalars* gs,

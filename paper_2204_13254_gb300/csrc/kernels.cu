@@ -868,7 +868,7 @@ __global__ void k_solve_end(PcgScalars* sc) {
     sc->refinements += 1;
     if (sc->status != DD_OK) sc->step_status = sc->status;
     else if (!sc->done && sc->step_status == DD_OK) sc->step_status = DD_ERR_NO_CONVERGENCE;
-    if (sc->wait_err) sc->step_status = DD_ERR_TIMEOUT;   // a packed-GEMV wait gave up (sticky until read)
+    if (sc->wait_err) sc->step_status = DD_ERR_TIMEOUT;   // a bounded wait gave up (sticky until read)
 }
 
 // graph mode: after an FP64 residual, run the next refinement pass (cond = 1) while

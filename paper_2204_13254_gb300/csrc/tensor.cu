@@ -464,7 +464,7 @@ int launch_tc_gemv(const dd_handle* h, int mode, XSrc xs, GemvOut go, const int3
         pmax = std::max(pmax, (int)td.P);
         qmax = std::max(qmax, (int)td.Q);
     }
-    const int parts = std::max(1, std::min((304 + ctas - 1) / ctas, pmax));
+    const int parts = std::max(1, std::min((2 * (int)h->n_sm + ctas - 1) / ctas, pmax));
     k_tc_stage<<<dim3((unsigned)ctas, (unsigned)qmax), kTcStageT, 0, (cudaStream_t)stream>>>(
         h->d.tcd[k], h->d.symd, h->n_sub_real, h->members, qmax, xs, h->d.xtc, skip);
     k_tc_gemv<<<dim3((unsigned)ctas, (unsigned)parts), 128, kTcSmem, (cudaStream_t)stream>>>(
