@@ -36,9 +36,9 @@
 // HBM traffic); the wide pivot block and the triangle each halve both against 32-wide
 // blocks over the full square; with a single matrix the pivots one after another.
 // Measured, 40 matrices of up to 2,454 rows with their 1,229-row coarse matrix, per
-// 64-wide block (mean over both): panel 0.06, update with the next pivot 0.28 ms, against
+// 64-wide block (mean over both): panel 0.07, update with the next pivot 0.28 ms, against
 // 0.51 + 0.09 (pivot, panels in FP64), 0.22 (slices) and 0.70 ms per 32-wide block over
-// the full square; the whole factorisation 25 against 170 ms.
+// the full square; the whole factorisation and a step 25.5 against 177 ms.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
