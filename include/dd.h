@@ -576,12 +576,13 @@ int dd_set_sym_config(dd_handle* h, int32_t kind, int32_t cl, int32_t st, int32_
 
 /* Failure-path testing aid for the bounded device waits.  With
  * first_wait_polls > 0, the first wait of every CTA of the packed GEMVs (FP32
- * tiles of DD_MIXED, fixed-point tiles of DD_FP64), of the one-kernel interface
- * solves, of the one-kernel Krylov steps and of the tensor-core elimination is
- * for something that never comes: it polls that many times and gives up, as a
- * wait on a lost copy or on a CTA that never arrives would: the CTA records the
- * failure in the device status word, waits (bounded) for the copies it has in
- * flight and exits.  dd_factor then returns DD_ERR_TIMEOUT, and so does a step
+ * tiles of DD_MIXED, fixed-point tiles of DD_FP64; not the tensor-core form), of
+ * the one-kernel interface solves, of the one-kernel Krylov steps and of the
+ * tensor-core elimination is for something that never comes: it polls that many
+ * times and gives up, as a wait on a lost copy or on a CTA that never arrives
+ * would: the CTA records the failure in the device status word, waits (bounded)
+ * for the copies it has in flight and exits.  dd_factor then returns
+ * DD_ERR_TIMEOUT, and so does a step
  * -- in eager mode at once, in graph mode from the first call that reads stats
  * -- which is not taken: e^n, e^{n-1} and the step counter stay where they were and the next
  * solve starts cold.  0 restores the normal waits (2^20 polls).  Synchronises
