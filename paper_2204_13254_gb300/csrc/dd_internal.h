@@ -257,7 +257,7 @@ struct GmresScalars {
     int32_t nh2;        // terms of the second projection k_gm_normalize applies (0 at a cycle start)
     uint32_t counter[4];
     uint32_t bar;       // arrivals at the grid barriers of the resident solve
-    uint32_t pad;
+    int32_t first_polls;   // PcgScalars::wait_first, beside the words that k_gm_step reads first
     double g[kMaxRestart + 1];
     double cs[kMaxRestart], sn[kMaxRestart];
     double y[kMaxRestart];

@@ -250,6 +250,7 @@ __global__ void k_gm_init(GmresScalars* gs, const PcgScalars* sc, double tol, do
     gs->m = m;
     gs->cycles = 0;
     gs->bar = 0u;
+    gs->first_polls = sc->wait_first;
     gs->counter[1] = gs->counter[2] = 0u;
     if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 1u);
 }
@@ -610,10 +611,10 @@ __global__ void __launch_bounds__(kSt, 1) k_gm_step(UView U, const double* w, co
     const int64_t nu = U.n1 + U.n2 + U.nc;
     const int j = gs->j, nv = j + 1, nb = (int)gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_failed = gs->first_polls;
     const bool ctl = (int)blockIdx.x == nb - 1;
     const int64_t ib = (int64_t)blockIdx.x * (kSt * E), i0 = ib + tid;
     const bool work = ib < nu;
-    if (tid == 0) s_failed = sc->wait_first;
     uint32_t* const bar_a = &gs->counter[1];
     uint32_t* const bar_b = &gs->counter[2];
     if (ctl) {

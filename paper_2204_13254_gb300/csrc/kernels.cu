@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_pcg_step(int64_t n_lambda, cons
     const int nb = (int)gridDim.x, tid = threadIdx.x;
     const int64_t m0 = blockIdx.x * (int64_t)kThreads + tid, stride = (int64_t)nb * kThreads;
     const double beta = sc->beta, rz = sc->rz;
-    if (tid == 0) s_failed = sc->wait_first;
+    const int first_polls = tid == 0 ? sc->wait_first : 0;
     double pn[E], qq[E], rr[E], lm[E], di[E];
     double v[1] = {0.0};
 #pragma unroll
@@ -794,7 +794,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_pcg_step(int64_t n_lambda, cons
         v[0] += pn[e] * qq[e];
     }
     block_sum<1>(v);
-    if (tid == 0) partials[blockIdx.x] = v[0];
+    if (tid == 0) {
+        partials[blockIdx.x] = v[0];
+        s_failed = first_polls;
+    }
     if (!grid_meet(&sc->counter[1], &sc->wait_err, &s_failed)) {   // the solve is void: leave the loop
         if (tid == 0) {
             sc->done = 1;
